@@ -97,10 +97,7 @@ int wd_context_create(const int dims[4], void* stream, wd_ctx** out) {
     return fail(WD_ERR_ARG, "the lattice must have fewer than 2^31 sites");
   wd_ctx* c = new (std::nothrow) wd_ctx();
   if (!c) return fail(WD_ERR_ARG, "out of host memory");
-  for (int m = 0; m < 4; ++m) c->g.L[m] = dims[m];
-  c->g.Lh = dims[0] / 2;
-  c->g.V = (long)dims[0] * dims[1] * dims[2] * dims[3];
-  c->g.Vh = c->g.V / 2;
+  c->g.set(dims);
   c->stream = (cudaStream_t)stream;
   cudaGetDevice(&c->device);
   const long Vh = c->g.Vh;

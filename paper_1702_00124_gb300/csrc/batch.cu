@@ -145,10 +145,7 @@ __device__ __forceinline__ void bhop_dir(const Geom& g, int par, long cb, const 
 #pragma unroll
   for (int fb = 0; fb < 2; ++fb) {
     const bool fwd = fb == 0;
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    if (fwd) n[MU] = (n[MU] + 1 == g.L[MU]) ? 0 : n[MU] + 1;
-    else n[MU] = (n[MU] == 0) ? g.L[MU] - 1 : n[MU] - 1;
-    const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+    const long nb = fwd ? g.template nbr<2 * MU>((unsigned)cb, c) : g.template nbr<2 * MU + 1>((unsigned)cb, c);
     cpx<float> U[9];
     if (fwd) gauge.load(MU, par, cb, U);
     else gauge.load(MU, 1 - par, nb, U);
@@ -165,7 +162,8 @@ __device__ __forceinline__ void bhop_dir(const Geom& g, int par, long cb, const 
       }
       if (fwd) {
         su3_mul(U, h, u);
-        spin_accum<MU, SF>(acc[k], u);
+        if constexpr (MU == 0) spin_accum<MU, SF, true>(acc[k], u);   // the first direction writes acc
+        else spin_accum<MU, SF>(acc[k], u);
       } else {
         su3_dag_mul(U, h, u);
         spin_accum<MU, -SF>(acc[k], u);
@@ -198,10 +196,6 @@ __device__ __forceinline__ void bhop_body(const BArgs& a, int vb, int fin, int f
     int c[4];
     L->g.coords(cb, a.out_par, c);
     cpx<float> acc[RPT][12];
-#pragma unroll
-    for (int k = 0; k < RPT; ++k)
-#pragma unroll
-      for (int j = 0; j < 12; ++j) acc[k][j] = mk<float>(0, 0);
     const float4* in = L->f[fin];
     if constexpr (R12) {
       GF32R12 G{L->g12, L->g.Vh};
@@ -269,8 +263,6 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, HOP_MINB) k_bhop_st(BArgs a, i
     Staged<HOP_NST, DAG, HA> S{ha, it.cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
     L->g.coords(it.cb, a.out_par, S.c);
     cpx<float> acc[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) acc[j] = mk<float>(0, 0);
     S.run(acc);
     if constexpr (XPAY) {
       cpx<float> yv[12];

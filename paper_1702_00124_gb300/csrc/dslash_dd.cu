@@ -141,9 +141,7 @@ __device__ __forceinline__ void hop_dir_lz(const HopArgs<SpDD, SpDD, SpDD, GDD>&
   constexpr int SB = -SF;
   const Geom& g = a.g;
   {
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    n[MU] = (n[MU] + 1 == g.L[MU]) ? 0 : n[MU] + 1;
-    const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+    const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
     cpx<dd> s[12], h[6];
     a.in.loadT(nb, s);
     spin_project<MU, SF>(s, h);
@@ -154,9 +152,7 @@ __device__ __forceinline__ void hop_dir_lz(const HopArgs<SpDD, SpDD, SpDD, GDD>&
     mul_accum_lz<MU, SF, false>(a.gauge, a.out_par, cb, h, acc);
   }
   {
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    n[MU] = (n[MU] == 0) ? g.L[MU] - 1 : n[MU] - 1;
-    const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+    const long nb = g.template nbr<2 * MU + 1>((unsigned)cb, c);
     cpx<dd> s[12], h[6];
     a.in.loadT(nb, s);
     spin_project<MU, SB>(s, h);

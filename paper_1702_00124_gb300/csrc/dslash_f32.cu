@@ -48,8 +48,6 @@ __global__ void __launch_bounds__(128) k_hop_poly(HopArgs<SpF32, SpF32, SpF32, G
   int c[4];
   a.g.coords(cb_, 0, c);
   cpx<float> acc[12];
-#pragma unroll
-  for (int j = 0; j < 12; ++j) acc[j] = mk<float>(0, 0);
   hop_dir<0, true>(a.g, 0, cb_, c, a.in, a.gauge, acc);
   hop_dir<1, true>(a.g, 0, cb_, c, a.in, a.gauge, acc);
   hop_dir<2, true>(a.g, 0, cb_, c, a.in, a.gauge, acc);
@@ -79,8 +77,6 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, HOP_MINB) k_hop_poly_st(HopArg
                                                                   (int)blockDim.x};
   a.g.coords(cb_, 0, S.c);
   cpx<float> acc[12];
-#pragma unroll
-  for (int j = 0; j < 12; ++j) acc[j] = mk<float>(0, 0);
   S.run(acc);
   cpx<float> yv[12], q[12];
   a.y.loadT(cb_, yv);

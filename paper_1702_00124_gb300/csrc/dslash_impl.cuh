@@ -28,17 +28,25 @@ __device__ __forceinline__ void spin_project(const cpx<T> (&s)[12], cpx<T> (&h)[
   }
 }
 
-template <int MU, int SG, class T>
+// acc += (1 + SG g_mu) (x) u; FIRST: acc is written, not added to
+template <int MU, int SG, bool FIRST = false, class T>
 __device__ __forceinline__ void spin_accum(cpx<T> (&acc)[12], const cpx<T> (&u)[6]) {
   using Gm = Gam<MU>;
   constexpr int q0 = (SG > 0 ? 0 : 2) - Gm::k0;
   constexpr int q1 = (SG > 0 ? 0 : 2) - Gm::k1;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    acc[c] = acc[c] + u[c];
-    acc[3 + c] = acc[3 + c] + u[3 + c];
-    acc[3 * Gm::p0 + c] = acc[3 * Gm::p0 + c] + ipow<q0>(u[c]);
-    acc[3 * Gm::p1 + c] = acc[3 * Gm::p1 + c] + ipow<q1>(u[3 + c]);
+    if constexpr (FIRST) {
+      acc[c] = u[c];
+      acc[3 + c] = u[3 + c];
+      acc[3 * Gm::p0 + c] = ipow<q0>(u[c]);
+      acc[3 * Gm::p1 + c] = ipow<q1>(u[3 + c]);
+    } else {
+      acc[c] = acc[c] + u[c];
+      acc[3 + c] = acc[3 + c] + u[3 + c];
+      acc[3 * Gm::p0 + c] = acc[3 * Gm::p0 + c] + ipow<q0>(u[c]);
+      acc[3 * Gm::p1 + c] = acc[3 * Gm::p1 + c] + ipow<q1>(u[3 + c]);
+    }
   }
 }
 
@@ -48,7 +56,7 @@ __device__ __forceinline__ void su3_mul(const cpx<T> (&U)[9], const cpx<T> (&h)[
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      o[3 * a + c] = U[3 * c] * h[3 * a] + U[3 * c + 1] * h[3 * a + 1] + U[3 * c + 2] * h[3 * a + 2];
+      o[3 * a + c] = cfma(U[3 * c + 2], h[3 * a + 2], cfma(U[3 * c + 1], h[3 * a + 1], cmul(U[3 * c], h[3 * a])));
 }
 
 template <class T>
@@ -57,7 +65,38 @@ __device__ __forceinline__ void su3_dag_mul(const cpx<T> (&U)[9], const cpx<T> (
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      o[3 * a + c] = cmulc(U[c], h[3 * a]) + cmulc(U[3 + c], h[3 * a + 1]) + cmulc(U[6 + c], h[3 * a + 2]);
+      o[3 * a + c] = cfma_c(U[6 + c], h[3 * a + 2], cfma_c(U[3 + c], h[3 * a + 1], cmul_c(U[c], h[3 * a])));
+}
+
+// The same from rows 0 and 1 of U alone (12-real links): an entry of row 2 is
+// formed where it is used, which keeps two registers live instead of six.
+template <class T>
+__device__ __forceinline__ cpx<T> row2_of(const cpx<T> (&U)[6], int k) {
+  return k == 0 ? cross_c(U[1], U[5], U[2], U[4]) : k == 1 ? cross_c(U[2], U[3], U[0], U[5]) : cross_c(U[0], U[4], U[1], U[3]);
+}
+template <class T>
+__device__ __forceinline__ void su3_mul_r12(const cpx<T> (&U)[6], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+      o[3 * a + c] = cfma(U[3 * c + 2], h[3 * a + 2], cfma(U[3 * c + 1], h[3 * a + 1], cmul(U[3 * c], h[3 * a])));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const cpx<T> r = row2_of(U, k);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) o[3 * a + 2] = k == 0 ? cmul(r, h[3 * a]) : cfma(r, h[3 * a + k], o[3 * a + 2]);
+  }
+}
+template <class T>
+__device__ __forceinline__ void su3_dag_mul_r12(const cpx<T> (&U)[6], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cpx<T> r = row2_of(U, c);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+      o[3 * a + c] = cfma_c(r, h[3 * a + 2], cfma_c(U[3 + c], h[3 * a + 1], cmul_c(U[c], h[3 * a])));
+  }
 }
 
 // |s|^2 of one site for a grid sum, returned in FP64.  FP32 sites are summed
@@ -93,6 +132,7 @@ struct HopArgs {
   CGState* st;
 };
 
+// both hops of direction MU; MU = 0 comes first and starts the accumulator
 template <int MU, bool DAG, class T, class In, class G>
 __device__ __forceinline__ void hop_dir(const Geom& g, int par, long cb, const int (&c)[4], const In& in,
                                         const G& gauge, cpx<T> (&acc)[12]) {
@@ -100,9 +140,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, int par, long cb, const i
   constexpr int SB = -SF;             // backward projector
   // forward neighbour x + mu
   {
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    n[MU] = (n[MU] + 1 == g.L[MU]) ? 0 : n[MU] + 1;
-    const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+    const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
     cpx<T> s[12], h[6], u[6], U[9];
     in.loadT(nb, s);
     gauge.load(MU, par, cb, U);
@@ -112,13 +150,11 @@ __device__ __forceinline__ void hop_dir(const Geom& g, int par, long cb, const i
       for (int j = 0; j < 6; ++j) h[j] = mk<T>(-h[j].r, -h[j].i);
     }
     su3_mul(U, h, u);
-    spin_accum<MU, SF>(acc, u);
+    spin_accum<MU, SF, MU == 0>(acc, u);   // direction 0 forward writes acc
   }
   // backward neighbour x - mu, link U_mu(x - mu)^dag
   {
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    n[MU] = (n[MU] == 0) ? g.L[MU] - 1 : n[MU] - 1;
-    const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+    const long nb = g.template nbr<2 * MU + 1>((unsigned)cb, c);
     cpx<T> s[12], h[6], u[6], U[9];
     in.loadT(nb, s);
     gauge.load(MU, 1 - par, nb, U);
@@ -142,8 +178,6 @@ __global__ void __launch_bounds__(MAXT) k_hop(HopArgs<In, Out, Y, G> a) {
     int c[4];
     a.g.coords(cb, a.out_par, c);
     cpx<T> acc[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) acc[j] = mk<T>(0, 0);
     hop_dir<0, DAG>(a.g, a.out_par, cb, c, a.in, a.gauge, acc);
     hop_dir<1, DAG>(a.g, a.out_par, cb, c, a.in, a.gauge, acc);
     hop_dir<2, DAG>(a.g, a.out_par, cb, c, a.in, a.gauge, acc);

@@ -105,13 +105,7 @@ struct Staged {
 
   __device__ __forceinline__ float4* slot(int b, int k) const { return buf + (b * 3 + k) * nt + tid; }
 
-  template <int D> __device__ __forceinline__ long nbr() const {
-    constexpr int MU = D >> 1;
-    int n[4] = {c[0], c[1], c[2], c[3]};
-    if constexpr ((D & 1) == 0) n[MU] = (n[MU] + 1 == a.g.L[MU]) ? 0 : n[MU] + 1;
-    else n[MU] = (n[MU] == 0) ? a.g.L[MU] - 1 : n[MU] - 1;
-    return a.g.cb_of(n[0], n[1], n[2], n[3]);
-  }
+  template <int D> __device__ __forceinline__ long nbr() const { return a.g.template nbr<D>((unsigned)cb, c); }
 
   template <int D> __device__ __forceinline__ void issue() const {
     if constexpr (D < 8) {
@@ -145,7 +139,7 @@ struct Staged {
     constexpr int MU = D >> 1;
     constexpr bool FWD = (D & 1) == 0;
     cpa_wait<NST - 1>();                       // direction D has landed
-    cpx<float> U[9], h[6], u[6];
+    cpx<float> U[6], h[6], u[6];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const float4 v = *slot(D % NB, j);
@@ -153,9 +147,6 @@ struct Staged {
       U[2 * j + 1] = {v.z, v.w};
     }
     issue<D + NST>();                          // refills the buffer of direction D - 1
-    U[6] = conj(U[1] * U[5] - U[2] * U[4]);
-    U[7] = conj(U[2] * U[3] - U[0] * U[5]);
-    U[8] = conj(U[0] * U[4] - U[1] * U[3]);
     constexpr int SF = DAG ? +1 : -1;
     constexpr int SG = FWD ? SF : -SF;
     spin_project<MU, SG>(s, h);
@@ -163,9 +154,9 @@ struct Staged {
 #pragma unroll
       for (int j = 0; j < 6; ++j) h[j] = mk<float>(-h[j].r, -h[j].i);
     }
-    if constexpr (FWD) su3_mul(U, h, u);
-    else su3_dag_mul(U, h, u);
-    spin_accum<MU, SG>(acc, u);
+    if constexpr (FWD) su3_mul_r12(U, h, u);
+    else su3_dag_mul_r12(U, h, u);
+    spin_accum<MU, SG, D == 0>(acc, u);        // direction 0 writes acc
   }
 
   // directions 0 .. NST - 1 go out before the first step
@@ -178,6 +169,9 @@ struct Staged {
 
   __device__ __forceinline__ void run(cpx<float> (&acc)[12]) const {
     prologue<0>();
+    run_after_prologue(acc);
+  }
+  __device__ __forceinline__ void run_after_prologue(cpx<float> (&acc)[12]) const {
     using In = typename std::remove_cv<decltype(a.in)>::type;
     if constexpr (spin_ahead<In>()) {
       typename In::Raw r0, r1;
@@ -214,8 +208,6 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, hop_minb<In>()) k_hop_st(HopAr
                                                          (int)blockDim.x};
     a.g.coords(cb, a.out_par, S.c);
     cpx<float> acc[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) acc[j] = mk<float>(0, 0);
     S.run(acc);
     if constexpr (XPAY) {
       cpx<float> yv[12];

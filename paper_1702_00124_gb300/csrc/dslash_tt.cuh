@@ -325,9 +325,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
           U[2 * j + 1] = {v.z, v.w};
         }
         TTFmt<In>::read(sb + TT_LINK_BYTES, is, s);
-        U[6] = conj(U[1] * U[5] - U[2] * U[4]);
-        U[7] = conj(U[2] * U[3] - U[0] * U[5]);
-        U[8] = conj(U[0] * U[4] - U[1] * U[3]);
+        third_row(U);
         constexpr int SF = DAG ? +1 : -1;
         const bool flip = (mu == 3) && (fwd ? t == a.g.L[3] - 1 : t == 0);
         // the projector and its reconstruction are compile-time per direction

@@ -88,9 +88,7 @@ template <int MU, class T, class S, class G>
 __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4],
                                           const cpx<T> (&Xs)[12], const cpx<T> (&Ys)[12]) {
   const Geom& g = a.g;
-  int n[4] = {c[0], c[1], c[2], c[3]};
-  n[MU] = (n[MU] + 1 == g.L[MU]) ? 0 : n[MU] + 1;
-  const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+  const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
   cpx<T> Xn[12], Yn[12];
   (par ? a.Xe : a.Xo).loadT(nb, Xn);
   (par ? a.Ye : a.Yo).loadT(nb, Yn);
@@ -166,9 +164,7 @@ struct ForceArgs2 {
 template <int MU, class T, class S, class G>
 __device__ __forceinline__ void force_dir2(const ForceArgs2<S, G>& a, int par, long cb, const int (&c)[4]) {
   const Geom& g = a.g;
-  int n[4] = {c[0], c[1], c[2], c[3]};
-  n[MU] = (n[MU] + 1 == g.L[MU]) ? 0 : n[MU] + 1;
-  const long nb = g.cb_of(n[0], n[1], n[2], n[3]);
+  const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
   cpx<T> U[9];
   a.gauge.load(MU, par, cb, U);
   const T bc = (MU == 3 && c[3] == g.L[3] - 1) ? (T)-1 : (T)1;

