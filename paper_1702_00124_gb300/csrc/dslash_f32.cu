@@ -11,9 +11,9 @@ int hop_f32(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out,
   SpF32 I = sp32(in), O = sp32(out), Y = y ? sp32(*y) : O;
   if (c->recon == WD_RECON_12) {
     if (tt_eligible(c)) return hop_tt(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
-    return hop_staged(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
+    return hop_r12(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
   }
-  return hop_with_gauge<float>(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg, false);
+  return hop_r18(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
 }
 
 // Self-test of the bounded barrier wait: thread 0 waits on a freshly
@@ -112,6 +112,19 @@ int khat_poly_step_f32(wd_ctx* c, double kappa, const Field& s, Field& t1, Field
     for (const Field* f : chk)
       if (((uintptr_t)f->data & 15) != 0) return fail(WD_ERR_ARG, "khat_poly_step_f32: fields must be 16-byte aligned");
     WD_TRY((tt_launch<true, 2, false>(c, a, pe)));
+  } else if (split_eligible(c, false)) {
+    const SplitPoly pe{sp32(v), sp32(s), sp32(sprev), (float)ca, (float)cmu, (float)cb};
+    const int nbs = nblocks(c->g.Vh, SPL_SITES);
+    if (c->recon == WD_RECON_12) {
+      HopArgs<SpF32, SpF32, SpF32, GF32R12> a{c->g, 0, sp32(t1), sp32(out), sp32(t2),
+                                              GF32R12{c->gauge32r12, c->g.Vh}, a2, reducer(c), nullptr};
+      k_hop_split<float, true, 2, false><<<nbs, SPL_THREADS, 0, c->stream>>>(a, pe);
+    } else {
+      HopArgs<SpF32, SpF32, SpF32, GF32> a{c->g, 0, sp32(t1), sp32(out), sp32(t2), GF32{c->gauge32, c->g.Vh}, a2,
+                                           reducer(c), nullptr};
+      k_hop_split<float, true, 2, false><<<nbs, SPL_THREADS, 0, c->stream>>>(a, pe);
+    }
+    WD_CHECK_LAUNCH();
   } else if (c->recon == WD_RECON_12) {
     HopArgs<SpF32, SpF32, SpF32, GF32R12> a{c->g, 0, sp32(t1), sp32(out), sp32(t2), GF32R12{c->gauge32r12, c->g.Vh},
                                             a2, reducer(c), nullptr};

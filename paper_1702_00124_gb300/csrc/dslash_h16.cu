@@ -18,14 +18,14 @@ static int hop_h(wd_ctx* c, int out_par, bool dag, const Field& in, const Field&
     return fail(WD_ERR_ARG, "hop_h16: output must be 16-bit of the same kind or FP32");
   }
   if (c->recon == WD_RECON_12) {
-    if (out.fmt == in.fmt) return hop_staged(c, out_par, dag, I, sp16<H>(out), Y, y != nullptr, alpha, norm_cg, in_cg);
-    if (out.fmt == WD_F32) return hop_staged(c, out_par, dag, I, sp32(out), Y, y != nullptr, alpha, norm_cg, in_cg);
+    if (out.fmt == in.fmt) return hop_r12(c, out_par, dag, I, sp16<H>(out), Y, y != nullptr, alpha, norm_cg, in_cg);
+    if (out.fmt == WD_F32) return hop_r12(c, out_par, dag, I, sp32(out), Y, y != nullptr, alpha, norm_cg, in_cg);
     return fail(WD_ERR_ARG, "hop_h16: output must be 16-bit of the same kind or FP32");
   }
   if (out.fmt == in.fmt)
-    return hop_with_gauge<float>(c, out_par, dag, I, sp16<H>(out), Y, y != nullptr, alpha, norm_cg, in_cg, false);
+    return hop_r18(c, out_par, dag, I, sp16<H>(out), Y, y != nullptr, alpha, norm_cg, in_cg);
   if (out.fmt == WD_F32)
-    return hop_with_gauge<float>(c, out_par, dag, I, sp32(out), Y, y != nullptr, alpha, norm_cg, in_cg, false);
+    return hop_r18(c, out_par, dag, I, sp32(out), Y, y != nullptr, alpha, norm_cg, in_cg);
   return fail(WD_ERR_ARG, "hop_h16: output must be 16-bit of the same kind or FP32");
 }
 

@@ -38,7 +38,7 @@
 // solver state when there is one), stops its work, and the producer waits
 // (again bounded) for the copies it has issued before the block ends.
 #pragma once
-#include "dslash_staged.cuh"
+#include "dslash_split.cuh"
 
 namespace wd {
 

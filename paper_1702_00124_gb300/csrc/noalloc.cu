@@ -27,7 +27,7 @@
 //     point must not be used.
 #include <mutex>
 
-#include "dslash_impl.cuh"
+#include "dslash_split.cuh"
 
 namespace wd {
 namespace {
@@ -62,7 +62,7 @@ int launch(cudaStream_t s, const Geom& g, int out_par, const double2* gauge, con
   using A = HopArgs<SpF64, SpF64, SpF64, GF64>;
   SpF64 I{const_cast<double2*>(in), g.Vh}, O{out, g.Vh}, Y{const_cast<double2*>(y ? y : in), g.Vh};
   A a{g, out_par, I, O, Y, GF64{gauge, g.Vh}, alpha, Reduce{nullptr, nullptr, nullptr}, nullptr};
-  k_hop<double, DAG, XPAY, false, 128, SpF64, SpF64, SpF64, GF64><<<nblocks(g.Vh, HOP_THREADS), HOP_THREADS, 0, s>>>(a);
+  k_hop_split<double, DAG, XPAY ? 1 : 0, false><<<nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s>>>(a, SplitPoly{});
   WD_CUDA(cudaGetLastError());
   return WD_OK;
 }
