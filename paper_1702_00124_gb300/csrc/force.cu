@@ -351,12 +351,9 @@ __global__ void __launch_bounds__(F_THREADS) k_gauge_action(Geom g, G gauge, Red
 int gauge_action_k(wd_ctx* c, double* S) {
   const int nb = nblocks(2 * c->g.Vh, F_THREADS);
   if (nb > RED_MAX_BLOCKS) return fail(WD_ERR_ARG, "gauge action: lattice too large");
-  k_gauge_action<<<nb, F_THREADS, 0, c->stream>>>(c->g, GF64{c->gauge64, c->g.Vh}, reducer(c));
+  k_gauge_action<<<nb, F_THREADS, 0, c->stream>>>(c->g, GF64{c->gauge64, c->g.Vh}, reducer_host(c));
   WD_CHECK_LAUNCH();
-  WD_CUDA(cudaMemcpyAsync(c->host_scalar, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  WD_CUDA(cudaStreamSynchronize(c->stream));
-  *S = c->host_scalar[0];
-  return WD_OK;
+  return fetch_host(c, 1, S);
 }
 
 }  // namespace wd

@@ -239,11 +239,11 @@ int kinetic_k(wd_ctx* c, const double* P, double* out) {
   const long n = 64 * c->g.Vh;
   const int nb = nblocks((n + 7) / 8, 256);
   if (nb > RED_MAX_BLOCKS) return fail(WD_ERR_ARG, "kinetic: lattice too large");
-  k_sumsq<<<nb, 256, 0, c->stream>>>(n, P, reducer(c));
+  k_sumsq<<<nb, 256, 0, c->stream>>>(n, P, reducer_host(c));
   WD_CHECK_LAUNCH();
-  WD_CUDA(cudaMemcpyAsync(c->host_scalar, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  WD_CUDA(cudaStreamSynchronize(c->stream));
-  *out = 0.5 * c->host_scalar[0];
+  double s;
+  WD_TRY(fetch_host(c, 1, &s));
+  *out = 0.5 * s;
   return WD_OK;
 }
 

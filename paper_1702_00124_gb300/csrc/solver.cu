@@ -210,20 +210,20 @@ static int download_state(wd_ctx* c) {
 // two FP32 words, the operator applied with error-free FP32 arithmetic, the
 // result rejoined in FP64): about 48 significant bits on the FP32 pipes.
 static int true_residual(wd_ctx* c, const Op& op, const Field& b, const Field& x, const Field& r,
-                         const Field& t, double* rr) {
+                         double* rr) {
+  WsGuard w(c);
   if (c->resid_dd && c->gauge_dd) {
-    WsGuard w(c);
     Field xd, td;
     WD_TRY(w.get(WD_DD, &xd));
     WD_TRY(w.get(WD_DD, &td));
     WD_TRY(convert(c, x, xd));
     WD_TRY(op_apply(c, op, xd, td, false));
-    WD_TRY(convert(c, td, t));
-  } else {
-    WD_TRY(op_apply(c, op, x, t, false));
+    return residual(c, b, td, r, rr);
   }
-  WD_TRY(axpby(c, 1.0, b, -1.0, t, r));
-  return norm2(c, r, rr);
+  Field t;
+  WD_TRY(w.get(WD_F64, &t));
+  WD_TRY(op_apply(c, op, x, t, false));
+  return residual(c, b, t, r, rr);
 }
 
 // Default reliable-update factor per sloppy precision: the iterated residual
@@ -277,16 +277,15 @@ static int cg_core(wd_ctx* c, const Op& op, const Field& b, const Field& x, cons
     return t < 100.0 * stop_rr ? final_rr : t;
   };
   WsGuard w(c);
-  Field r, t, xs, rs, ps, aps;
+  Field r, xs, rs, ps, aps;
   WD_TRY(w.get(WD_F64, &r));
-  WD_TRY(w.get(WD_F64, &t));
   double rr;
   if (x_zero) {   // r = b without applying A
     WD_TRY(zero(c, x));
     WD_TRY(convert(c, b, r));
     rr = bb;
   } else {
-    WD_TRY(true_residual(c, op, b, x, r, t, &rr));
+    WD_TRY(true_residual(c, op, b, x, r, &rr));
   }
   if (!std::isfinite(rr)) return fail(WD_ERR_NAN, "cg: non-finite initial residual");
   int status = WD_OK;
@@ -319,14 +318,12 @@ static int cg_core(wd_ctx* c, const Op& op, const Field& b, const Field& x, cons
       if (st.flag & FLAG_NAN) { status = fail(WD_ERR_NAN, "cg: non-finite value in the iteration"); break; }
       if (st.flag == 0) continue;
       // fold the sloppy increment into x and recompute the FP64 residual
-      WD_TRY(convert(c, xs, t));
-      WD_TRY(axpby(c, 1.0, x, 1.0, t, x));
-      WD_TRY(true_residual(c, op, b, x, r, t, &rr));
+      WD_TRY(fold(c, xs, x));
+      WD_TRY(true_residual(c, op, b, x, r, &rr));
       inf.reliable_updates += 1;
       if (!std::isfinite(rr)) { status = fail(WD_ERR_NAN, "cg: non-finite true residual"); break; }
       if (rr <= stop_rr) break;
       if (st.flag & FLAG_MAXITER) { status = fail(WD_ERR_NOCONV, "cg: maxiter reached"); break; }
-      WD_TRY(zero(c, xs));
       WD_TRY(convert(c, r, rs));
       st.beta = rr / st.rr_old;
       st.rr = rr;

@@ -218,7 +218,7 @@ int term_action(wd_ctx* c, const wd_term& t, const Field& phi, const wd_cg_param
   WD_TRY(w.get(WD_F64, &b));
   WD_TRY(w.get(WD_F64, &X));
   WD_TRY(w.get(WD_F64, &AX));
-  double re, xax;
+  double re[2], xax[2];   // hi + lo
   switch (t.kind) {
     case WD_TERM_PLAIN:
     case WD_TERM_HASENBUSCH: {
@@ -226,25 +226,23 @@ int term_action(wd_ctx* c, const wd_term& t, const Field& phi, const wd_cg_param
       else WD_TRY(mhat(c, t.kappa_h, true, phi, b));
       WD_TRY(solve(c, t.kappa, nullptr, b, X, p));
       WD_TRY(mhat(c, t.kappa, false, X, AX));       // |M X|^2 = X^dag K X
-      WD_TRY(dot(c, b, X, &re, nullptr));
-      WD_TRY(norm2(c, AX, &xax));
-      *S = 2.0 * re - xax;
+      WD_TRY(dot_hl(c, b, X, re));
+      WD_TRY(dot_hl(c, AX, AX, xax));
+      *S = (2.0 * re[0] - xax[0]) + (2.0 * re[1] - xax[1]);
       if (Xo) WD_TRY(convert(c, X, *Xo));
       if (Yo) WD_TRY(convert(c, AX, *Yo));
       return WD_OK;
     }
     case WD_TERM_POLY: {
       WD_TRY(poly_apply_hp(c, t.kappa, t.poly, phi, AX));
-      WD_TRY(dot(c, phi, AX, &re, nullptr));
-      *S = re;
+      WD_TRY(dot(c, phi, AX, S, nullptr));
       return WD_OK;
     }
     case WD_TERM_RATIO: {
       PolyCoef q;
       WD_TRY(ratio_coef(t.poly, t.poly_lo, &q));
       WD_TRY(roots_apply_hp(c, t.kappa, q, phi, AX));
-      WD_TRY(dot(c, phi, AX, &re, nullptr));
-      *S = re;
+      WD_TRY(dot(c, phi, AX, S, nullptr));
       return WD_OK;
     }
     case WD_TERM_FILTERED: {
@@ -252,9 +250,9 @@ int term_action(wd_ctx* c, const wd_term& t, const Field& phi, const wd_cg_param
       WD_TRY(solve(c, t.kappa, &t.poly, phi, X, p));
       WD_TRY(poly_apply_hp(c, t.kappa, t.poly, X, tmp));
       WD_TRY(khat_hp(c, t.kappa, tmp, AX));
-      WD_TRY(dot(c, phi, X, &re, nullptr));
-      WD_TRY(dot(c, X, AX, &xax, nullptr));
-      *S = 2.0 * re - xax;
+      WD_TRY(dot_hl(c, phi, X, re));
+      WD_TRY(dot_hl(c, X, AX, xax));
+      *S = (2.0 * re[0] - xax[0]) + (2.0 * re[1] - xax[1]);
       if (Xo) WD_TRY(convert(c, X, *Xo));
       return WD_OK;
     }

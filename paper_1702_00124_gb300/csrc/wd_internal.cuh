@@ -316,6 +316,15 @@ template <class H> struct Sp16 {
       p[j * stride + i] = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
+  // components 4 j .. 4 j + 3 of site i (one stored word)
+  __device__ __forceinline__ void word(long i, int j, cpx<float> (&s)[4]) const {
+    const float n = __ldg(nrm + i);
+    const uint4 v = __ldg(p + j * stride + i);
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      s[q] = {n * H16Traits<H>::to_f((unsigned short)(w[q] & 0xffffu)), n * H16Traits<H>::to_f((unsigned short)(w[q] >> 16))};
+  }
   // the stored words of one site (16-bit values and the norm), loaded ahead of their use
   struct Raw { uint4 v[3]; float n; };
   __device__ __forceinline__ void loadRaw(long i, Raw& r) const {
@@ -487,6 +496,64 @@ __device__ __forceinline__ bool grid_sum(const Reduce& r, double (&v)[NV], doubl
   return true;
 }
 
+// The same for results the host reads, which are written as hi + lo pairs
+// (out[k], out[NV + k]): the last block adds the partial sums with two-sums
+// (Knuth), so the result carries the blocks' own rounding only.  An action is a
+// difference of two such sums whose derivative is compared with forces.
+struct Sum2 {
+  double s, c;
+};
+__device__ __forceinline__ Sum2 sum2_add(Sum2 a, double s, double c) {
+  const double t = a.s + s, z = t - a.s;
+  return {t, a.c + (((a.s - (t - z)) + (s - z)) + c)};
+}
+template <int NV> __device__ __forceinline__ void grid_sum_hl(const Reduce& r, double (&v)[NV]) {
+  __shared__ double sh[NV * 32];
+  __shared__ Sum2 sh2[NV * 32];
+  __shared__ bool last;
+  block_sum<NV>(v, sh);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) r.partial[blockIdx.x * NV + k] = v[k];
+    __threadfence();
+    last = atomicAdd(r.counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  Sum2 a[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) a[k] = {0.0, 0.0};
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) a[k] = sum2_add(a[k], __ldcg(r.partial + b * NV + k), 0.0);
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int lv = 0; lv < 2; ++lv) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      if (lv == 1) a[k] = lane < nw ? sh2[k * 32 + lane] : Sum2{0.0, 0.0};
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        a[k] = sum2_add(a[k], __shfl_down_sync(0xffffffffu, a[k].s, o), __shfl_down_sync(0xffffffffu, a[k].c, o));
+      if (lv == 0 && lane == 0) sh2[k * 32 + wid] = a[k];
+    }
+    if (lv == 0) {
+      __syncthreads();
+      if (wid != 0) return;
+    }
+  }
+  if (lane != 0) return;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const double h = a[k].s + a[k].c;
+    r.out[k] = h;
+    r.out[NV + k] = (a[k].s - h) + a[k].c;
+  }
+  *r.counter = 0u;
+}
+
 // ----------------------------------------------------------------------------
 // Solver state kept on the device so that iterations can be queued without
 // host round trips.  Kernels return at once when flag != 0.
@@ -613,6 +680,10 @@ struct WsGuard {
 Field wrap_f64(wd_ctx* c, const double* p);
 
 inline Reduce reducer(wd_ctx* c) { return Reduce{c->red_partial, c->red_counter, c->red_out}; }
+// sums the host reads: written straight to the context's pinned scratch, read by
+// fetch_host after the stream's synchronisation (no copy in between)
+inline Reduce reducer_host(wd_ctx* c) { return Reduce{c->red_partial, c->red_counter, c->host_scalar}; }
+int fetch_host(wd_ctx* c, int nv, double* out);
 constexpr int RED_MAX_BLOCKS = 1 << 16;
 
 // bounded-wait self-test (dslash_f32.cu)
@@ -639,12 +710,14 @@ int caxpby(wd_ctx* c, double ar, double ai, const Field& x, double br, double bi
 int zero(wd_ctx* c, const Field& f);
 int dot(wd_ctx* c, const Field& a, const Field& b, double* re, double* im);   // host result
 int norm2(wd_ctx* c, const Field& a, double* out);                           // host result
+int dot_hl(wd_ctx* c, const Field& a, const Field& b, double re[2]);          // Re <a, b> as hi + lo, FP64 fields
+int residual(wd_ctx* c, const Field& b, const Field& t, const Field& r, double* rr);   // r = b - t, host |r|^2
+int fold(wd_ctx* c, const Field& s, const Field& x);                          // x += s, s = 0
 int cg_update(wd_ctx* c, const Field& x, const Field& r, const Field& p, const Field& Ap);
 int cg_pupdate(wd_ctx* c, const Field& r, const Field& p);
 int cg_dot_pap(wd_ctx* c, const Field& p, const Field& Ap);
 int poly_step(wd_ctx* c, double a, double mu, double b, const Field& v, const Field& s,
               const Field& Ks, const Field& sprev, const Field& out);
-int gamma5(wd_ctx* c, const Field& in, const Field& out);
 
 // solver layer (solver.cu)
 int khat_any(wd_ctx* c, double kappa, const Field& in, const Field& out);   // FP64 fields
