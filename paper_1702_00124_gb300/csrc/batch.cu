@@ -45,8 +45,8 @@ struct SpIL {
   float4* p;
   long stride;    // Vh * nr
   int nr, r;
-  template <class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
-    SpF32{p, stride}.loadT(i * nr + r, s);
+  template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
+    SpF32{p, stride}.template loadT<RO>(i * nr + r, s);
   }
   template <class T> __device__ __forceinline__ void store(long i, const cpx<T> (&s)[12]) const {
     SpF32{p, stride}.store(i * nr + r, s);

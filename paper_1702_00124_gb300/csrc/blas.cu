@@ -20,6 +20,9 @@
 namespace wd {
 
 constexpr int BL_THREADS = 256;
+// plain load (not the read-only path: see pdl_wait)
+template <class W> __device__ __forceinline__ W ldw(const W* p) { return *p; }
+
 constexpr int SUM_BLOCKS = 8 * 152;   // eight blocks per SM: a full GB300
 
 
@@ -87,43 +90,49 @@ inline int sum_blocks(long n) { return (int)std::min<long>(SUM_BLOCKS, (n + BL_T
 // conversions site by site (a 16-bit side)
 template <class T, class In, class Out>
 __global__ void k_convert(long n, In in, Out out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cpx<T> s[12];
-  in.loadT(i, s);
+  in.template loadT<false>(i, s);
   out.store(i, s);
 }
 // the same word by word; blockIdx.y = word of the format with fewer words
 __global__ void k_f64_to_f32(long n, const double2* in, float4* out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i >= n) return;
-  const double2 a = __ldg(in + 2 * j * n + i), b = __ldg(in + (2 * j + 1) * n + i);
+  const double2 a = ldw(in + 2 * j * n + i), b = ldw(in + (2 * j + 1) * n + i);
   out[j * n + i] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
 }
 __global__ void k_f32_to_f64(long n, const float4* in, double2* out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i >= n) return;
-  const float4 v = __ldg(in + j * n + i);
+  const float4 v = ldw(in + j * n + i);
   out[2 * j * n + i] = make_double2((double)v.x, (double)v.y);
   out[(2 * j + 1) * n + i] = make_double2((double)v.z, (double)v.w);
 }
 __global__ void k_f64_to_dd(long n, const double2* in, float4* out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double2 v = __ldg(in + i);
+  const double2 v = ldw(in + i);
   const dd r(v.x), m(v.y);
   out[i] = make_float4(r.hi, r.lo, m.hi, m.lo);
 }
 __global__ void k_dd_to_f64(long n, const float4* in, double2* out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 v = __ldg(in + i);
+  const float4 v = ldw(in + i);
   out[i] = make_double2((double)dd(v.x, v.y), (double)dd(v.z, v.w));
 }
 template <class W>
 __global__ void k_copy(long n, const W* in, W* out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = __ldg(in + i);
+  if (i < n) out[i] = ldw(in + i);
 }
 
 int convert(wd_ctx* c, const Field& in, const Field& out) {
@@ -132,25 +141,25 @@ int convert(wd_ctx* c, const Field& in, const Field& out) {
   const dim3 g6(nblocks(n, BL_THREADS), 6);
   const int fi = in.fmt, fo = out.fmt;
   if (fi == WD_F64 && fo == WD_F64) {
-    k_copy<double2><<<n12, BL_THREADS, 0, c->stream>>>(12 * n, (const double2*)in.data, (double2*)out.data);
+    pdl_launch(k_copy<double2>, n12, BL_THREADS, 0, c->stream, 12 * n, (const double2*)in.data, (double2*)out.data);
   } else if (fi == WD_DD && fo == WD_DD) {
-    k_copy<float4><<<n12, BL_THREADS, 0, c->stream>>>(12 * n, (const float4*)in.data, (float4*)out.data);
+    pdl_launch(k_copy<float4>, n12, BL_THREADS, 0, c->stream, 12 * n, (const float4*)in.data, (float4*)out.data);
   } else if (fi == WD_F32 && fo == WD_F32) {
-    k_copy<float4><<<nblocks(6 * n, BL_THREADS), BL_THREADS, 0, c->stream>>>(6 * n, (const float4*)in.data,
+    pdl_launch(k_copy<float4>, nblocks(6 * n, BL_THREADS), BL_THREADS, 0, c->stream, 6 * n, (const float4*)in.data,
                                                                              (float4*)out.data);
   } else if (fi == WD_F64 && fo == WD_F32) {
-    k_f64_to_f32<<<g6, BL_THREADS, 0, c->stream>>>(n, (const double2*)in.data, (float4*)out.data);
+    pdl_launch(k_f64_to_f32, g6, BL_THREADS, 0, c->stream, n, (const double2*)in.data, (float4*)out.data);
   } else if (fi == WD_F32 && fo == WD_F64) {
-    k_f32_to_f64<<<g6, BL_THREADS, 0, c->stream>>>(n, (const float4*)in.data, (double2*)out.data);
+    pdl_launch(k_f32_to_f64, g6, BL_THREADS, 0, c->stream, n, (const float4*)in.data, (double2*)out.data);
   } else if (fi == WD_F64 && fo == WD_DD) {
-    k_f64_to_dd<<<n12, BL_THREADS, 0, c->stream>>>(12 * n, (const double2*)in.data, (float4*)out.data);
+    pdl_launch(k_f64_to_dd, n12, BL_THREADS, 0, c->stream, 12 * n, (const double2*)in.data, (float4*)out.data);
   } else if (fi == WD_DD && fo == WD_F64) {
-    k_dd_to_f64<<<n12, BL_THREADS, 0, c->stream>>>(12 * n, (const float4*)in.data, (double2*)out.data);
+    pdl_launch(k_dd_to_f64, n12, BL_THREADS, 0, c->stream, 12 * n, (const float4*)in.data, (double2*)out.data);
   } else {
     return with_fmt(in, [&](auto I) {
       return with_fmt(out, [&](auto O) {
         using T = typename Pick<decltype(I), decltype(O)>::T;
-        k_convert<T><<<nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream>>>(n, I, O);
+        pdl_launch(k_convert<T, decltype(I), decltype(O)>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, I, O);
         WD_CHECK_LAUNCH();
         return (int)WD_OK;
       });
@@ -166,13 +175,14 @@ template <class F, bool REAL>
 __global__ void k_axpby(long n, typename Words<F>::T ar, typename Words<F>::T ai, const typename Words<F>::W* x,
                         typename Words<F>::T br, typename Words<F>::T bi, const typename Words<F>::W* y,
                         typename Words<F>::W* out) {
+  pdl_enter();
   using Q = Words<F>;
   using T = typename Q::T;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cpx<T> a[Q::NC], b[Q::NC];
-  Q::get(__ldg(x + i), a);
-  Q::get(__ldg(y + i), b);
+  Q::get(ldw(x + i), a);
+  Q::get(ldw(y + i), b);
 #pragma unroll
   for (int j = 0; j < Q::NC; ++j) {
     if constexpr (REAL) a[j] = ar * a[j] + br * b[j];
@@ -183,11 +193,12 @@ __global__ void k_axpby(long n, typename Words<F>::T ar, typename Words<F>::T ai
 // the same for 16-bit fields, site by site
 template <class T, class F>
 __global__ void k_caxpby(long n, T ar, T ai, F x, T br, T bi, F y, F out) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cpx<T> a[12], b[12];
-  x.loadT(i, a);
-  y.loadT(i, b);
+  x.template loadT<false>(i, a);
+  y.template loadT<false>(i, b);
   const cpx<T> ca = mk(ar, ai), cb = mk(br, bi);
 #pragma unroll
   for (int j = 0; j < 12; ++j) a[j] = ca * a[j] + cb * b[j];
@@ -202,17 +213,17 @@ static void axpby_words(wd_ctx* c, double ar, double ai, const Field& x, double 
   const long m = nwords<F>(c->g.Vh);
   const int nb = nblocks(m, BL_THREADS);
   if (ai == 0.0 && bi == 0.0)
-    k_axpby<F, true><<<nb, BL_THREADS, 0, c->stream>>>(m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
+    pdl_launch(k_axpby<F, true>, nb, BL_THREADS, 0, c->stream, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
                                                        (const W*)y.data, (W*)out.data);
   else
-    k_axpby<F, false><<<nb, BL_THREADS, 0, c->stream>>>(m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
+    pdl_launch(k_axpby<F, false>, nb, BL_THREADS, 0, c->stream, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
                                                         (const W*)y.data, (W*)out.data);
 }
 template <class H>
 static void axpby_16(wd_ctx* c, double ar, double ai, const Field& x, double br, double bi, const Field& y,
                      const Field& out) {
   const long n = c->g.Vh;
-  k_caxpby<float><<<nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream>>>(n, (float)ar, (float)ai, sp16<H>(x), (float)br,
+  pdl_launch(k_caxpby<float, Sp16<H>>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, (float)ar, (float)ai, sp16<H>(x), (float)br,
                                                                         (float)bi, sp16<H>(y), sp16<H>(out));
 }
 
@@ -245,12 +256,13 @@ int zero(wd_ctx* c, const Field& f) {
 // inner products
 template <class T, class A, class B>
 __global__ void __launch_bounds__(BL_THREADS) k_dot(long n, A a, B b, Reduce red) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   double v[2] = {0.0, 0.0};
   if (i < n) {
     cpx<T> x[12], y[12];
-    a.loadT(i, x);
-    b.loadT(i, y);
+    a.template loadT<false>(i, x);
+    b.template loadT<false>(i, y);
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
       cpx<T> p = cmulc(x[j], y[j]);
@@ -263,18 +275,20 @@ __global__ void __launch_bounds__(BL_THREADS) k_dot(long n, A a, B b, Reduce red
 }
 // FP64 fields, word by word: <a, b>, and |a|^2
 __global__ void __launch_bounds__(BL_THREADS) k_dot64(long n, const double2* a, const double2* b, Reduce red) {
+  pdl_enter();
   double v[2] = {0.0, 0.0};
   for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
-    const double2 x = __ldg(a + i), y = __ldg(b + i);
+    const double2 x = ldw(a + i), y = ldw(b + i);
     v[0] = fma(x.y, y.y, fma(x.x, y.x, v[0]));
     v[1] = fma(-x.y, y.x, fma(x.x, y.y, v[1]));
   }
   grid_sum_hl<2>(red, v);
 }
 __global__ void __launch_bounds__(BL_THREADS) k_norm64(long n, const double2* a, Reduce red) {
+  pdl_enter();
   double v[1] = {0.0};
   for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
-    const double2 x = __ldg(a + i);
+    const double2 x = ldw(a + i);
     v[0] = fma(x.y, x.y, fma(x.x, x.x, v[0]));
   }
   grid_sum_hl<1>(red, v);
@@ -294,14 +308,14 @@ int dot(wd_ctx* c, const Field& a, const Field& b, double* re, double* im) {
   const long n = c->g.Vh;
   WD_TRY(check_sum(c));
   if (a.fmt == WD_F64 && b.fmt == WD_F64) {
-    k_dot64<<<sum_blocks(12 * n), BL_THREADS, 0, c->stream>>>(12 * n, (const double2*)a.data, (const double2*)b.data,
+    pdl_launch(k_dot64, sum_blocks(12 * n), BL_THREADS, 0, c->stream, 12 * n, (const double2*)a.data, (const double2*)b.data,
                                                               reducer_host(c));
     WD_CHECK_LAUNCH();
   } else {
     WD_TRY(with_fmt(a, [&](auto A) {
       return with_fmt(b, [&](auto B) {
         using T = typename Pick<decltype(A), decltype(B)>::T;
-        k_dot<T><<<nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream>>>(n, A, B, reducer_host(c));
+        pdl_launch(k_dot<T, decltype(A), decltype(B)>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, A, B, reducer_host(c));
         WD_CHECK_LAUNCH();
         return (int)WD_OK;
       });
@@ -319,11 +333,11 @@ int dot_hl(wd_ctx* c, const Field& a, const Field& b, double re[2]) {
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
   if (a.data == b.data) {
-    k_norm64<<<sum_blocks(n), BL_THREADS, 0, c->stream>>>(n, (const double2*)a.data, reducer_host(c));
+    pdl_launch(k_norm64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, reducer_host(c));
     WD_CHECK_LAUNCH();
     return fetch_host(c, 2, re);
   }
-  k_dot64<<<sum_blocks(n), BL_THREADS, 0, c->stream>>>(n, (const double2*)a.data, (const double2*)b.data, reducer_host(c));
+  pdl_launch(k_dot64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, (const double2*)b.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   double v[4];
   WD_TRY(fetch_host(c, 4, v));
@@ -336,7 +350,7 @@ int norm2(wd_ctx* c, const Field& a, double* out) {
   if (a.fmt != WD_F64) return dot(c, a, a, out, nullptr);
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
-  k_norm64<<<sum_blocks(n), BL_THREADS, 0, c->stream>>>(n, (const double2*)a.data, reducer_host(c));
+  pdl_launch(k_norm64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   return fetch_host(c, 1, out);
 }
@@ -345,15 +359,16 @@ int norm2(wd_ctx* c, const Field& a, double* out) {
 template <class F>
 __global__ void __launch_bounds__(BL_THREADS) k_resid(long n, const double2* b, const typename Words<F>::W* t, double2* r,
                                                       Reduce red) {
+  pdl_enter();
   double v[1] = {0.0};
   for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
-    const double2 x = __ldg(b + i);
+    const double2 x = ldw(b + i);
     double2 y;
     if constexpr (std::is_same<F, SpDD>::value) {
-      const float4 w = __ldg(t + i);
+      const float4 w = ldw(t + i);
       y = make_double2((double)dd(w.x, w.y), (double)dd(w.z, w.w));
     } else {
-      y = __ldg(t + i);
+      y = ldw(t + i);
     }
     const double2 d = make_double2(x.x - y.x, x.y - y.y);
     r[i] = d;
@@ -368,10 +383,10 @@ int residual(wd_ctx* c, const Field& b, const Field& t, const Field& r, double* 
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
   if (t.fmt == WD_F64)
-    k_resid<SpF64><<<sum_blocks(n), BL_THREADS, 0, c->stream>>>(n, (const double2*)b.data, (const double2*)t.data,
+    pdl_launch(k_resid<SpF64>, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const double2*)t.data,
                                                                 (double2*)r.data, reducer_host(c));
   else
-    k_resid<SpDD><<<sum_blocks(n), BL_THREADS, 0, c->stream>>>(n, (const double2*)b.data, (const float4*)t.data,
+    pdl_launch(k_resid<SpDD>, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const float4*)t.data,
                                                                (double2*)r.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   return fetch_host(c, 1, rr);
@@ -379,6 +394,7 @@ int residual(wd_ctx* c, const Field& b, const Field& t, const Field& r, double* 
 
 // x += s, x FP64 and s FP32 or FP64 (a solver's increment); s is left zero
 __global__ void k_fold32(long n, float4* s, double2* x) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i >= n) return;
   const float4 v = s[j * n + i];
@@ -392,6 +408,7 @@ __global__ void k_fold32(long n, float4* s, double2* x) {
   s[j * n + i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 __global__ void k_fold64(long n, double2* s, double2* x) {
+  pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double2 v = s[i], a = x[i];
@@ -402,9 +419,9 @@ int fold(wd_ctx* c, const Field& s, const Field& x) {
   const long n = c->g.Vh;
   if (x.fmt != WD_F64 || (s.fmt != WD_F64 && s.fmt != WD_F32)) return fail(WD_ERR_ARG, "fold: x FP64, s FP32 or FP64");
   if (s.fmt == WD_F32)
-    k_fold32<<<dim3(nblocks(n, BL_THREADS), 6), BL_THREADS, 0, c->stream>>>(n, (float4*)s.data, (double2*)x.data);
+    pdl_launch(k_fold32, dim3(nblocks(n, BL_THREADS), 6), BL_THREADS, 0, c->stream, n, (float4*)s.data, (double2*)x.data);
   else
-    k_fold64<<<nblocks(12 * n, BL_THREADS), BL_THREADS, 0, c->stream>>>(12 * n, (double2*)s.data, (double2*)x.data);
+    pdl_launch(k_fold64, nblocks(12 * n, BL_THREADS), BL_THREADS, 0, c->stream, 12 * n, (double2*)s.data, (double2*)x.data);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }
@@ -427,6 +444,7 @@ template <class F>
 __global__ void __launch_bounds__(BL_THREADS) k_cg_update(long n, typename Words<F>::W* x, const typename Words<F>::W* p,
                                                           typename Words<F>::W* r, const typename Words<F>::W* ap,
                                                           CGState* st, Reduce red) {
+  pdl_enter();
   using Q = Words<F>;
   using T = typename Q::T;
   if (st->flag != 0) return;
@@ -435,9 +453,9 @@ __global__ void __launch_bounds__(BL_THREADS) k_cg_update(long n, typename Words
   for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
     cpx<T> xv[Q::NC], pv[Q::NC], rv[Q::NC], av[Q::NC];
     Q::get(x[i], xv);
-    Q::get(__ldg(p + i), pv);
+    Q::get(ldw(p + i), pv);
     Q::get(r[i], rv);
-    Q::get(__ldg(ap + i), av);
+    Q::get(ldw(ap + i), av);
     T q = 0;
 #pragma unroll
     for (int j = 0; j < Q::NC; ++j) {
@@ -456,6 +474,7 @@ __global__ void __launch_bounds__(BL_THREADS) k_cg_update(long n, typename Words
 template <class P>
 __global__ void __launch_bounds__(BL_THREADS) k_cg_update16(long Vh, float4* x, P p, float4* r, const float4* ap,
                                                             CGState* st, Reduce red) {
+  pdl_enter();
   if (st->flag != 0) return;
   const float al = (float)st->alpha;
   double v[1] = {0.0};
@@ -468,7 +487,7 @@ __global__ void __launch_bounds__(BL_THREADS) k_cg_update16(long Vh, float4* x, 
     for (int h = 0; h < 2; ++h) {
       const long e = (2 * j + h) * Vh + i;
       float4 xv = x[e], rv = r[e];
-      const float4 av = __ldg(ap + e);
+      const float4 av = ldw(ap + e);
       const cpx<float> a = pv[2 * h], b = pv[2 * h + 1];
       xv = make_float4(fmaf(al, a.r, xv.x), fmaf(al, a.i, xv.y), fmaf(al, b.r, xv.z), fmaf(al, b.i, xv.w));
       rv = make_float4(fmaf(-al, av.x, rv.x), fmaf(-al, av.y, rv.y), fmaf(-al, av.z, rv.z), fmaf(-al, av.w, rv.w));
@@ -485,6 +504,7 @@ __global__ void __launch_bounds__(BL_THREADS) k_cg_update16(long Vh, float4* x, 
 // p = r + beta p, word by word
 template <class F>
 __global__ void k_cg_pupdate_w(long n, const typename Words<F>::W* r, typename Words<F>::W* p, CGState* st) {
+  pdl_enter();
   using Q = Words<F>;
   using T = typename Q::T;
   if (st->flag != 0) return;
@@ -492,7 +512,7 @@ __global__ void k_cg_pupdate_w(long n, const typename Words<F>::W* r, typename W
   if (i >= n) return;
   const T be = (T)st->beta;
   cpx<T> rv[Q::NC], pv[Q::NC];
-  Q::get(__ldg(r + i), rv);
+  Q::get(ldw(r + i), rv);
   Q::get(p[i], pv);
 #pragma unroll
   for (int j = 0; j < Q::NC; ++j) pv[j] = mk(fma_t(be, pv[j].r, rv[j].r), fma_t(be, pv[j].i, rv[j].i));
@@ -501,13 +521,14 @@ __global__ void k_cg_pupdate_w(long n, const typename Words<F>::W* r, typename W
 // 16-bit p: the scale of a site is its largest component
 template <class T, class R, class P>
 __global__ void k_cg_pupdate(long n, R r, P p, CGState* st) {
+  pdl_enter();
   if (st->flag != 0) return;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const T be = (T)st->beta;
   cpx<T> rv[12], pv[12];
-  r.loadT(i, rv);
-  p.loadT(i, pv);
+  r.template loadT<false>(i, rv);
+  p.template loadT<false>(i, pv);
 #pragma unroll
   for (int j = 0; j < 12; ++j) pv[j] = rv[j] + be * pv[j];
   p.store(i, pv);
@@ -516,14 +537,15 @@ __global__ void k_cg_pupdate(long n, R r, P p, CGState* st) {
 template <class F>
 __global__ void __launch_bounds__(BL_THREADS) k_cg_dot_pap(long n, const typename Words<F>::W* p,
                                                            const typename Words<F>::W* ap, CGState* st, Reduce red) {
+  pdl_enter();
   using Q = Words<F>;
   using T = typename Q::T;
   if (st->flag != 0) return;
   double v[1] = {0.0};
   for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
     cpx<T> pv[Q::NC], av[Q::NC];
-    Q::get(__ldg(p + i), pv);
-    Q::get(__ldg(ap + i), av);
+    Q::get(ldw(p + i), pv);
+    Q::get(ldw(ap + i), av);
     T q = 0;
 #pragma unroll
     for (int j = 0; j < Q::NC; ++j) q = fma_t(pv[j].r, av[j].r, fma_t(pv[j].i, av[j].i, q));
@@ -543,19 +565,19 @@ int cg_update(wd_ctx* c, const Field& x, const Field& r, const Field& p, const F
     return fail(WD_ERR_ARG, "cg_update: x, r, Ap must share FP64 or FP32");
   if (x.fmt == WD_F64 && p.fmt == WD_F64) {
     const long m = nwords<SpF64>(n);
-    k_cg_update<SpF64><<<sum_blocks(m), BL_THREADS, 0, c->stream>>>(m, (double2*)x.data, (const double2*)p.data,
+    pdl_launch(k_cg_update<SpF64>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (double2*)x.data, (const double2*)p.data,
                                                                     (double2*)r.data, (const double2*)Ap.data, c->cgs,
                                                                     reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_F32) {
     const long m = nwords<SpF32>(n);
-    k_cg_update<SpF32><<<sum_blocks(m), BL_THREADS, 0, c->stream>>>(m, (float4*)x.data, (const float4*)p.data,
+    pdl_launch(k_cg_update<SpF32>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (float4*)x.data, (const float4*)p.data,
                                                                     (float4*)r.data, (const float4*)Ap.data, c->cgs,
                                                                     reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_F16) {
-    k_cg_update16<<<sum_blocks(3 * n), BL_THREADS, 0, c->stream>>>(n, (float4*)x.data, sp16<__half>(p), (float4*)r.data,
+    pdl_launch(k_cg_update16<Sp16<__half>>, sum_blocks(3 * n), BL_THREADS, 0, c->stream, n, (float4*)x.data, sp16<__half>(p), (float4*)r.data,
                                                                    (const float4*)Ap.data, c->cgs, reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_BF16) {
-    k_cg_update16<<<sum_blocks(3 * n), BL_THREADS, 0, c->stream>>>(n, (float4*)x.data, sp16<__nv_bfloat16>(p),
+    pdl_launch(k_cg_update16<Sp16<__nv_bfloat16>>, sum_blocks(3 * n), BL_THREADS, 0, c->stream, n, (float4*)x.data, sp16<__nv_bfloat16>(p),
                                                                    (float4*)r.data, (const float4*)Ap.data, c->cgs,
                                                                    reducer(c));
   } else {
@@ -569,16 +591,16 @@ int cg_pupdate(wd_ctx* c, const Field& r, const Field& p) {
   const long n = c->g.Vh;
   if (r.fmt == WD_F64 && p.fmt == WD_F64) {
     const long m = nwords<SpF64>(n);
-    k_cg_pupdate_w<SpF64><<<nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream>>>(m, (const double2*)r.data,
+    pdl_launch(k_cg_pupdate_w<SpF64>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, (const double2*)r.data,
                                                                                 (double2*)p.data, c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_F32) {
     const long m = nwords<SpF32>(n);
-    k_cg_pupdate_w<SpF32><<<nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream>>>(m, (const float4*)r.data,
+    pdl_launch(k_cg_pupdate_w<SpF32>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, (const float4*)r.data,
                                                                                 (float4*)p.data, c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_F16) {
-    k_cg_pupdate<float><<<nblocks(n, 128), 128, 0, c->stream>>>(n, sp32(r), sp16<__half>(p), c->cgs);
+    pdl_launch(k_cg_pupdate<float, SpF32, Sp16<__half>>, nblocks(n, 128), 128, 0, c->stream, n, sp32(r), sp16<__half>(p), c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_BF16) {
-    k_cg_pupdate<float><<<nblocks(n, 128), 128, 0, c->stream>>>(n, sp32(r), sp16<__nv_bfloat16>(p), c->cgs);
+    pdl_launch(k_cg_pupdate<float, SpF32, Sp16<__nv_bfloat16>>, nblocks(n, 128), 128, 0, c->stream, n, sp32(r), sp16<__nv_bfloat16>(p), c->cgs);
   } else {
     return fail(WD_ERR_ARG, "cg_pupdate: r must be FP64 or FP32, p of its format or 16-bit");
   }
@@ -591,11 +613,11 @@ int cg_dot_pap(wd_ctx* c, const Field& p, const Field& Ap) {
     return fail(WD_ERR_ARG, "cg_dot_pap: p and Ap must share FP64 or FP32");
   if (p.fmt == WD_F64) {
     const long m = nwords<SpF64>(c->g.Vh);
-    k_cg_dot_pap<SpF64><<<sum_blocks(m), BL_THREADS, 0, c->stream>>>(m, (const double2*)p.data, (const double2*)Ap.data,
+    pdl_launch(k_cg_dot_pap<SpF64>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (const double2*)p.data, (const double2*)Ap.data,
                                                                      c->cgs, reducer(c));
   } else {
     const long m = nwords<SpF32>(c->g.Vh);
-    k_cg_dot_pap<SpF32><<<sum_blocks(m), BL_THREADS, 0, c->stream>>>(m, (const float4*)p.data, (const float4*)Ap.data,
+    pdl_launch(k_cg_dot_pap<SpF32>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (const float4*)p.data, (const float4*)Ap.data,
                                                                      c->cgs, reducer(c));
   }
   WD_CHECK_LAUNCH();
@@ -608,15 +630,16 @@ template <class F>
 __global__ void k_poly_step(long n, typename Words<F>::T a, typename Words<F>::T mu, typename Words<F>::T b,
                             const typename Words<F>::W* v, const typename Words<F>::W* s,
                             const typename Words<F>::W* ks, const typename Words<F>::W* sp, typename Words<F>::W* out) {
+  pdl_enter();
   using Q = Words<F>;
   using T = typename Q::T;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   cpx<T> vv[Q::NC], sv[Q::NC], kv[Q::NC], pv[Q::NC];
-  Q::get(__ldg(v + i), vv);
-  Q::get(__ldg(s + i), sv);
-  Q::get(__ldg(ks + i), kv);
-  Q::get(__ldg(sp + i), pv);
+  Q::get(ldw(v + i), vv);
+  Q::get(ldw(s + i), sv);
+  Q::get(ldw(ks + i), kv);
+  Q::get(ldw(sp + i), pv);
 #pragma unroll
   for (int j = 0; j < Q::NC; ++j) vv[j] = a * (vv[j] + mu * sv[j] - kv[j]) - b * pv[j];
   out[i] = Q::put(vv);
@@ -628,7 +651,7 @@ static void poly_step_words(wd_ctx* c, double a, double mu, double b, const Fiel
   using T = typename Words<F>::T;
   using W = typename Words<F>::W;
   const long m = nwords<F>(c->g.Vh);
-  k_poly_step<F><<<nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream>>>(m, T(a), T(mu), T(b), (const W*)v.data,
+  pdl_launch(k_poly_step<F>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, T(a), T(mu), T(b), (const W*)v.data,
                                                                        (const W*)s.data, (const W*)Ks.data,
                                                                        (const W*)sprev.data, (W*)out.data);
 }

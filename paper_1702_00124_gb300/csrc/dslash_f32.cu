@@ -71,23 +71,30 @@ __global__ void __launch_bounds__(128) k_hop_poly(HopArgs<SpF32, SpF32, SpF32, G
 __global__ void __launch_bounds__(HOP_ST_THREADS, HOP_MINB) k_hop_poly_st(HopArgs<SpF32, SpF32, SpF32, GF32R12> a, SpF32 v, SpF32 s,
                                                      SpF32 sp, float ca, float cmu, float cb) {
   extern __shared__ float4 sbuf[];
-  const long cb_ = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (cb_ >= a.g.Vh) return;
+  pdl_trigger();
+  const long site = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long cb_ = site < a.g.Vh ? site : 0;
   Staged<HOP_NST, true, HopArgs<SpF32, SpF32, SpF32, GF32R12>> S{a, cb_, {0, 0, 0, 0}, sbuf, (int)threadIdx.x,
                                                                   (int)blockDim.x};
   a.g.coords(cb_, 0, S.c);
+  S.template prologue<0>();
+  pdl_wait();
+  if (site >= a.g.Vh) {
+    cpa_wait<0>();
+    return;
+  }
   cpx<float> acc[12];
-  S.run(acc);
+  S.run_after_prologue(acc);
   cpx<float> yv[12], q[12];
-  a.y.loadT(cb_, yv);
+  a.y.template loadT<false>(cb_, yv);
   const float al = (float)a.alpha;
 #pragma unroll
   for (int j = 0; j < 12; ++j) acc[j] = yv[j] + al * acc[j];   // K s
-  v.loadT(cb_, yv);
-  s.loadT(cb_, q);
+  v.template loadT<false>(cb_, yv);
+  s.template loadT<false>(cb_, q);
 #pragma unroll
   for (int j = 0; j < 12; ++j) yv[j] = yv[j] + cmu * q[j] - acc[j];
-  sp.loadT(cb_, q);
+  sp.template loadT<false>(cb_, q);
 #pragma unroll
   for (int j = 0; j < 12; ++j) yv[j] = ca * yv[j] - cb * q[j];
   a.out.store(cb_, yv);
@@ -118,18 +125,18 @@ int khat_poly_step_f32(wd_ctx* c, double kappa, const Field& s, Field& t1, Field
     if (c->recon == WD_RECON_12) {
       HopArgs<SpF32, SpF32, SpF32, GF32R12> a{c->g, 0, sp32(t1), sp32(out), sp32(t2),
                                               GF32R12{c->gauge32r12, c->g.Vh}, a2, reducer(c), nullptr};
-      k_hop_split<float, true, 2, false><<<nbs, SPL_THREADS, 0, c->stream>>>(a, pe);
+      pdl_launch(k_hop_split<float, true, 2, false, SpF32, SpF32, SpF32, GF32R12>, nbs, SPL_THREADS, 0, c->stream, a, pe);
     } else {
       HopArgs<SpF32, SpF32, SpF32, GF32> a{c->g, 0, sp32(t1), sp32(out), sp32(t2), GF32{c->gauge32, c->g.Vh}, a2,
                                            reducer(c), nullptr};
-      k_hop_split<float, true, 2, false><<<nbs, SPL_THREADS, 0, c->stream>>>(a, pe);
+      pdl_launch(k_hop_split<float, true, 2, false, SpF32, SpF32, SpF32, GF32>, nbs, SPL_THREADS, 0, c->stream, a, pe);
     }
     WD_CHECK_LAUNCH();
   } else if (c->recon == WD_RECON_12) {
     HopArgs<SpF32, SpF32, SpF32, GF32R12> a{c->g, 0, sp32(t1), sp32(out), sp32(t2), GF32R12{c->gauge32r12, c->g.Vh},
                                             a2, reducer(c), nullptr};
-    k_hop_poly_st<<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a, sp32(v), sp32(s), sp32(sprev), (float)ca,
-                                                                      (float)cmu, (float)cb);
+    pdl_launch(k_hop_poly_st, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a, sp32(v), sp32(s), sp32(sprev), (float)ca,
+               (float)cmu, (float)cb);
     WD_CHECK_LAUNCH();
   } else {
     HopArgs<SpF32, SpF32, SpF32, GF32> a{c->g, 0, sp32(t1), sp32(out), sp32(t2), GF32{c->gauge32, c->g.Vh}, a2,

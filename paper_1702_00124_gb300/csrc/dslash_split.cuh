@@ -29,9 +29,11 @@ namespace wd {
 constexpr int SPL_SITES = 32;
 constexpr int SPL_THREADS = 8 * SPL_SITES;
 
-// u = (U or U^dag) (projected neighbour spinor) of direction D
+// u = (U or U^dag) (projected neighbour spinor) of direction D; waits for the
+// preceding kernels between the link's loads and the spinor's; false if the solver
+// has stopped
 template <int D, bool DAG, class T, class A>
-__device__ __forceinline__ void split_dir(const A& a, unsigned cb, const int (&c)[4], cpx<T> (&u)[6]) {
+__device__ __forceinline__ bool split_dir(const A& a, unsigned cb, const int (&c)[4], cpx<T> (&u)[6]) {
   constexpr int MU = D >> 1;
   constexpr bool FWD = (D & 1) == 0;
   constexpr int SG = FWD == DAG ? +1 : -1;
@@ -39,7 +41,9 @@ __device__ __forceinline__ void split_dir(const A& a, unsigned cb, const int (&c
   cpx<T> s[12], h[6], U[9];
   if constexpr (FWD) a.gauge.load(MU, a.out_par, cb, U);
   else a.gauge.load(MU, 1 - a.out_par, nb, U);
-  a.in.loadT(nb, s);
+  pdl_wait();
+  if (a.st != nullptr && a.st->flag != 0) return false;
+  a.in.template loadT<false>(nb, s);
   spin_project<MU, SG>(s, h);
   if (MU == 3 && (FWD ? c[3] == a.g.L[3] - 1 : c[3] == 0)) {
 #pragma unroll
@@ -47,6 +51,7 @@ __device__ __forceinline__ void split_dir(const A& a, unsigned cb, const int (&c
   }
   if constexpr (FWD) su3_mul(U, h, u);
   else su3_dag_mul(U, h, u);
+  return true;
 }
 
 // component J = 3 spin + colour of sum_D (1 + SG g_mu) (x) u_D; u = shared [8][6][32] + lane
@@ -104,39 +109,41 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
   constexpr bool WORDS = F64 || (std::is_same<Out, SpF32>::value && std::is_same<Y, SpF32>::value);
   static_assert(EPI != 2 || (WORDS && !F64), "the fused Chebyshev step is FP32");
   __shared__ cpx<T> sh[8 * 6 * SPL_SITES];
-  if (a.st != nullptr && a.st->flag != 0) return;
+  pdl_trigger();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long site = (long)blockIdx.x * SPL_SITES + lane;
   const bool ok = site < a.g.Vh;
   const unsigned cb = ok ? (unsigned)site : 0u;   // a lane without a site repeats site 0 and stores nothing
   int c[4];
   a.g.coords(cb, a.out_par, c);
-  // the epilogue's operands are requested before the directions' products
+  cpx<T> u[6];
+  bool run;
+  switch (w) {
+    case 0: run = split_dir<0, DAG>(a, cb, c, u); break;
+    case 1: run = split_dir<1, DAG>(a, cb, c, u); break;
+    case 2: run = split_dir<2, DAG>(a, cb, c, u); break;
+    case 3: run = split_dir<3, DAG>(a, cb, c, u); break;
+    case 4: run = split_dir<4, DAG>(a, cb, c, u); break;
+    case 5: run = split_dir<5, DAG>(a, cb, c, u); break;
+    case 6: run = split_dir<6, DAG>(a, cb, c, u); break;
+    default: run = split_dir<7, DAG>(a, cb, c, u); break;
+  }
+  if (!run) return;
+  // the epilogue's operands are requested before the products meet
   double2 y0, y1;
   float4 yv, vv, sv, pv;
   if constexpr (EPI >= 1 && WORDS) {
     if constexpr (F64) {
-      y0 = __ldg(a.y.p + w * a.y.stride + cb);
-      if (w < 4) y1 = __ldg(a.y.p + (8 + w) * a.y.stride + cb);
+      y0 = a.y.p[w * a.y.stride + cb];
+      if (w < 4) y1 = a.y.p[(8 + w) * a.y.stride + cb];
     } else if (w < 6) {
-      yv = __ldg(a.y.p + w * a.y.stride + cb);
+      yv = a.y.p[w * a.y.stride + cb];
       if constexpr (EPI == 2) {
-        vv = __ldg(pe.v.p + w * pe.v.stride + cb);
-        sv = __ldg(pe.s.p + w * pe.s.stride + cb);
-        pv = __ldg(pe.sp.p + w * pe.sp.stride + cb);
+        vv = pe.v.p[w * pe.v.stride + cb];
+        sv = pe.s.p[w * pe.s.stride + cb];
+        pv = pe.sp.p[w * pe.sp.stride + cb];
       }
     }
-  }
-  cpx<T> u[6];
-  switch (w) {
-    case 0: split_dir<0, DAG>(a, cb, c, u); break;
-    case 1: split_dir<1, DAG>(a, cb, c, u); break;
-    case 2: split_dir<2, DAG>(a, cb, c, u); break;
-    case 3: split_dir<3, DAG>(a, cb, c, u); break;
-    case 4: split_dir<4, DAG>(a, cb, c, u); break;
-    case 5: split_dir<5, DAG>(a, cb, c, u); break;
-    case 6: split_dir<6, DAG>(a, cb, c, u); break;
-    default: split_dir<7, DAG>(a, cb, c, u); break;
   }
 #pragma unroll
   for (int k = 0; k < 6; ++k) sh[(w * 6 + k) * SPL_SITES + lane] = u[k];
@@ -193,7 +200,7 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
       for (int j = 0; j < 12; ++j) acc[j] = sh2[j * SPL_SITES + lane];
       if constexpr (EPI == 1) {
         cpx<T> y[12];
-        a.y.loadT(cb, y);
+        a.y.template loadT<false>(cb, y);
 #pragma unroll
         for (int j = 0; j < 12; ++j) acc[j] = y[j] + al * acc[j];
       }
@@ -204,8 +211,17 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
     }
   }
   if constexpr (NORM) {
+    // the warps' values meet in warp 0 first: one FP64 tree in a block, not eight
+    __shared__ double shn[SPL_THREADS];
+    shn[threadIdx.x] = part[0];
+    __syncthreads();
+    part[0] = 0.0;
+    if (w == 0) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) part[0] += shn[k * 32 + lane];
+    }
     double tot[1];
-    if (grid_sum<1>(a.red, part, tot)) {
+    if (grid_sum<1, true>(a.red, part, tot)) {
       CGState* st = a.st;
       if (st != nullptr) {
         st->pAp = tot[0];
@@ -228,13 +244,19 @@ int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, 
   if (norm && (dag || !xpay)) return fail(WD_ERR_ARG, "hop: the |out|^2 epilogue exists for M_hat only");
   const int nb = nblocks(c->g.Vh, SPL_SITES);
   const SplitPoly pe{};
+  // An early start puts a kernel's blocks where the one before has left room.  FP64
+  // blocks fill the pipe of their SM, so between one block for every other SM
+  // and two for each the early ones pile up on the idle SMs: K_hat at 8^3 x 16
+  // (128 blocks) 49.6 us, early 91.7; 4^4 (4) 47.6 and 36.0, 12^4 (324) 106.9
+  // and 96.8, 16^3 x 32 (2048) 437 and 426.
+  const bool early = !std::is_same<T, double>::value || 2 * nb <= c->nsm || nb >= 2 * c->nsm;
   if (!dag) {
-    if (!xpay) k_hop_split<T, false, 0, false><<<nb, SPL_THREADS, 0, c->stream>>>(a, pe);
-    else if (!norm) k_hop_split<T, false, 1, false><<<nb, SPL_THREADS, 0, c->stream>>>(a, pe);
-    else k_hop_split<T, false, 1, true><<<nb, SPL_THREADS, 0, c->stream>>>(a, pe);
+    if (!xpay) pdl_launch_if(early, k_hop_split<T, false, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
+    else if (!norm) pdl_launch_if(early, k_hop_split<T, false, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
+    else pdl_launch_if(early, k_hop_split<T, false, 1, true, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
   } else {
-    if (!xpay) k_hop_split<T, true, 0, false><<<nb, SPL_THREADS, 0, c->stream>>>(a, pe);
-    else k_hop_split<T, true, 1, false><<<nb, SPL_THREADS, 0, c->stream>>>(a, pe);
+    if (!xpay) pdl_launch_if(early, k_hop_split<T, true, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
+    else pdl_launch_if(early, k_hop_split<T, true, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
   }
   WD_CHECK_LAUNCH();
   return WD_OK;

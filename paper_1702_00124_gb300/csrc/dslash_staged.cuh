@@ -34,11 +34,6 @@ namespace wd {
 #ifndef WD_HOP_MINB_16
 #define WD_HOP_MINB_16 6
 #endif
-// L2 prefetch size of the stencil's global reads: 0 none, 1 the link copies
-// fetch 256-byte L2 lines, 2 the neighbour spinor reads as well
-#ifndef WD_HOP_L2_256
-#define WD_HOP_L2_256 0
-#endif
 constexpr int HOP_NST = WD_HOP_STAGES;                 // link directions in flight
 // neighbour spinor of direction D + 1 loaded into registers while D is computed:
 // 0 never, 1 for FP32 spinors (0.1133 -> 0.1112 ms per hop; 16-bit spinors gain
@@ -56,39 +51,9 @@ constexpr size_t HOP_STAGE_SMEM = (size_t)(HOP_NST + 1) * 3 * HOP_ST_THREADS * s
 
 __device__ __forceinline__ void cpa16(float4* sdst, const float4* gsrc) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
-#if WD_HOP_L2_256 >= 1
-  asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;\n" ::"r"(sa), "l"(gsrc) : "memory");
-#else
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gsrc) : "memory");
-#endif
 }
 
-// read-only 16-byte load with the L2 prefetch size of WD_HOP_L2_256 >= 2
-__device__ __forceinline__ float4 ldg_stencil(const float4* p) {
-#if WD_HOP_L2_256 >= 2
-  float4 v;
-  asm volatile("ld.global.nc.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "l"(p));
-  return v;
-#else
-  return __ldg(p);
-#endif
-}
-
-// neighbour spinor of the staged stencil: FP32 through ldg_stencil, other
-// formats through their own loader
-template <class S> __device__ __forceinline__ void load_nbr(const S& in, long i, cpx<float> (&s)[12]) {
-  in.loadT(i, s);
-}
-template <> __device__ __forceinline__ void load_nbr<SpF32>(const SpF32& in, long i, cpx<float> (&s)[12]) {
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const float4 v = ldg_stencil(in.p + j * in.stride + i);
-    s[2 * j] = {v.x, v.y};
-    s[2 * j + 1] = {v.z, v.w};
-  }
-}
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cpa_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
@@ -121,7 +86,7 @@ struct Staged {
 
   template <int D> __device__ __forceinline__ void step(cpx<float> (&acc)[12]) const {
     cpx<float> s[12];
-    load_nbr(a.in, nbr<D>(), s);
+    a.in.template loadT<false>(nbr<D>(), s);
     compute<D>(acc, s);
   }
 
@@ -200,25 +165,30 @@ struct Staged {
 template <bool DAG, bool XPAY, bool NORM, class In, class Out, class Y>
 __global__ void __launch_bounds__(HOP_ST_THREADS, hop_minb<In>()) k_hop_st(HopArgs<In, Out, Y, GF32R12> a) {
   extern __shared__ float4 sbuf[];
-  if (a.st != nullptr && a.st->flag != 0) return;
-  const long cb = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  double part[1] = {0.0};
-  if (cb < a.g.Vh) {
-    Staged<HOP_NST, DAG, HopArgs<In, Out, Y, GF32R12>> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x,
-                                                         (int)blockDim.x};
-    a.g.coords(cb, a.out_par, S.c);
-    cpx<float> acc[12];
-    S.run(acc);
-    if constexpr (XPAY) {
-      cpx<float> yv[12];
-      a.y.loadT(cb, yv);
-      const float al = (float)a.alpha;
-#pragma unroll
-      for (int j = 0; j < 12; ++j) acc[j] = yv[j] + al * acc[j];
-    }
-    if constexpr (NORM) part[0] = site_norm2(acc);
-    a.out.store(cb, acc);
+  pdl_trigger();
+  const long site = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool ok = site < a.g.Vh;
+  const long cb = ok ? site : 0;               // a thread without a site repeats site 0 and stores nothing
+  Staged<HOP_NST, DAG, HopArgs<In, Out, Y, GF32R12>> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
+  a.g.coords(cb, a.out_par, S.c);
+  S.template prologue<0>();                    // the links do not depend on the kernels before
+  pdl_wait();
+  if (a.st != nullptr && a.st->flag != 0) {
+    cpa_wait<0>();
+    return;
   }
+  cpx<float> acc[12];
+  S.run_after_prologue(acc);
+  if constexpr (XPAY) {
+    cpx<float> yv[12];
+    a.y.template loadT<false>(cb, yv);
+    const float al = (float)a.alpha;
+#pragma unroll
+    for (int j = 0; j < 12; ++j) acc[j] = yv[j] + al * acc[j];
+  }
+  double part[1] = {0.0};
+  if constexpr (NORM) { if (ok) part[0] = site_norm2(acc); }
+  if (ok) a.out.store(cb, acc);
   if constexpr (NORM) {
     double tot[1];
     if (grid_sum<1>(a.red, part, tot)) {
@@ -242,12 +212,12 @@ int hop_staged(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, cons
   HopArgs<In, Out, Y, GF32R12> a{c->g, out_par, I, O, Yv, GF32R12{c->gauge32r12, c->g.Vh}, alpha, reducer(c), st};
   const int nb = nblocks(c->g.Vh, HOP_ST_THREADS);
   if (!dag) {
-    if (!xpay) k_hop_st<false, false, false><<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a);
-    else if (!norm_cg) k_hop_st<false, true, false><<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a);
-    else k_hop_st<false, true, true><<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a);
+    if (!xpay) pdl_launch(k_hop_st<false, false, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
+    else if (!norm_cg) pdl_launch(k_hop_st<false, true, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
+    else pdl_launch(k_hop_st<false, true, true, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
   } else {
-    if (!xpay) k_hop_st<true, false, false><<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a);
-    else k_hop_st<true, true, false><<<nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream>>>(a);
+    if (!xpay) pdl_launch(k_hop_st<true, false, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
+    else pdl_launch(k_hop_st<true, true, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
   }
   WD_CHECK_LAUNCH();
   return WD_OK;

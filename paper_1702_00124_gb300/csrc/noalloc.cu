@@ -58,11 +58,15 @@ int scratch_address(double2** out) {
 
 template <bool DAG, bool XPAY>
 int launch(cudaStream_t s, const Geom& g, int out_par, const double2* gauge, const double2* in, double2* out,
-           const double2* y, double alpha) {
+           const double2* y, double alpha, bool first = false) {
   using A = HopArgs<SpF64, SpF64, SpF64, GF64>;
   SpF64 I{const_cast<double2*>(in), g.Vh}, O{out, g.Vh}, Y{const_cast<double2*>(y ? y : in), g.Vh};
   A a{g, out_par, I, O, Y, GF64{gauge, g.Vh}, alpha, Reduce{nullptr, nullptr, nullptr}, nullptr};
-  k_hop_split<double, DAG, XPAY ? 1 : 0, false><<<nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s>>>(a, SplitPoly{});
+  // the first of the four hops starts after everything before it on the stream: the
+  // caller's own kernels may write the links it reads
+  auto k = k_hop_split<double, DAG, XPAY ? 1 : 0, false, SpF64, SpF64, SpF64, GF64>;
+  if (first) k<<<nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s>>>(a, SplitPoly{});
+  else pdl_launch(k, nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s, a, SplitPoly{});
   WD_CUDA(cudaGetLastError());
   return WD_OK;
 }
@@ -95,7 +99,7 @@ extern "C" int mdagm_apply_noalloc(const int dims[4], const double* gauge_eo, do
   const double2* x = (const double2*)in;
   double2* y = (double2*)out;
   const double a = -kappa * kappa;
-  WD_TRY((launch<false, false>(s, g, 1, G, x, t1, nullptr, 0.0)));   // t1 = D_oe x
+  WD_TRY((launch<false, false>(s, g, 1, G, x, t1, nullptr, 0.0, true)));   // t1 = D_oe x
   WD_TRY((launch<false, true>(s, g, 0, G, t1, t2, x, a)));           // t2 = x - k^2 D_eo t1 = M_hat x
   WD_TRY((launch<true, false>(s, g, 1, G, t2, t1, nullptr, 0.0)));   // t1 = D^dag_oe t2
   WD_TRY((launch<true, true>(s, g, 0, G, t1, y, t2, a)));            // out = M_hat^dag t2

@@ -213,23 +213,70 @@ struct Geom {
 };
 
 // ----------------------------------------------------------------------------
+// Programmatic dependent launch.  A chain of small kernels on one stream is
+// spaced by the launch latency: 4.1 us a kernel launched plainly, 1.35 us when a
+// kernel may start while its predecessor drains (GB300, chains of 128 x 128
+// threads).  The FP32 and 16-bit stencils on 12-real links, the eight-threads-per-site
+// stencil and the vector kernels call pdl_enter (or pdl_trigger at the top and pdl_wait)
+// and are launched by pdl_launch.  The register-only, double-float, force and batched
+// kernels are not: they run for tens of microseconds and lose more to plain
+// loads than the overlap gains (18-real FP32 K_hat at 32^3 x 64 680 -> 813 us,
+// double-float 2345 -> 2494 us).
+//   - Before pdl_wait a kernel reads nothing but its arguments and the link copies.
+//     Links are written by kernels that never trigger (k_step_T, k_pack,
+//     k_gauge_lowprec) and by copies, so a kernel that starts after them,
+//     or after a kernel that did, finds them complete.
+//   - pdl_wait returns when every earlier kernel of the stream has completed: each
+//     of them has waited for its own predecessor.  Spinors, sums and the solver
+//     state are read after it, by plain loads (loadT<false>; a read-only load could
+//     be moved across it).
+//   - A kernel that neither triggers nor waits starts when all before it are done.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+  pdl_trigger();
+  pdl_wait();
+}
+template <class... P, class... A>
+inline void pdl_launch_if(bool early, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);   // the caller checks cudaGetLastError
+}
+template <class... P, class... A>
+inline void pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
+  pdl_launch_if(true, k, grid, block, smem, s, a...);
+}
+
+// ----------------------------------------------------------------------------
 // spinor storage formats
+
+// RO: through the read-only path (the compiler may move the load across
+// anything); else a plain load, which stays behind pdl_wait
+template <bool RO, class W> __device__ __forceinline__ W ldx(const W* p) {
+  if constexpr (RO) return __ldg(p);
+  else return *p;
+}
 struct SpF64 {
   using real = double;
   static constexpr int fmt = WD_F64;
   double2* p;
   long stride;
-  __device__ __forceinline__ void load(long i, cpx<double> (&s)[12]) const {
-#pragma unroll
-    for (int j = 0; j < 12; ++j) { double2 v = __ldg(p + j * stride + i); s[j] = {v.x, v.y}; }
-  }
   template <class T> __device__ __forceinline__ void store(long i, const cpx<T> (&s)[12]) const {
 #pragma unroll
     for (int j = 0; j < 12; ++j) p[j * stride + i] = make_double2((double)s[j].r, (double)s[j].i);
   }
-  template <class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
+  template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
 #pragma unroll
-    for (int j = 0; j < 12; ++j) { double2 v = __ldg(p + j * stride + i); s[j] = {(T)v.x, (T)v.y}; }
+    for (int j = 0; j < 12; ++j) { double2 v = ldx<RO>(p + j * stride + i); s[j] = {(T)v.x, (T)v.y}; }
   }
 };
 
@@ -238,10 +285,10 @@ struct SpF32 {
   static constexpr int fmt = WD_F32;
   float4* p;
   long stride;
-  template <class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
+  template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      float4 v = __ldg(p + j * stride + i);
+      float4 v = ldx<RO>(p + j * stride + i);
       s[2 * j] = {(T)v.x, (T)v.y};
       s[2 * j + 1] = {(T)v.z, (T)v.w};
     }
@@ -256,7 +303,7 @@ struct SpF32 {
   struct Raw { float4 v[6]; };
   __device__ __forceinline__ void loadRaw(long i, Raw& r) const {
 #pragma unroll
-    for (int j = 0; j < 6; ++j) r.v[j] = __ldg(p + j * stride + i);
+    for (int j = 0; j < 6; ++j) r.v[j] = ldx<false>(p + j * stride + i);
   }
   template <class T> __device__ __forceinline__ static void unpack(const Raw& r, cpx<T> (&s)[12]) {
 #pragma unroll
@@ -285,11 +332,11 @@ template <class H> struct Sp16 {
   uint4* p;
   float* nrm;
   long stride;
-  template <class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
-    const float n = __ldg(nrm + i);
+  template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
+    const float n = ldx<RO>(nrm + i);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      uint4 v = __ldg(p + j * stride + i);
+      uint4 v = ldx<RO>(p + j * stride + i);
       unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -318,8 +365,8 @@ template <class H> struct Sp16 {
   }
   // components 4 j .. 4 j + 3 of site i (one stored word)
   __device__ __forceinline__ void word(long i, int j, cpx<float> (&s)[4]) const {
-    const float n = __ldg(nrm + i);
-    const uint4 v = __ldg(p + j * stride + i);
+    const float n = ldx<false>(nrm + i);
+    const uint4 v = ldx<false>(p + j * stride + i);
     const unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int q = 0; q < 4; ++q)
@@ -328,9 +375,9 @@ template <class H> struct Sp16 {
   // the stored words of one site (16-bit values and the norm), loaded ahead of their use
   struct Raw { uint4 v[3]; float n; };
   __device__ __forceinline__ void loadRaw(long i, Raw& r) const {
-    r.n = __ldg(nrm + i);
+    r.n = ldx<false>(nrm + i);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) r.v[j] = __ldg(p + j * stride + i);
+    for (int j = 0; j < 3; ++j) r.v[j] = ldx<false>(p + j * stride + i);
   }
   template <class T> __device__ __forceinline__ static void unpack(const Raw& r, cpx<T> (&s)[12]) {
 #pragma unroll
@@ -361,10 +408,10 @@ struct SpDD {
   static constexpr int fmt = WD_DD;
   float4* p;
   long stride;
-  template <class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
+  template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
-      const float4 v = __ldg(p + j * stride + i);
+      const float4 v = ldx<RO>(p + j * stride + i);
       s[j] = {dd_to<T>(dd(v.x, v.y)), dd_to<T>(dd(v.z, v.w))};
     }
   }
@@ -464,11 +511,21 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh /* [NV*32]
 }
 
 // Returns true in thread 0 of the last block, with tot[] = the grid sums.
-template <int NV>
+// WARP0: the values lie in warp 0 alone.
+template <int NV, bool WARP0 = false>
 __device__ __forceinline__ bool grid_sum(const Reduce& r, double (&v)[NV], double (&tot)[NV]) {
   __shared__ double sh[NV * 32];
   __shared__ bool last;
-  block_sum<NV>(v, sh);
+  if constexpr (WARP0) {
+    if (threadIdx.x < 32) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    }
+  } else {
+    block_sum<NV>(v, sh);
+  }
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) r.partial[blockIdx.x * NV + k] = v[k];
