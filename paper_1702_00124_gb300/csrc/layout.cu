@@ -4,42 +4,93 @@
 
 namespace wd {
 
-// One thread per lexicographic site.  The lexicographic field holds
-// nouter * nchunk * chunk doubles per site (outer index = mu or nothing);
-// the EO field is [outer][parity][nchunk][Vh] of `chunk` doubles when
-// parity < 0 (both parities), or [nchunk][Vh] for one parity.
-template <bool UNPACK>
-__global__ void k_pack(Geom g, int nouter, int nchunk, int chunk, int parity, const double* src,
-                       double* dst) {
-  const long lex = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (lex >= g.V) return;
-  const int x = (int)(lex % g.L[0]);
-  long r = lex / g.L[0];
-  const int y = (int)(r % g.L[1]); r /= g.L[1];
-  const int z = (int)(r % g.L[2]);
-  const int t = (int)(r / g.L[2]);
-  const int par = (x + y + z + t) & 1;
-  if (parity >= 0 && par != parity) return;
-  const long cb = lex >> 1;
-  const long per_site = (long)nouter * nchunk * chunk;
-  for (int o = 0; o < nouter; ++o) {
-    const long base = parity >= 0 ? 0 : (long)(o * 2 + par) * nchunk;
-    for (int j = 0; j < nchunk; ++j) {
-      const long eo = ((base + j) * g.Vh + cb) * chunk;
-      const long lx = lex * per_site + ((long)o * nchunk + j) * chunk;
-      for (int w = 0; w < chunk; ++w) {
-        if (UNPACK) dst[lx + w] = src[eo + w];
-        else dst[eo + w] = src[lx + w];
+// Lexicographic field: W elements of C doubles per site, W = nouter x nchunk
+// (outer index = mu or nothing).  EO field: [outer][parity][nchunk][Vh] elements
+// when parity < 0 (both parities), or [nchunk][Vh] for one parity.
+//
+// A block moves PACK_S consecutive lexicographic sites through shared memory: the
+// lexicographic side is then one contiguous run, the EO side runs of PACK_S / 2
+// elements (sites 2k and 2k + 1 share checkerboard index k), so both are
+// coalesced.  One site per thread left the lexicographic side at a stride of a
+// whole site (576 bytes for links).  Links at 32^3 x 64: pack 0.69 -> 0.46 ms, unpack
+// 1.97 -> 0.44 ms (2.4 GB, 0.36 ms at the copy peak).
+// The lexicographic side needs 8-byte alignment only; VEC: elements of the EO side
+// move as 16-byte words.
+constexpr int PACK_S = 64, PACK_THREADS = 256;
+
+template <int C, bool VEC, bool UNPACK>
+__global__ void __launch_bounds__(PACK_THREADS) k_pack(Geom g, int nchunk, int W, int parity, const double* src,
+                                                       double* dst) {
+  extern __shared__ double2 pack_sh[];
+  double* sh = reinterpret_cast<double*>(pack_sh);   // [PACK_S][P]
+  const int D = W * C, P = D + (C == 2 ? 2 : 1 - (D & 1));
+  const long lex0 = (long)blockIdx.x * PACK_S;
+  const int n = (int)(g.V - lex0 < PACK_S ? g.V - lex0 : PACK_S), half = n / 2;   // V is even
+  const int npar = parity >= 0 ? 1 : 2;
+  // which of the sites 2k, 2k + 1 of this block has the parity
+  auto site_of = [&](int k, int par) -> int {
+    const unsigned r = (unsigned)((lex0 >> 1) + k);
+    const unsigned r0 = g.dx.div(r), r1 = g.dy.div(r0), r2 = g.dz.div(r1);
+    const int p0 = (int)((r0 - r1 * g.dy.d) + (r1 - r2 * g.dz.d) + r2) & 1;   // parity of the site with even x
+    return 2 * k + (p0 != par ? 1 : 0);
+  };
+  if constexpr (!UNPACK) {
+    for (int e = threadIdx.x; e < n * D; e += PACK_THREADS) {
+      const int s = e / D;
+      sh[s * P + (e - s * D)] = src[lex0 * D + e];
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < npar * W * half; e += PACK_THREADS) {
+    const int q = e / half, k = e - q * half;
+    const int p = q / W, w = q - p * W;
+    const int par = parity >= 0 ? parity : p;
+    const int o = w / nchunk, j = w - o * nchunk;
+    const long base = parity >= 0 ? w : (long)(o * 2 + par) * nchunk + j;
+    const long eo = (base * g.Vh + (lex0 >> 1) + k) * C;
+    double* at = sh + site_of(k, par) * P + w * C;
+    if constexpr (VEC) {
+      if constexpr (UNPACK) *reinterpret_cast<double2*>(at) = *reinterpret_cast<const double2*>(src + eo);
+      else *reinterpret_cast<double2*>(dst + eo) = *reinterpret_cast<const double2*>(at);
+    } else {
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        if constexpr (UNPACK) at[c] = src[eo + c];
+        else dst[eo + c] = at[c];
+      }
+    }
+  }
+  if constexpr (UNPACK) {
+    __syncthreads();
+    if (parity < 0) {
+      for (int e = threadIdx.x; e < n * D; e += PACK_THREADS) {
+        const int s = e / D;
+        dst[lex0 * D + e] = sh[s * P + (e - s * D)];
+      }
+    } else {   // sites of the other parity are left as they are
+      for (int e = threadIdx.x; e < half * D; e += PACK_THREADS) {
+        const int k = e / D, s = site_of(k, parity);
+        dst[(lex0 + s) * D + (e - k * D)] = sh[s * P + (e - k * D)];
       }
     }
   }
 }
 
+template <int C, bool VEC>
+static void pack_launch(wd_ctx* c, bool unpack, int nouter, int nchunk, int parity, const double* src, double* dst) {
+  const int W = nouter * nchunk, D = W * C;
+  const size_t sm = sizeof(double) * PACK_S * (D + (C == 2 ? 2 : 1 - (D & 1)));   // links: 37.9 KB
+  const int nb = (int)((c->g.V + PACK_S - 1) / PACK_S);
+  if (unpack) k_pack<C, VEC, true><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, nchunk, W, parity, src, dst);
+  else k_pack<C, VEC, false><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, nchunk, W, parity, src, dst);
+}
+
 int pack_k(wd_ctx* c, bool unpack, int nouter, int nchunk, int chunk, int parity, const double* src,
            double* dst) {
-  const int nb = nblocks(c->g.V, 128);
-  if (unpack) k_pack<true><<<nb, 128, 0, c->stream>>>(c->g, nouter, nchunk, chunk, parity, src, dst);
-  else k_pack<false><<<nb, 128, 0, c->stream>>>(c->g, nouter, nchunk, chunk, parity, src, dst);
+  const bool aligned = ((uintptr_t)(unpack ? src : dst) & 15) == 0;   // the EO side
+  if (chunk == 2 && aligned) pack_launch<2, true>(c, unpack, nouter, nchunk, parity, src, dst);
+  else if (chunk == 2) pack_launch<2, false>(c, unpack, nouter, nchunk, parity, src, dst);
+  else pack_launch<1, false>(c, unpack, nouter, nchunk, parity, src, dst);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }
