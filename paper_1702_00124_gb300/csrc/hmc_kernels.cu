@@ -10,7 +10,13 @@
 // symmetry f_j(-c0) = (-1)^j conj(f_j(c0)), which keeps the denominator
 // 9u^2 - w^2 away from zero.  The product is reunitarised (Gram-Schmidt on
 // rows 0 and 1, row 2 = (r0 x r1)^*) and written to the FP64 links and to
-// both FP32 link copies in the same pass.
+// both FP32 link copies in the same pass.  Row 2 of the reunitarised product
+// comes from the other two, so row 2 of exp(iQ) and of the product is never formed.
+// Bound by the FP64 pipe: 472 bytes a link would take 0.58 ms at 32^3 x 64, about 400
+// FP64 instructions a link (33 ns each on 608 schedulers, 32 links) 5.3 ms.
+// Measured 7.55 ms with whole matrices, divisions and square roots; 5.62 ms with two
+// rows and Newton steps from FP32 seeds; 5.35 ms with the FP32 copies rounded by
+// integer operations.
 //
 // Random numbers: Philox4x64-10 (Salmon, Moraes, Dror, Shaw, SC'11) with key
 // (seed, 0) and counter (j, stream, 0, 0); the four words of block j give
@@ -47,25 +53,43 @@ __device__ __forceinline__ double sinc_series(double y) {
   return fma(t, y, 1.0);
 }
 
-// Q is Hermitian and traceless: Q2 = Q^2 is Hermitian, so its diagonal is
-// real and its lower triangle the conjugate of the upper one.
-__device__ __forceinline__ void cayley_hamilton_exp(const cpx<double> (&Q)[9], cpx<double> (&E)[9]) {
-  const double q00 = Q[0].r, q11 = Q[4].r, q22 = Q[8].r;
-  const cpx<double> q01 = Q[1], q02 = Q[2], q12 = Q[5];
-  const double n01 = norm2(q01), n02 = norm2(q02), n12 = norm2(q12);
-  cpx<double> Q2[9];
-  Q2[0] = mk(q00 * q00 + n01 + n02, 0.0);
-  Q2[4] = mk(q11 * q11 + n01 + n12, 0.0);
-  Q2[8] = mk(q22 * q22 + n02 + n12, 0.0);
-  Q2[1] = (q00 + q11) * q01 + q02 * conj(q12);
-  Q2[2] = (q00 + q22) * q02 + q01 * q12;
-  Q2[5] = (q11 + q22) * q12 + conj(q01) * q02;
-  Q2[3] = conj(Q2[1]);
-  Q2[6] = conj(Q2[2]);
-  Q2[7] = conj(Q2[5]);
-  const double c1 = 0.5 * (Q2[0].r + Q2[4].r + Q2[8].r);
+// 1/sqrt(x) and 1/x for x > 0 within FP32's range: an FP32 seed (relative error
+// about 1e-7) and two Newton steps, each squaring the error.  GB300 runs FP64 at
+// 1/64 of the FP32 rate; the division and square root of the language cost several
+// times as many FP64 instructions.
+__device__ __forceinline__ bool beyond_seed(double x) { return __double2hiint(x) >= 0x46000000; }   // x > 1e29, inf, NaN
+__device__ __forceinline__ double rsqrt_newton(double x) {
+  if (beyond_seed(x)) return 1.0 / sqrt(x);
+  double y = (double)rsqrtf((float)x);
+  const double hx = 0.5 * x;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) y = y * fma(-hx, y * y, 1.5);
+  return y;
+}
+__device__ __forceinline__ double rcp_newton(double x) {
+  if (beyond_seed(x)) return 1.0 / x;
+  double y = (double)(1.0f / (float)x);
+#pragma unroll
+  for (int it = 0; it < 2; ++it) y = fma(y, fma(-x, y, 1.0), y);
+  return y;
+}
+
+// Rows 0 and 1 of exp(iQ), Q Hermitian and traceless with diagonal q00, q11, q22
+// and upper triangle q01, q02, q12.  Row 2 follows from them (SU(3)).
+__device__ __forceinline__ void cayley_hamilton_rows(double q00, double q11, double q22, cpx<double> q01,
+                                                     cpx<double> q02, cpx<double> q12, cpx<double> (&E)[6]) {
+  const double n01 = fma(q01.r, q01.r, q01.i * q01.i), n02 = fma(q02.r, q02.r, q02.i * q02.i),
+               n12 = fma(q12.r, q12.r, q12.i * q12.i);
+  // Q^2, with q00 + q11 = -q22 and its permutations
+  const cpx<double> m = cmul(q01, q12);
+  const double s00 = fma(q00, q00, n01 + n02), s11 = fma(q11, q11, n01 + n12);
+  const double c1 = 0.5 * (s00 + s11 + fma(q22, q22, n02 + n12));
+  cpx<double> s01 = cfma_c(q12, q02, mk(-q22 * q01.r, -q22 * q01.i));
+  cpx<double> s02 = mk(fma(-q11, q02.r, m.r), fma(-q11, q02.i, m.i));
+  cpx<double> s12 = cfma_c(q01, q02, mk(-q00 * q12.r, -q00 * q12.i));
   // c0 = det Q = q00 q11 q22 + 2 Re(q01 q12 q02^*) - q00 |q12|^2 - q11 |q02|^2 - q22 |q01|^2
-  const double c0 = q00 * q11 * q22 + 2.0 * (q01 * q12 * conj(q02)).r - q00 * n12 - q11 * n02 - q22 * n01;
+  double c0 = 2.0 * fma(m.r, q02.r, m.i * q02.i);
+  c0 = fma(q22, fma(q00, q11, -n01), fma(-q11, n02, fma(-q00, n12, c0)));
   cpx<double> f0, f1, f2;
   if (c1 < 1e-24) {
     f0 = mk(1.0, 0.0);
@@ -73,18 +97,20 @@ __device__ __forceinline__ void cayley_hamilton_exp(const cpx<double> (&Q)[9], c
     f2 = mk(-0.5, 0.0);
   } else {
     const bool neg = c0 < 0;
-    const double c0a = fabs(c0);
-    const double t3 = c1 / 3.0;
-    const double st3 = sqrt(t3);                   // sqrt(c1/3)
-    const double c0max = 2.0 * t3 * st3;           // 2 (c1/3)^{3/2}
-    double r = c0a / c0max;
+    const double t3 = c1 * (1.0 / 3.0);
+    const double y = rsqrt_newton(t3);             // 1 / sqrt(c1 / 3)
+    const double st3 = t3 * y;
+    double r = 0.5 * fabs(c0) * (y * y * y);       // |c0| / (2 (c1/3)^{3/2})
     r = r > 1.0 ? 1.0 : r;
     // cs = cos(th/3), th = acos(r) in [0, pi/2]: the root of 4 cs^3 - 3 cs = r
     // in [cos(pi/6), 1], where the derivative 12 cs^2 - 3 lies in [6, 9]; an
-    // FP32 seed and two Newton steps in FP64
-    double cs = (double)cosf(acosf((float)r) * (1.0f / 3.0f));
+    // FP32 seed and two Newton steps whose FP64 residual is scaled by the FP32
+    // derivative: the error shrinks by 1e-7 a step
+    const float csf = cosf(acosf((float)r) * (1.0f / 3.0f));
+    const double inv = (double)(1.0f / (12.0f * csf * csf - 3.0f));
+    double cs = (double)csf;
 #pragma unroll
-    for (int it = 0; it < 2; ++it) cs -= (cs * (4.0 * cs * cs - 3.0) - r) / (12.0 * cs * cs - 3.0);
+    for (int it = 0; it < 2; ++it) cs = fma(-inv, fma(cs, fma(4.0 * cs, cs, -3.0), -r), cs);
     const double u = st3 * cs;
     const double u2 = u * u;
     const double w2 = c1 * (1.0 - cs) * (1.0 + cs);  // w = sqrt(c1) sin(th/3)
@@ -104,102 +130,101 @@ __device__ __forceinline__ void cayley_hamilton_exp(const cpx<double> (&Q)[9], c
     } else {
       sincos(u, &su, &cu);
     }
-    const cpx<double> e2 = mk(cu * cu - su * su, 2.0 * su * cu);   // exp(2iu)
-    const cpx<double> em = mk(cu, -su);                              // exp(-iu)
-    const cpx<double> h0 = (u2 - w2) * e2 + em * mk(8 * u2 * cw, 2 * u * (3 * u2 + w2) * xi0);
-    const cpx<double> h1 = (2 * u) * e2 - em * mk(2 * u * cw, -(3 * u2 - w2) * xi0);
-    const cpx<double> h2 = e2 - em * mk(cw, 3 * u * xi0);
-    const double den = 1.0 / (9 * u2 - w2);
-    f0 = den * h0;
-    f1 = den * h1;
-    f2 = den * h2;
+    const cpx<double> e2 = mk(fma(cu, cu, -su * su), 2.0 * su * cu);   // exp(2iu)
+    const cpx<double> em = mk(cu, -su);                                  // exp(-iu)
+    const double den = rcp_newton(fma(9.0, u2, -w2));
+    const double tu = 2.0 * u;
+    const cpx<double> k0 = mk(8.0 * u2 * cw, tu * fma(3.0, u2, w2) * xi0);
+    const cpx<double> k1 = mk(-tu * cw, fma(3.0, u2, -w2) * xi0);
+    const cpx<double> k2 = mk(-cw, -3.0 * u * xi0);
+    const double d0 = u2 - w2;
+    f0 = cfma(em, k0, mk(d0 * e2.r, d0 * e2.i));
+    f1 = cfma(em, k1, mk(tu * e2.r, tu * e2.i));
+    f2 = cfma(em, k2, e2);
+    f0 = mk(den * f0.r, den * f0.i);
+    f1 = mk(den * f1.r, den * f1.i);
+    f2 = mk(den * f2.r, den * f2.i);
     if (neg) {
       f0 = conj(f0);
       f1 = mk(-f1.r, f1.i);
       f2 = conj(f2);
     }
   }
-#pragma unroll
-  for (int j = 0; j < 9; ++j) E[j] = f1 * Q[j] + f2 * Q2[j];
-  E[0] = E[0] + f0;
-  E[4] = E[4] + f0;
-  E[8] = E[8] + f0;
+  E[0] = mk(fma(f2.r, s00, fma(f1.r, q00, f0.r)), fma(f2.i, s00, fma(f1.i, q00, f0.i)));
+  E[1] = cfma(f2, s01, cmul(f1, q01));
+  E[2] = cfma(f2, s02, cmul(f1, q02));
+  E[3] = cfma(f2, conj(s01), cmul(f1, conj(q01)));
+  E[4] = mk(fma(f2.r, s11, fma(f1.r, q11, f0.r)), fma(f2.i, s11, fma(f1.i, q11, f0.i)));
+  E[5] = cfma(f2, s12, cmul(f1, q12));
 }
 
+// 1/sqrt(n) of a squared row norm.  The rows come from a product of unitary
+// matrices, so n = 1 + d with d a few 1e-16: 1 - d/2 + 3 d^2/8 - 5 d^3/16 (next
+// term below 3e-21 for |d| < 1e-5) replaces the square root; links loaded less
+// accurately than that take it.
+__device__ __forceinline__ double inv_norm(double n) {
+  const double d = n - 1.0;
+  if (fabs(d) < 1e-5) return fma(d, fma(d, fma(d, -0.3125, 0.375), -0.5), 1.0);
+  return 1.0 / sqrt(n);
+}
+
+// Gram-Schmidt on rows 0 and 1, row 2 = (r0 x r1)^*
 __device__ __forceinline__ void reunitarize(cpx<double> (&U)[9]) {
   double n0 = 0;
 #pragma unroll
-  for (int j = 0; j < 3; ++j) n0 += norm2(U[j]);
-  n0 = 1.0 / sqrt(n0);
+  for (int j = 0; j < 3; ++j) n0 = fma(U[j].r, U[j].r, fma(U[j].i, U[j].i, n0));
+  n0 = inv_norm(n0);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) U[j] = n0 * U[j];
-  cpx<double> d = mk(0.0, 0.0);
+  for (int j = 0; j < 3; ++j) U[j] = mk(n0 * U[j].r, n0 * U[j].i);
+  const cpx<double> d = cfma_c(U[2], U[5], cfma_c(U[1], U[4], cmul_c(U[0], U[3])));
+  const cpx<double> md = mk(-d.r, -d.i);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) d = d + cmulc(U[j], U[3 + j]);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) U[3 + j] = U[3 + j] - d * U[j];
+  for (int j = 0; j < 3; ++j) U[3 + j] = cfma(md, U[j], U[3 + j]);
   double n1 = 0;
 #pragma unroll
-  for (int j = 0; j < 3; ++j) n1 += norm2(U[3 + j]);
-  n1 = 1.0 / sqrt(n1);
+  for (int j = 3; j < 6; ++j) n1 = fma(U[j].r, U[j].r, fma(U[j].i, U[j].i, n1));
+  n1 = inv_norm(n1);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) U[3 + j] = n1 * U[3 + j];
-  U[6] = conj(U[1] * U[5] - U[2] * U[4]);
-  U[7] = conj(U[2] * U[3] - U[0] * U[5]);
-  U[8] = conj(U[0] * U[4] - U[1] * U[3]);
-}
-
-// Hermitian traceless matrix from algebra coordinates: sum_a p_a lambda_a / 2
-__device__ __forceinline__ void alg_matrix(const double (&p)[8], double s, cpx<double> (&Q)[9]) {
-  const double h = 0.5 * s;
-  const double r3 = 0.57735026918962576451;
-  Q[0] = mk(h * (p[2] + r3 * p[7]), 0.0);
-  Q[4] = mk(h * (-p[2] + r3 * p[7]), 0.0);
-  Q[8] = mk(h * (-2.0 * r3 * p[7]), 0.0);
-  Q[1] = mk(h * p[0], -h * p[1]);
-  Q[3] = mk(h * p[0], h * p[1]);
-  Q[2] = mk(h * p[3], -h * p[4]);
-  Q[6] = mk(h * p[3], h * p[4]);
-  Q[5] = mk(h * p[5], -h * p[6]);
-  Q[7] = mk(h * p[5], h * p[6]);
+  for (int j = 3; j < 6; ++j) U[j] = mk(n1 * U[j].r, n1 * U[j].i);
+  third_row(U);
 }
 
 __global__ void __launch_bounds__(H_THREADS) k_step_T(Geom g, const double* P, double eps, double2* U64,
                                                       float2* U32, float4* U12, float4* Udd) {
   const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= 8 * g.Vh) return;
-  const long cb = tid % g.Vh;
   const int mp = (int)(tid / g.Vh);   // mu * 2 + parity
+  const long cb = tid - mp * g.Vh;
   double p[8];
 #pragma unroll
   for (int a = 0; a < 8; ++a) p[a] = P[((long)mp * 8 + a) * g.Vh + cb];
-  cpx<double> Q[9], E[9], U[9], V[9];
-  alg_matrix(p, eps, Q);
-  cayley_hamilton_exp(Q, E);
   double2* u = U64 + (long)mp * 9 * g.Vh + cb;
+  cpx<double> E[6], U[9], V[9];
 #pragma unroll
   for (int j = 0; j < 9; ++j) { double2 v = u[j * g.Vh]; U[j] = mk(v.x, v.y); }
+  // Q = eps sum_a p_a lambda_a / 2
+  const double h = 0.5 * eps, d3 = h * p[2], d8 = (h * 0.57735026918962576451) * p[7];
+  cayley_hamilton_rows(d8 + d3, d8 - d3, -2.0 * d8, mk(h * p[0], -h * p[1]), mk(h * p[3], -h * p[4]),
+                       mk(h * p[5], -h * p[6]), E);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) V[3 * i + j] = E[3 * i] * U[j] + E[3 * i + 1] * U[3 + j] + E[3 * i + 2] * U[6 + j];
+    for (int j = 0; j < 3; ++j) V[3 * i + j] = cfma(E[3 * i + 2], U[6 + j], cfma(E[3 * i + 1], U[3 + j], cmul(E[3 * i], U[j])));
   reunitarize(V);
 #pragma unroll
   for (int j = 0; j < 9; ++j) u[j * g.Vh] = make_double2(V[j].r, V[j].i);
   float2* v32 = U32 + (long)mp * 9 * g.Vh + cb;
+  float2 f[9];
 #pragma unroll
-  for (int j = 0; j < 9; ++j) v32[j * g.Vh] = make_float2((float)V[j].r, (float)V[j].i);
+  for (int j = 0; j < 9; ++j) v32[j * g.Vh] = f[j] = make_float2(f32_of(V[j].r), f32_of(V[j].i));
   float4* v12 = U12 + (long)mp * 3 * g.Vh + cb;
 #pragma unroll
-  for (int j = 0; j < 3; ++j)
-    v12[j * g.Vh] = make_float4((float)V[2 * j].r, (float)V[2 * j].i, (float)V[2 * j + 1].r, (float)V[2 * j + 1].i);
+  for (int j = 0; j < 3; ++j) v12[j * g.Vh] = make_float4(f[2 * j].x, f[2 * j].y, f[2 * j + 1].x, f[2 * j + 1].y);
   if (Udd != nullptr) {
     float4* vd = Udd + (long)mp * 9 * g.Vh + cb;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) {
-      const dd r(V[j].r), m(V[j].i);
-      vd[j * g.Vh] = make_float4(r.hi, r.lo, m.hi, m.lo);
-    }
+    for (int j = 0; j < 9; ++j)
+      vd[j * g.Vh] = make_float4(f[j].x, f32_of(V[j].r - f64_of(f[j].x)), f[j].y, f32_of(V[j].i - f64_of(f[j].y)));
   }
 }
 

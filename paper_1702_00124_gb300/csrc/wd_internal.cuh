@@ -127,6 +127,24 @@ __host__ __device__ __forceinline__ dd operator*(dd a, dd b) {
 }
 
 // ----------------------------------------------------------------------------
+// FP64 <-> FP32 by integer operations, bit for bit the hardware conversions.  Those
+// run on the FP64 pipe (33 ns per warp instruction and scheduler, as an FMA does);
+// in kernels that the FP64 pipe bounds a conversion is worth as much as an FMA.
+__device__ __forceinline__ float f32_of(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), a = hi & 0x7fffffffu;
+  if (a - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)v;   // not a normal FP32 number (or it rounds beyond): zero, tiny, huge, NaN
+  unsigned q = __funnelshift_l(lo, a - 0x38000000u, 3);   // exponent rebiased, 23 mantissa bits
+  const unsigned rem = lo << 3;                            // the bits below, against one half (even on a tie)
+  q += (rem + (q & 1u)) > 0x80000000u ? 1u : 0u;
+  return __uint_as_float(q | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double f64_of(float v) {
+  const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f800000u - 0x00800000u) return (double)v;   // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// ----------------------------------------------------------------------------
 // Gamma matrices, DeGrand-Rossi chiral basis (gamma_5 = diag(1,1,-1,-1)).
 // Each gamma_mu has one non-zero per row; row a (a = 0,1) couples to column
 // PERM[mu][a] with value i^PH[mu][a]:
