@@ -40,7 +40,7 @@ __device__ __forceinline__ void mat_mul(const cpx<T> (&A)[9], const cpx<T> (&B)[
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) C[3 * i + j] = A[3 * i] * B[j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
+    for (int j = 0; j < 3; ++j) C[3 * i + j] = cfma(A[3 * i + 2], B[6 + j], cfma(A[3 * i + 1], B[3 + j], cmul(A[3 * i], B[j])));
 }
 // C = A B^dag
 template <class T>
@@ -49,7 +49,7 @@ __device__ __forceinline__ void mat_mul_nd(const cpx<T> (&A)[9], const cpx<T> (&
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      C[3 * i + j] = A[3 * i] * conj(B[3 * j]) + A[3 * i + 1] * conj(B[3 * j + 1]) + A[3 * i + 2] * conj(B[3 * j + 2]);
+      C[3 * i + j] = cfma_c(B[3 * j + 2], A[3 * i + 2], cfma_c(B[3 * j + 1], A[3 * i + 1], cmul_c(B[3 * j], A[3 * i])));
 }
 // C = A^dag B
 template <class T>
@@ -57,7 +57,7 @@ __device__ __forceinline__ void mat_mul_dn(const cpx<T> (&A)[9], const cpx<T> (&
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) C[3 * i + j] = cmulc(A[i], B[j]) + cmulc(A[3 + i], B[3 + j]) + cmulc(A[6 + i], B[6 + j]);
+    for (int j = 0; j < 3; ++j) C[3 * i + j] = cfma_c(A[6 + i], B[6 + j], cfma_c(A[3 + i], B[3 + j], cmul_c(A[i], B[j])));
 }
 
 // h_a(X) for the projector (1 + SG g_mu): 2 x 3 complex
@@ -72,170 +72,153 @@ __device__ __forceinline__ void outer_acc(cpx<T> (&A)[9], const cpx<T> (&h)[6], 
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) A[3 * i + j] = A[3 * i + j] + h[i] * conj(k[j]) + h[3 + i] * conj(k[3 + j]);
+    for (int j = 0; j < 3; ++j) A[3 * i + j] = cfma_c(k[3 + j], h[3 + i], cfma_c(k[j], h[i], A[3 * i + j]));
 }
 
+// F += coef sum_i dRe(Y_i^dag D X_i) over n groups of NP (Y, X) pairs.
+//
+// Re(i tr(T_a M)) is the same for -M and M^dag, so -A2 U^dag counts as U A2^dag: with
+// A = A1 + A2^dag the link's derivative is that of W = U A, one matrix product
+// for all pairs of a group.  A is summed over a group's pairs in the arithmetic of the fields,
+// the groups' derivatives in FP64, and F is read and written once for all of
+// them.  A polynomial term has one group of two pairs per root; its segment of
+// roots goes out in one launch.
+//
+// Block: 32 sites of one parity x 4 directions, one warp a direction, so that
+// a site's own spinors are read once from L2 and three times from L1.
+//
+// Measured at 16^3 x 32 (FP32): the kernel before it (one thread per site, two products
+// per pair, F updated for every pair of pairs) 94 us per root, 16 roots 1.51 ms; the
+// whole polynomial force of degree 16 3.02 -> 2.39 ms.
+constexpr int F_MAXP = 16;   // pairs per launch
 template <class S, class G>
 struct ForceArgs {
   Geom g;
-  S Ye, Yo, Xe, Xo;
+  S Ye[F_MAXP], Yo[F_MAXP], Xe[F_MAXP], Xo[F_MAXP];
   G gauge;
   double coef;
-  double* F;   // [4][2][8][Vh]
+  int n;                     // groups
+  double* F;                 // [4][2][8][Vh]
 };
 
-template <int MU, class T, class S, class G>
-__device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4],
-                                          const cpx<T> (&Xs)[12], const cpx<T> (&Ys)[12]) {
-  const Geom& g = a.g;
-  const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
-  cpx<T> Xn[12], Yn[12];
-  (par ? a.Xe : a.Xo).loadT(nb, Xn);
-  (par ? a.Ye : a.Yo).loadT(nb, Yn);
-  cpx<T> A1[9], A2[9], h[6], k[6];
-#pragma unroll
-  for (int j = 0; j < 9; ++j) { A1[j] = mk<T>(0, 0); A2[j] = mk<T>(0, 0); }
-  half_of<MU, -1>(Xn, h);
-  half_of<MU, -1>(Ys, k);
-  outer_acc(A1, h, k);
-  half_of<MU, +1>(Xs, h);
-  half_of<MU, +1>(Yn, k);
-  outer_acc(A2, h, k);
-  cpx<T> U[9], W[9], t[9];
-  a.gauge.load(MU, par, cb, U);
-  mat_mul(U, A1, W);
-  mat_mul_nd(A2, U, t);
-  const T bc = (MU == 3 && c[3] == g.L[3] - 1) ? (T)-1 : (T)1;
-#pragma unroll
-  for (int j = 0; j < 9; ++j) W[j] = bc * (W[j] - t[j]);
-  T f[8];
-  proj_ta(W, f);
-  double* F = a.F + ((long)(MU * 2 + par) * 8) * g.Vh + cb;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) F[q * g.Vh] += a.coef * (double)f[q];
-}
+__device__ __forceinline__ double to_f64(float v) { return f64_of(v); }
+__device__ __forceinline__ double to_f64(double v) { return v; }
 
-template <class T, class S, class G>
-__global__ void __launch_bounds__(F_THREADS) k_force(ForceArgs<S, G> a) {
-  const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= 2 * a.g.Vh) return;
-  const int par = (int)(tid / a.g.Vh);
-  const long cb = tid - par * a.g.Vh;
-  int c[4];
-  a.g.coords(cb, par, c);
-  cpx<T> Xs[12], Ys[12];
-  (par ? a.Xo : a.Xe).loadT(cb, Xs);
-  (par ? a.Yo : a.Ye).loadT(cb, Ys);
-  force_dir<0, T>(a, par, cb, c, Xs, Ys);
-  force_dir<1, T>(a, par, cb, c, Xs, Ys);
-  force_dir<2, T>(a, par, cb, c, Xs, Ys);
-  force_dir<3, T>(a, par, cb, c, Xs, Ys);
-}
-
-int force_outer(wd_ctx* c, double coef, const Field& Ye, const Field& Yo, const Field& Xe,
-                const Field& Xo, double* F, int prec) {
-  const int nb = nblocks(2 * c->g.Vh, F_THREADS);
-  if (Ye.fmt != Yo.fmt || Ye.fmt != Xe.fmt || Ye.fmt != Xo.fmt) return fail(WD_ERR_ARG, "force: formats differ");
-  if (Ye.fmt == WD_F64 && prec == WD_F64) {
-    ForceArgs<SpF64, GF64> a{c->g, sp64(Ye), sp64(Yo), sp64(Xe), sp64(Xo), GF64{c->gauge64, c->g.Vh}, coef, F};
-    k_force<double><<<nb, F_THREADS, 0, c->stream>>>(a);
-  } else if (Ye.fmt == WD_F32) {
-    ForceArgs<SpF32, GF32> a{c->g, sp32(Ye), sp32(Yo), sp32(Xe), sp32(Xo), GF32{c->gauge32, c->g.Vh}, coef, F};
-    k_force<float><<<nb, F_THREADS, 0, c->stream>>>(a);
-  } else {
-    return fail(WD_ERR_ARG, "force: fields must be FP64 (prec FP64) or FP32");
-  }
-  WD_CHECK_LAUNCH();
-  return WD_OK;
-}
-
-// Two (Y, X) pairs in one pass: F += coef0 * dRe(Y0^dag D X0) + coef1 * dRe(Y1^dag D X1),
-// so the links and F are read and written once for both (the polynomial-term force
-// has two pairs per factor).
-template <class S, class G>
-struct ForceArgs2 {
-  Geom g;
-  S Ye[2], Yo[2], Xe[2], Xo[2];
-  G gauge;
-  double coef[2];
-  double* F;
-};
-
-template <int MU, class T, class S, class G>
-__device__ __forceinline__ void force_dir2(const ForceArgs2<S, G>& a, int par, long cb, const int (&c)[4]) {
+template <int MU, int NP, class T, class S, class G>
+__device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4], bool ok) {
   const Geom& g = a.g;
   const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
   cpx<T> U[9];
   a.gauge.load(MU, par, cb, U);
-  const T bc = (MU == 3 && c[3] == g.L[3] - 1) ? (T)-1 : (T)1;
-  double fs[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int i = 0; i < a.n; ++i) {
+    cpx<T> A[9];
 #pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    cpx<T> Xs[12], Ys[12], Xn[12], Yn[12];
-    (par ? a.Xo[p] : a.Xe[p]).loadT(cb, Xs);
-    (par ? a.Yo[p] : a.Ye[p]).loadT(cb, Ys);
-    (par ? a.Xe[p] : a.Xo[p]).loadT(nb, Xn);
-    (par ? a.Ye[p] : a.Yo[p]).loadT(nb, Yn);
-    cpx<T> A1[9], A2[9], h[6], k[6];
+    for (int j = 0; j < 9; ++j) A[j] = mk<T>(0, 0);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) { A1[j] = mk<T>(0, 0); A2[j] = mk<T>(0, 0); }
-    half_of<MU, -1>(Xn, h);
-    half_of<MU, -1>(Ys, k);
-    outer_acc(A1, h, k);
-    half_of<MU, +1>(Xs, h);
-    half_of<MU, +1>(Yn, k);
-    outer_acc(A2, h, k);
-    cpx<T> W[9], t[9];
-    mat_mul(U, A1, W);
-    mat_mul_nd(A2, U, t);
-#pragma unroll
-    for (int j = 0; j < 9; ++j) W[j] = bc * (W[j] - t[j]);
+    for (int q = 0; q < NP; ++q) {
+      const int p = i * NP + q;
+      cpx<T> s[12], h[6], k[6];
+      (par ? a.Xe[p] : a.Xo[p]).loadT(nb, s);      // A1: (1 - g) X(x+mu) with (1 - g) Y(x)
+      half_of<MU, -1>(s, h);
+      (par ? a.Yo[p] : a.Ye[p]).loadT(cb, s);
+      half_of<MU, -1>(s, k);
+      outer_acc(A, h, k);
+      (par ? a.Ye[p] : a.Yo[p]).loadT(nb, s);      // A2^dag: (1 + g) Y(x+mu) with (1 + g) X(x)
+      half_of<MU, +1>(s, h);
+      (par ? a.Xo[p] : a.Xe[p]).loadT(cb, s);
+      half_of<MU, +1>(s, k);
+      outer_acc(A, h, k);
+    }
+    cpx<T> W[9];
+    mat_mul(U, A, W);
     T f[8];
     proj_ta(W, f);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) fs[q] += a.coef[p] * (double)f[q];
+    for (int q = 0; q < 8; ++q) acc[q] += to_f64(f[q]);
   }
+  // links across the time boundary carry the fermion sign
+  const double k = (MU == 3 && c[3] == g.L[3] - 1) ? -a.coef : a.coef;
   double* F = a.F + ((long)(MU * 2 + par) * 8) * g.Vh + cb;
+  if (ok) {
 #pragma unroll
-  for (int q = 0; q < 8; ++q) F[q * g.Vh] += fs[q];
+    for (int q = 0; q < 8; ++q) F[q * g.Vh] = fma(k, acc[q], F[q * g.Vh]);
+  }
 }
 
-template <class T, class S, class G>
-__global__ void __launch_bounds__(F_THREADS) k_force2(ForceArgs2<S, G> a) {
-  const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= 2 * a.g.Vh) return;
-  const int par = (int)(tid / a.g.Vh);
-  const long cb = tid - par * a.g.Vh;
+template <class T, int NP, class S, class G>
+__global__ void __launch_bounds__(F_THREADS) k_force(ForceArgs<S, G> a) {
+  const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
+  const int par = blockIdx.y;
+  const long site = (long)blockIdx.x * 32 + lane;
+  const bool ok = site < a.g.Vh;
+  const long cb = ok ? site : 0;               // a lane without a site repeats site 0 and stores nothing
   int c[4];
   a.g.coords(cb, par, c);
-  force_dir2<0, T>(a, par, cb, c);
-  force_dir2<1, T>(a, par, cb, c);
-  force_dir2<2, T>(a, par, cb, c);
-  force_dir2<3, T>(a, par, cb, c);
+  switch (mu) {
+    case 0: force_dir<0, NP, T>(a, par, cb, c, ok); break;
+    case 1: force_dir<1, NP, T>(a, par, cb, c, ok); break;
+    case 2: force_dir<2, NP, T>(a, par, cb, c, ok); break;
+    default: force_dir<3, NP, T>(a, par, cb, c, ok); break;
+  }
 }
 
-int force_outer2(wd_ctx* c, const double coef[2], const Field* Ye, const Field* Yo, const Field* Xe,
-                 const Field* Xo, double* F) {
-  const int nb = nblocks(2 * c->g.Vh, F_THREADS);
-  const int f = Ye[0].fmt;
-  for (int p = 0; p < 2; ++p)
-    if (Ye[p].fmt != f || Yo[p].fmt != f || Xe[p].fmt != f || Xo[p].fmt != f)
-      return fail(WD_ERR_ARG, "force2: formats differ");
-  if (f == WD_F64) {
-    ForceArgs2<SpF64, GF64> a{c->g, {sp64(Ye[0]), sp64(Ye[1])}, {sp64(Yo[0]), sp64(Yo[1])},
-                              {sp64(Xe[0]), sp64(Xe[1])}, {sp64(Xo[0]), sp64(Xo[1])},
-                              GF64{c->gauge64, c->g.Vh}, {coef[0], coef[1]}, F};
-    k_force2<double><<<nb, F_THREADS, 0, c->stream>>>(a);
-  } else if (f == WD_F32) {
-    ForceArgs2<SpF32, GF32> a{c->g, {sp32(Ye[0]), sp32(Ye[1])}, {sp32(Yo[0]), sp32(Yo[1])},
-                              {sp32(Xe[0]), sp32(Xe[1])}, {sp32(Xo[0]), sp32(Xo[1])},
-                              GF32{c->gauge32, c->g.Vh}, {coef[0], coef[1]}, F};
-    k_force2<float><<<nb, F_THREADS, 0, c->stream>>>(a);
-  } else {
-    return fail(WD_ERR_ARG, "force2: fields must be FP64 or FP32");
+template <class T, int NP, class S, class G>
+static void force_launch(wd_ctx* c, const G& gauge, double coef, int n, const Field* Ye, const Field* Yo,
+                         const Field* Xe, const Field* Xo, double* F) {
+  using P = decltype(S::p);
+  const long Vh = c->g.Vh;
+  for (int i0 = 0; i0 < n; i0 += F_MAXP / NP) {
+    ForceArgs<S, G> a{};
+    a.g = c->g;
+    a.gauge = gauge;
+    a.coef = coef;
+    a.F = F;
+    a.n = n - i0 < F_MAXP / NP ? n - i0 : F_MAXP / NP;
+    for (int p = 0; p < a.n * NP; ++p) {
+      const int s = i0 * NP + p;
+      a.Ye[p] = S{(P)Ye[s].data, Vh};
+      a.Yo[p] = S{(P)Yo[s].data, Vh};
+      a.Xe[p] = S{(P)Xe[s].data, Vh};
+      a.Xo[p] = S{(P)Xo[s].data, Vh};
+    }
+    k_force<T, NP><<<dim3(nblocks(Vh, 32), 2), F_THREADS, 0, c->stream>>>(a);
+    c->launches += 1;
   }
-  WD_CHECK_LAUNCH();
+}
+
+static int force_groups(wd_ctx* c, double coef, int n, int np, const Field* Ye, const Field* Yo, const Field* Xe,
+                        const Field* Xo, double* F) {
+  const int f = Ye[0].fmt;
+  for (int p = 0; p < n * np; ++p)
+    if (Ye[p].fmt != f || Yo[p].fmt != f || Xe[p].fmt != f || Xo[p].fmt != f)
+      return fail(WD_ERR_ARG, "force: formats differ");
+  const long Vh = c->g.Vh;
+  if (f == WD_F64) {
+    const GF64 G{c->gauge64, Vh};
+    if (np == 1) force_launch<double, 1, SpF64>(c, G, coef, n, Ye, Yo, Xe, Xo, F);
+    else force_launch<double, 2, SpF64>(c, G, coef, n, Ye, Yo, Xe, Xo, F);
+  } else if (f == WD_F32) {
+    const GF32 G{c->gauge32, Vh};
+    if (np == 1) force_launch<float, 1, SpF32>(c, G, coef, n, Ye, Yo, Xe, Xo, F);
+    else force_launch<float, 2, SpF32>(c, G, coef, n, Ye, Yo, Xe, Xo, F);
+  } else {
+    return fail(WD_ERR_ARG, "force: fields must be FP64 or FP32");
+  }
+  WD_CUDA(cudaGetLastError());
   return WD_OK;
+}
+
+int force_outer(wd_ctx* c, double coef, const Field& Ye, const Field& Yo, const Field& Xe,
+                const Field& Xo, double* F, int prec) {
+  if (Ye.fmt == WD_F64 && prec != WD_F64) return fail(WD_ERR_ARG, "force: fields must be FP64 (prec FP64) or FP32");
+  return force_groups(c, coef, 1, 1, &Ye, &Yo, &Xe, &Xo, F);
+}
+
+// n groups of two pairs: entries 2 i and 2 i + 1 of the arrays
+int force_pairs(wd_ctx* c, double coef, int n, const Field* Ye, const Field* Yo, const Field* Xe, const Field* Xo,
+                double* F) {
+  return force_groups(c, coef, n, 2, Ye, Yo, Xe, Xo, F);
 }
 
 // ----------------------------------------------------------------------------
@@ -251,6 +234,9 @@ __device__ __forceinline__ void step(const Geom& g, int (&c)[4], int mu, int d) 
   c[mu] = v < 0 ? v + g.L[mu] : (v >= g.L[mu] ? v - g.L[mu] : v);
 }
 
+// One thread per site, every direction in turn.  Measured at 32^3 x 64 (FP32): 1.60 ms,
+// 1.26 ms with the products as FMA chains.  One warp per direction with the planes
+// unrolled took 1.39 ms (links of 18 reals: three at a time fill the registers).
 template <class T, class G>
 __global__ void __launch_bounds__(F_THREADS) k_gauge_force(Geom g, G gauge, double coef, double* F) {
   const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -299,7 +285,7 @@ __global__ void __launch_bounds__(F_THREADS) k_gauge_force(Geom g, G gauge, doub
     proj_ta(W, f);
     double* Fp = F + ((long)(mu * 2 + par) * 8) * g.Vh + cb;
 #pragma unroll
-    for (int a = 0; a < 8; ++a) Fp[a * g.Vh] += coef * (double)f[a];
+    for (int a = 0; a < 8; ++a) Fp[a * g.Vh] = fma(coef, (double)f[a], Fp[a * g.Vh]);
   }
 }
 

@@ -91,13 +91,14 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
   const int nseg = (m + seg - 1) / seg;
   WsGuard w(c);
   // buf: the R of one segment; ro / mr / mro: D_oe R, M_hat R and D^dag_oe M_hat R
-  // of those R, formed while K_hat is applied to them in the segment rebuild
-  std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg);
-  Field L, Ln, ML, cur, Lo, MLo, KR;
+  // of those R, formed while K_hat is applied to them in the segment rebuild;
+  // L, lo, ml, mlo: the same of the segment's L
+  std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg), L(seg), lo(seg), ml(seg), mlo(seg);
+  Field Ln, cur, KR;
   for (auto& x : cp) WD_TRY(w.get(f, &x));
-  for (auto* v : {&buf, &ro, &mr, &mro})
+  for (auto* v : {&buf, &ro, &mr, &mro, &L, &lo, &ml, &mlo})
     for (auto& x : *v) WD_TRY(w.get(f, &x));
-  for (Field* x : {&L, &Ln, &ML, &cur, &Lo, &MLo, &KR}) WD_TRY(w.get(f, x));
+  for (Field* x : {&Ln, &cur, &KR}) WD_TRY(w.get(f, x));
   const double k2 = kappa * kappa;
   auto seg_end = [&](int s) { return std::min((s + 1) * seg, m) - 1; };
   // backward pass: R_{m-1} = v, R_{k-1} = (K - r_k) R_k; keep R at segment ends
@@ -107,7 +108,8 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
     if (k > 0) WD_TRY(k_minus(c, kappa, rr[k], ri[k], cur, cur));
   }
   // forward pass over k with L_k; R_k rebuilt from the segment's checkpoint
-  WD_TRY(convert(c, v, L));
+  WD_TRY(convert(c, v, L[0]));
+  std::vector<Field> Ye(2 * seg), Yo(2 * seg), Xe(2 * seg), Xo(2 * seg);
   for (int s = 0; s < nseg; ++s) {
     const int a = s * seg, b = seg_end(s);
     WD_TRY(convert(c, cp[s], buf[b - a]));
@@ -122,30 +124,31 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
     }
     for (int k = a; k <= b; ++k) {
       const int j = k - a;
-      const Field& R = buf[j];
-      // Lo = D_oe L, ML = M_hat L, MLo = D^dag_oe ML (the odd halves of L~ and
+      // lo = D_oe L, ml = M_hat L, mlo = D^dag_oe ml (the odd halves of L~ and
       // (M L)~), and the same for R (kept from the rebuild except for its
-      // first vector): each used twice below
-      WD_TRY(hop(c, 1, false, L, Lo, nullptr, 0.0, false, false));
-      WD_TRY(hop(c, 0, false, Lo, ML, &L, -k2, false, false));
-      WD_TRY(hop(c, 1, true, ML, MLo, nullptr, 0.0, false, false));
+      // first vector)
+      WD_TRY(hop(c, 1, false, L[j], lo[j], nullptr, 0.0, false, false));
+      WD_TRY(hop(c, 0, false, lo[j], ml[j], &L[j], -k2, false, false));
+      WD_TRY(hop(c, 1, true, ml[j], mlo[j], nullptr, 0.0, false, false));
       if (j == 0) {
-        WD_TRY(hop(c, 1, false, R, ro[0], nullptr, 0.0, false, false));
-        WD_TRY(hop(c, 0, false, ro[0], mr[0], &R, -k2, false, false));
+        WD_TRY(hop(c, 1, false, buf[0], ro[0], nullptr, 0.0, false, false));
+        WD_TRY(hop(c, 0, false, ro[0], mr[0], &buf[0], -k2, false, false));
         WD_TRY(hop(c, 1, true, mr[0], mro[0], nullptr, 0.0, false, false));
       }
-      // Re((M R)~^dag dD L~) and Re((M L)~^dag dD R~), one pass over the links
-      const double cf[2] = {-coef * scale * k2, -coef * scale * k2};
-      const Field Ye[2] = {mr[j], ML}, Yo[2] = {mro[j], MLo}, Xe[2] = {L, R}, Xo[2] = {Lo, ro[j]};
-      WD_TRY(force_outer2(c, cf, Ye, Yo, Xe, Xo, F));
+      // Re((M R)~^dag dD L~) and Re((M L)~^dag dD R~)
+      Ye[2 * j] = mr[j], Yo[2 * j] = mro[j], Xe[2 * j] = L[j], Xo[2 * j] = lo[j];
+      Ye[2 * j + 1] = ml[j], Yo[2 * j + 1] = mlo[j], Xe[2 * j + 1] = buf[j], Xo[2 * j + 1] = ro[j];
       if (k < m - 1) {
-        // K L = M^dag (M L) = ML - kappa^2 D^dag_eo MLo: one more hop
-        WD_TRY(hop(c, 0, true, MLo, Ln, &ML, -k2, false, false));
+        // K L = M^dag (M L) = ml - kappa^2 D^dag_eo mlo: one more hop
+        WD_TRY(hop(c, 0, true, mlo[j], KR, &ml[j], -k2, false, false));
         c->nmat += 1;
-        WD_TRY(caxpby(c, 1.0, 0.0, Ln, -rr[k], ri[k], L, Ln));   // (K - conj r_k) L
-        std::swap(L, Ln);
+        const Field& nx = k < b ? L[j + 1] : Ln;
+        WD_TRY(caxpby(c, 1.0, 0.0, KR, -rr[k], ri[k], L[j], nx));   // (K - conj r_k) L
       }
     }
+    // the segment's pairs in one pass over the links and F
+    WD_TRY(force_pairs(c, -coef * scale * k2, b - a + 1, Ye.data(), Yo.data(), Xe.data(), Xo.data(), F));
+    std::swap(L[0], Ln);
   }
   return WD_OK;
 }

@@ -785,6 +785,7 @@ int caxpby(wd_ctx* c, double ar, double ai, const Field& x, double br, double bi
 int zero(wd_ctx* c, const Field& f);
 int dot(wd_ctx* c, const Field& a, const Field& b, double* re, double* im);   // host result
 int norm2(wd_ctx* c, const Field& a, double* out);                           // host result
+int norm2_any(wd_ctx* c, const Field& b, const Field& x, double* bb, bool* nonzero);   // |b|^2, x != 0
 int dot_hl(wd_ctx* c, const Field& a, const Field& b, double re[2]);          // Re <a, b> as hi + lo, FP64 fields
 int residual(wd_ctx* c, const Field& b, const Field& t, const Field& r, double* rr);   // r = b - t, host |r|^2
 int fold(wd_ctx* c, const Field& s, const Field& x);                          // x += s, s = 0
@@ -816,8 +817,8 @@ int gaussian_draw_k(wd_ctx* c, int what, int parity, uint64_t seed, uint64_t str
 // force layer (force.cu)
 int force_outer(wd_ctx* c, double coef, const Field& Ye, const Field& Yo, const Field& Xe,
                 const Field& Xo, double* F, int prec);
-int force_outer2(wd_ctx* c, const double coef[2], const Field* Ye, const Field* Yo, const Field* Xe,
-                 const Field* Xo, double* F);
+int force_pairs(wd_ctx* c, double coef, int n, const Field* Ye, const Field* Yo, const Field* Xe, const Field* Xo,
+                double* F);
 
 // polynomial helpers (host)
 struct PolyCoef {
