@@ -346,6 +346,33 @@ int dot_hl(wd_ctx* c, const Field& a, const Field& b, double re[2]) {
   return WD_OK;
 }
 
+// |b|^2 and whether x has an entry that is not zero, in one pass
+__global__ void __launch_bounds__(BL_THREADS) k_norm_any(long n, const double2* b, const double2* x, Reduce red) {
+  pdl_enter();
+  double v[2] = {0.0, 0.0};
+  bool any = false;
+  for (long i = (long)blockIdx.x * BL_THREADS + threadIdx.x; i < n; i += (long)gridDim.x * BL_THREADS) {
+    const double2 w = ldw(b + i), z = ldw(x + i);
+    v[0] = fma(w.y, w.y, fma(w.x, w.x, v[0]));
+    any = any || z.x != 0.0 || z.y != 0.0;     // true for NaN
+  }
+  v[1] = any ? 1.0 : 0.0;
+  grid_sum_hl<2>(red, v);
+}
+int norm2_any(wd_ctx* c, const Field& b, const Field& x, double* bb, bool* nonzero) {
+  if (b.fmt != WD_F64 || x.fmt != WD_F64) return fail(WD_ERR_ARG, "norm2_any: FP64 fields");
+  WD_TRY(check_sum(c));
+  const long n = 12 * c->g.Vh;
+  pdl_launch(k_norm_any, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const double2*)x.data,
+             reducer_host(c));
+  WD_CHECK_LAUNCH();
+  double v[4];
+  WD_TRY(fetch_host(c, 4, v));
+  *bb = v[0];
+  *nonzero = v[1] != 0.0;
+  return WD_OK;
+}
+
 int norm2(wd_ctx* c, const Field& a, double* out) {
   if (a.fmt != WD_F64) return dot(c, a, a, out, nullptr);
   WD_TRY(check_sum(c));

@@ -257,7 +257,9 @@ static int cg_core(wd_ctx* c, const Op& op, const Field& b, const Field& x, cons
 
   wd_cg_info inf{};
   double bb;
-  WD_TRY(norm2(c, b, &bb));
+  bool guess = false;   // x holds a guess other than zero
+  if (x_zero) WD_TRY(norm2(c, b, &bb));
+  else WD_TRY(norm2_any(c, b, x, &bb, &guess));
   if (bb == 0.0) {
     WD_TRY(zero(c, x));
     if (info) *info = inf;
@@ -280,8 +282,10 @@ static int cg_core(wd_ctx* c, const Op& op, const Field& b, const Field& x, cons
   Field r, xs, rs, ps, aps;
   WD_TRY(w.get(WD_F64, &r));
   double rr;
-  if (x_zero) {   // r = b without applying A
-    WD_TRY(zero(c, x));
+  if (!guess) {
+    // r = b - A 0 is b itself: no operator application (n + 1 FP64-accurate K_hat
+    // for K P: 51 of 400 ms of a filtered solve at 32^3 x 64)
+    if (x_zero) WD_TRY(zero(c, x));
     WD_TRY(convert(c, b, r));
     rr = bb;
   } else {
