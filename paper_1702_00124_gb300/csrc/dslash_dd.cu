@@ -8,23 +8,25 @@
 // six products, each product is split exactly by an FMA (two-product, with
 // the cross terms of the low words), the high words are summed exactly
 // (two-sum) and every rounding error is added into one FP32 word.  The site's
-// accumulator keeps that unnormalised form across its directions and is
-// normalised once, before the store.  Links are read one row (column, for
-// U^dag) at a time, where they are used, to keep the live register set small.
+// sum over directions keeps that unnormalised form, folded once half way and
+// normalised before the store.
 //
-// One hop is DD_DIRS_PER_LAUNCH directions per launch (forward and backward
-// hop each): the first launch writes the output, later ones add to it, the
-// last applies the y + alpha D x epilogue.  All eight directions in one kernel
-// overflow the instruction cache ("no instruction" stalls in ncu, 1.24 ms per
-// hop at 32^3 x 64); one direction per launch re-reads and re-writes the
-// partial sum three times (0.77 ms); two directions per launch took 0.60 ms,
-// and 0.58 ms with the register cap of four 128-thread blocks per SM (a few
-// bytes of spill in the last launch).
-#include "dslash_impl.cuh"
+// Eight threads per site, one per neighbour direction, as dslash_split.cuh: a block
+// is 32 sites, warp w forms U h (U^dag h) of direction w, the products meet in
+// shared memory and the block's warps share the components of the sum.  The
+// product is one piece of code for every direction (rows or conjugated columns by
+// stride and sign), the projection one per mu, so the kernel stays inside the
+// instruction cache; all eight directions unrolled in one thread did not (1.24 ms per hop at
+// 32^3 x 64), which had split the hop into two launches with a partial sum in
+// between.  Bound by FP32 issue: about 9,000 FP32 instructions a site, 230 us per hop at
+// 32^3 x 64; 1.6 GB would take 240 us.
+// K_hat in a chain (conversions included), two launches -> this: 32^3 x 64 2349 -> 1992 us,
+// 24^4 501 -> 338, 16^3 x 32 201 -> 143, 8^3 x 16 113 -> 30, 4^4 115 -> 19; without the
+// links' way through shared memory 2126, 365, 157, 29, 27.  Error against FP64
+// 3.26e-15 at every size, as before (3.52e-15 without the fold half way).
+#include "dslash_staged.cuh"
 
 namespace wd {
-
-constexpr int DD_DIRS_PER_LAUNCH = 2;
 
 // value s + c with c the collected rounding errors (not normalised)
 struct lz {
@@ -61,11 +63,9 @@ __device__ __forceinline__ lz lz_first(dd x, dd y) {
 }
 __device__ __forceinline__ dd neg(dd x) { return dd(-x.hi, -x.lo); }
 __device__ __forceinline__ dd lz_norm(const lz& a) { return dd_2sum(a.s, a.c); }
-
-// one double-float link element U_{row,col} of U_mu(x) (x = site i of parity par)
-__device__ __forceinline__ cpx<dd> link_dd(const GDD& G, int mu, int par, long i, int row, int col) {
-  const float4 v = __ldg(G.p + ((long)(mu * 2 + par) * 9 + 3 * row + col) * G.stride + i);
-  return {dd(v.x, v.y), dd(v.z, v.w)};
+__device__ __forceinline__ lz lz_fold(const lz& a) {
+  const dd n = lz_norm(a);
+  return {n.hi, n.lo};
 }
 
 // a += i^K u
@@ -87,18 +87,12 @@ __device__ __forceinline__ void lz_add_ipow(lzc& a, const lzc& u) {
   }
 }
 
-// (U h)_c (DAG = false) or (U^dag h)_c (DAG = true) for one colour vector h
-// of the half spinor, from row (column) c of U
-template <bool DAG>
-__device__ __forceinline__ lzc su3_row_lz(const cpx<dd> (&u)[3], const cpx<dd>* h) {
+// sum_k u_k h_k of one colour vector h: re = ur vr - ui vi, im = ur vi + ui vr
+__device__ __forceinline__ lzc row_lz(const cpx<dd> (&u)[3], const cpx<dd>* h) {
   lz re, im;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const cpx<dd> v = h[k];
-    // U h:     re = ur vr - ui vi, im = ur vi + ui vr
-    // U^dag h: re = ur vr + ui vi, im = ur vi - ui vr
-    const dd ui_re = DAG ? u[k].i : neg(u[k].i);
-    const dd ui_im = DAG ? neg(u[k].i) : u[k].i;
     if (k == 0) {
       re = lz_first(u[k].r, v.r);
       im = lz_first(u[k].r, v.i);
@@ -106,117 +100,143 @@ __device__ __forceinline__ lzc su3_row_lz(const cpx<dd> (&u)[3], const cpx<dd>* 
       lz_fma(re, u[k].r, v.r);
       lz_fma(im, u[k].r, v.i);
     }
-    lz_fma(re, ui_re, v.i);
-    lz_fma(im, ui_im, v.r);
+    lz_fma(re, neg(u[k].i), v.i);
+    lz_fma(im, u[k].i, v.r);
   }
   return {re, im};
 }
 
-// acc += (1 + SG g_mu) (x) [U or U^dag] h, colour by colour
-template <int MU, int SG, bool DAG>
-__device__ __forceinline__ void mul_accum_lz(const GDD& G, int par, long i, const cpx<dd> (&h)[6],
-                                             lzc (&acc)[12]) {
+__device__ __forceinline__ dd flip(dd x, unsigned m) {   // m = 0 or the sign bit
+  return dd(__uint_as_float(__float_as_uint(x.hi) ^ m), __uint_as_float(__float_as_uint(x.lo) ^ m));
+}
+
+// h = psi_a + sg i^k psi_PERM(a) of the neighbour spinor, sg = +1 (m = 0) or -1 (m = the sign bit)
+template <int MU>
+__device__ __forceinline__ void project_dd(const SpDD& in, long i, unsigned m, cpx<dd> (&h)[6]) {
   using Gm = Gam<MU>;
-  constexpr int q0 = (SG > 0 ? 0 : 2) - Gm::k0;
-  constexpr int q1 = (SG > 0 ? 0 : 2) - Gm::k1;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    cpx<dd> u[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) u[k] = DAG ? link_dd(G, MU, par, i, k, c) : link_dd(G, MU, par, i, c, k);
-    const lzc o0 = su3_row_lz<DAG>(u, h);
-    const lzc o1 = su3_row_lz<DAG>(u, h + 3);
-    lz_add_ipow<0>(acc[c], o0);
-    lz_add_ipow<0>(acc[3 + c], o1);
-    lz_add_ipow<q0>(acc[3 * Gm::p0 + c], o0);
-    lz_add_ipow<q1>(acc[3 * Gm::p1 + c], o1);
+  for (int c = 0; c < 6; ++c) {
+    const int cc = c < 3 ? c : c - 3;
+    const int q = 3 * (c < 3 ? Gm::p0 : Gm::p1) + cc;
+    const float4 a = in.p[c * in.stride + i], b = in.p[q * in.stride + i];
+    cpx<dd> v = {dd(b.x, b.y), dd(b.z, b.w)};
+    v = c < 3 ? ipow<Gm::k0>(v) : ipow<Gm::k1>(v);
+    h[c] = {dd(a.x, a.y) + flip(v.r, m), dd(a.z, a.w) + flip(v.i, m)};
   }
 }
 
-// forward and backward hop in direction MU (same structure as hop_dir)
-template <int MU, bool DAG>
-__device__ __forceinline__ void hop_dir_lz(const HopArgs<SpDD, SpDD, SpDD, GDD>& a, long cb, const int (&c)[4],
-                                           lzc (&acc)[12]) {
-  constexpr int SF = DAG ? +1 : -1;
-  constexpr int SB = -SF;
-  const Geom& g = a.g;
-  {
-    const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
-    cpx<dd> s[12], h[6];
-    a.in.loadT(nb, s);
-    spin_project<MU, SF>(s, h);
-    if (MU == 3 && c[3] == g.L[3] - 1) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) h[j] = {neg(h[j].r), neg(h[j].i)};
-    }
-    mul_accum_lz<MU, SF, false>(a.gauge, a.out_par, cb, h, acc);
-  }
-  {
-    const long nb = g.template nbr<2 * MU + 1>((unsigned)cb, c);
-    cpx<dd> s[12], h[6];
-    a.in.loadT(nb, s);
-    spin_project<MU, SB>(s, h);
-    if (MU == 3 && c[3] == 0) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) h[j] = {neg(h[j].r), neg(h[j].i)};
-    }
-    mul_accum_lz<MU, SB, true>(a.gauge, 1 - a.out_par, nb, h, acc);
-  }
+// component of sum_D (1 + SG g_mu) (x) u_D: of the upper spins (LOW = 0, j = 3 spin + colour)
+// or of spin LOW = 2, 3 (j = colour); u = shared [8][6][32] + lane
+template <int LOW, int D, bool DAG>
+__device__ __forceinline__ void sum_term(const float4* u, int j, lzc& acc) {
+  constexpr int MU = D >> 1;
+  constexpr int SG = ((D & 1) == 0) == DAG ? +1 : -1;
+  using Gm = Gam<MU>;
+  constexpr bool first = LOW == Gm::p0;
+  constexpr int q = LOW == 0 ? 0 : (SG > 0 ? 0 : 2) - (first ? Gm::k0 : Gm::k1);
+  const int k = LOW == 0 ? j : (first ? j : 3 + j);
+  const float4 v = u[(D * 6 + k) * 32];
+  lz_add_ipow<q>(acc, lzc{{v.x, v.y}, {v.z, v.w}});
+}
+template <int LOW, bool DAG> __device__ __forceinline__ lzc sum_dirs(const float4* u, int j) {
+  lzc acc = {{0.f, 0.f}, {0.f, 0.f}};
+  sum_term<LOW, 0, DAG>(u, j, acc);
+  sum_term<LOW, 1, DAG>(u, j, acc);
+  sum_term<LOW, 2, DAG>(u, j, acc);
+  sum_term<LOW, 3, DAG>(u, j, acc);
+  // half way the error word is folded in: the later errors add to a smaller word
+  acc = {lz_fold(acc.r), lz_fold(acc.i)};
+  sum_term<LOW, 4, DAG>(u, j, acc);
+  sum_term<LOW, 5, DAG>(u, j, acc);
+  sum_term<LOW, 6, DAG>(u, j, acc);
+  sum_term<LOW, 7, DAG>(u, j, acc);
+  return acc;
 }
 
-// directions MU0 .. MU0 + NMU - 1 of one hop
-template <int MU0, int NMU, bool DAG, bool FIRST, bool LAST, bool XPAY>
-__global__ void __launch_bounds__(128, 4) k_hop_dd(HopArgs<SpDD, SpDD, SpDD, GDD> a) {
-  const long cb = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (cb >= a.g.Vh) return;
+template <bool DAG, bool XPAY>
+__global__ void __launch_bounds__(256, 3) k_hop_dd(HopArgs<SpDD, SpDD, SpDD, GDD> a) {
+  extern __shared__ float4 sh[];              // [8][6][32] products, [9][256] links
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long site = (long)blockIdx.x * 32 + lane;
+  const bool ok = site < a.g.Vh;
+  const unsigned cb = ok ? (unsigned)site : 0u;   // a lane without a site repeats site 0 and stores nothing
   int c[4];
   a.g.coords(cb, a.out_par, c);
-  lzc acc[12];
-  if constexpr (FIRST) {
+  const bool fwd = (w & 1) == 0;
+  const int mu = w >> 1;
+  unsigned nb;
+  switch (w) {
+    case 0: nb = a.g.nbr<0>(cb, c); break;
+    case 1: nb = a.g.nbr<1>(cb, c); break;
+    case 2: nb = a.g.nbr<2>(cb, c); break;
+    case 3: nb = a.g.nbr<3>(cb, c); break;
+    case 4: nb = a.g.nbr<4>(cb, c); break;
+    case 5: nb = a.g.nbr<5>(cb, c); break;
+    case 6: nb = a.g.nbr<6>(cb, c); break;
+    default: nb = a.g.nbr<7>(cb, c); break;
+  }
+  // the nine link entries come through shared memory (cp.async, each thread its own):
+  // in flight from the start without holding registers, and before the wait, for
+  // they do not depend on the kernels before.  Rows of U_mu(x), or columns of
+  // U_mu(x - mu) for the conjugate
+  const long gs = a.gauge.stride;
+  const float4* q = a.gauge.p + (long)(mu * 2 + (fwd ? a.out_par : 1 - a.out_par)) * 9 * gs + (fwd ? cb : nb);
+  const long row = fwd ? 3 * gs : gs, col = fwd ? gs : 3 * gs;
+  float4* lk = sh + 8 * 6 * 32 + threadIdx.x;
 #pragma unroll
-    for (int j = 0; j < 12; ++j) acc[j] = {{0.f, 0.f}, {0.f, 0.f}};
-  } else {
+  for (int k = 0; k < 3; ++k)
 #pragma unroll
-    for (int j = 0; j < 12; ++j) {
-      const float4 v = __ldg(a.out.p + j * a.out.stride + cb);
-      acc[j] = {{v.x, v.y}, {v.z, v.w}};
+    for (int l = 0; l < 3; ++l) cpa16(lk + (3 * k + l) * 256, q + k * row + l * col);
+  cpa_commit();
+  pdl_wait();
+  const unsigned m = fwd == DAG ? 0u : 0x80000000u;   // projector 1 + SG g_mu
+  cpx<dd> h[6];
+  switch (mu) {
+    case 0: project_dd<0>(a.in, nb, m, h); break;
+    case 1: project_dd<1>(a.in, nb, m, h); break;
+    case 2: project_dd<2>(a.in, nb, m, h); break;
+    default: project_dd<3>(a.in, nb, m, h); break;
+  }
+  // the antiperiodic sign goes into the link
+  const bool wrap = mu == 3 && (fwd ? c[3] == a.g.L[3] - 1 : c[3] == 0);
+  const unsigned mr = wrap ? 0x80000000u : 0u, mi = mr ^ (fwd ? 0u : 0x80000000u);
+  cpa_wait<0>();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cpx<dd> u[3];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const float4 v = lk[(3 * k + l) * 256];
+      u[l] = {flip(dd(v.x, v.y), mr), flip(dd(v.z, v.w), mi)};
     }
+    const lzc o0 = row_lz(u, h), o1 = row_lz(u, h + 3);
+    sh[(w * 6 + k) * 32 + lane] = make_float4(o0.r.s, o0.r.c, o0.i.s, o0.i.c);
+    sh[(w * 6 + 3 + k) * 32 + lane] = make_float4(o1.r.s, o1.r.c, o1.i.s, o1.i.c);
   }
-  hop_dir_lz<MU0, DAG>(a, cb, c, acc);
-  if constexpr (NMU > 1) hop_dir_lz<MU0 + 1, DAG>(a, cb, c, acc);
-  if constexpr (NMU > 2) {
-    hop_dir_lz<MU0 + 2, DAG>(a, cb, c, acc);
-    hop_dir_lz<MU0 + 3, DAG>(a, cb, c, acc);
-  }
-  // normalise, apply the epilogue and store one complex at a time
+  __syncthreads();
+  // component w, for warps 0 to 3 also component 8 + w (three for every scheduler)
+  const float4* us = sh + lane;
   const dd al(a.alpha);
-#pragma unroll
-  for (int j = 0; j < 12; ++j) {
-    cpx<dd> r = {lz_norm(acc[j].r), lz_norm(acc[j].i)};
-    if constexpr (LAST && XPAY) {
-      const float4 v = __ldg(a.y.p + j * a.y.stride + cb);
+  for (int j = w; j < 12; j += 8) {
+    const lzc t = j < 6 ? sum_dirs<0, DAG>(us, j) : (j < 9 ? sum_dirs<2, DAG>(us, j - 6) : sum_dirs<3, DAG>(us, j - 9));
+    cpx<dd> r = {lz_norm(t.r), lz_norm(t.i)};
+    if constexpr (XPAY) {
+      const float4 v = a.y.p[j * a.y.stride + cb];
       r = cpx<dd>{dd(v.x, v.y), dd(v.z, v.w)} + al * r;
     }
-    a.out.p[j * a.out.stride + cb] = make_float4(r.r.hi, r.r.lo, r.i.hi, r.i.lo);
+    if (ok) a.out.p[j * a.out.stride + cb] = make_float4(r.r.hi, r.r.lo, r.i.hi, r.i.lo);
   }
 }
 
 template <bool DAG, bool XPAY>
-static int hop_dd_split(wd_ctx* c, const HopArgs<SpDD, SpDD, SpDD, GDD>& a) {
-  const int nb = nblocks(c->g.Vh, 128);
-  if constexpr (DD_DIRS_PER_LAUNCH == 4) {
-    k_hop_dd<0, 4, DAG, true, true, XPAY><<<nb, 128, 0, c->stream>>>(a);
-  } else if constexpr (DD_DIRS_PER_LAUNCH == 2) {
-    k_hop_dd<0, 2, DAG, true, false, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    k_hop_dd<2, 2, DAG, false, true, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    c->launches += 1;
-  } else {
-    k_hop_dd<0, 1, DAG, true, false, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    k_hop_dd<1, 1, DAG, false, false, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    k_hop_dd<2, 1, DAG, false, false, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    k_hop_dd<3, 1, DAG, false, true, XPAY><<<nb, 128, 0, c->stream>>>(a);
-    c->launches += 3;
-  }
+static int hop_dd_launch(wd_ctx* c, const HopArgs<SpDD, SpDD, SpDD, GDD>& a) {
+  constexpr int sm = (8 * 6 * 32 + 9 * 256) * (int)sizeof(float4);   // 61 KB: three blocks per SM
+  const int nb = nblocks(c->g.Vh, 32);
+  // early starts pile FP32-bound blocks up on idle SMs as they do FP64-bound ones (dslash_split.cuh)
+  const bool early = 2 * nb <= c->nsm || nb >= 2 * c->nsm;
+  WD_CUDA(cudaFuncSetAttribute(k_hop_dd<DAG, XPAY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  pdl_launch_if(early, k_hop_dd<DAG, XPAY>, nb, 256, sm, c->stream, a);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }
@@ -228,12 +248,12 @@ int hop_dd(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, 
   if (c->gauge_dd == nullptr) return fail(WD_ERR_STATE, "hop_dd: no double-float link copy");
   if (norm_cg || in_cg) return fail(WD_ERR_ARG, "hop_dd: not used inside queued CG iterations");
   if (out.data == in.data || (y && out.data == y->data))
-    return fail(WD_ERR_ARG, "hop_dd: the output accumulates in place and may not alias an input");
+    return fail(WD_ERR_ARG, "hop_dd: the output may not alias an input");
   SpDD I = spdd(in), O = spdd(out), Y = y ? spdd(*y) : O;
   HopArgs<SpDD, SpDD, SpDD, GDD> a{c->g, out_par, I, O, Y, GDD{c->gauge_dd, c->g.Vh}, alpha,
                                     Reduce{nullptr, nullptr, nullptr}, nullptr};
-  if (!dag) return y ? hop_dd_split<false, true>(c, a) : hop_dd_split<false, false>(c, a);
-  return y ? hop_dd_split<true, true>(c, a) : hop_dd_split<true, false>(c, a);
+  if (!dag) return y ? hop_dd_launch<false, true>(c, a) : hop_dd_launch<false, false>(c, a);
+  return y ? hop_dd_launch<true, true>(c, a) : hop_dd_launch<true, false>(c, a);
 }
 
 }  // namespace wd
