@@ -24,6 +24,7 @@
 namespace wd {
 
 constexpr int B_MAXR = 8;   // right-hand sides per lattice
+constexpr int BHOP_NST = 2; // link directions in flight of the staged batched hop
 
 enum BField { BF_P = 0, BF_AP, BF_R, BF_X, BF_T1, BF_T2, BF_N };
 
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(256) k_bhop(BArgs a, int fin, int fout, int fy
 // is computed (dslash_staged.cuh); the item's lattice supplies geometry, links
 // and fields.  Blocks of HOP_ST_THREADS items.
 template <bool DAG, bool XPAY, bool NORM>
-__global__ void __launch_bounds__(HOP_ST_THREADS, HOP_MINB) k_bhop_st(BArgs a, int fin, int fout, int fy) {
+__global__ void __launch_bounds__(HOP_ST_THREADS, 5) k_bhop_st(BArgs a, int fin, int fout, int fy) {
   extern __shared__ float4 sbuf[];
   const BItem it = b_item(a, blockIdx.x, 1);
   const BLat* L = it.L;
@@ -260,10 +261,11 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, HOP_MINB) k_bhop_st(BArgs a, i
     using HA = HopArgs<SpIL, SpIL, SpIL, GF32R12>;
     const HA ha{L->g, a.out_par, in, out, in, GF32R12{L->g12, L->g.Vh}, 0.0, Reduce{nullptr, nullptr, nullptr},
                 nullptr};
-    Staged<HOP_NST, DAG, HA> S{ha, it.cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
+    Staged<BHOP_NST, 0, DAG, HA> S{ha, it.cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
     L->g.coords(it.cb, a.out_par, S.c);
     cpx<float> acc[12];
-    S.run(acc);
+    S.template prologue<0>();
+    S.run_after_prologue(acc);
     if constexpr (XPAY) {
       cpx<float> yv[12];
       SpIL{L->f[fy], stride, L->nr, r}.loadT(it.cb, yv);
@@ -586,7 +588,7 @@ static int b_hop(wd_batch* b, int out_par, bool dag, int fin, int fout, int fy, 
     else k_bhop<D, X, N, R, 1><<<b->nblocks, b->threads, 0, b->stream>>>(a, fin, fout, fy);                \
   } while (0)
   if (r12 && b->staged) {
-#define WD_BS(D, X, N) k_bhop_st<D, X, N><<<b->nblocks, HOP_ST_THREADS, HOP_STAGE_SMEM, b->stream>>>(a, fin, fout, fy)
+#define WD_BS(D, X, N) k_bhop_st<D, X, N><<<b->nblocks, HOP_ST_THREADS, hop_smem<GF32R12>(BHOP_NST), b->stream>>>(a, fin, fout, fy)
     if (!dag) {
       if (fy < 0) WD_BS(false, false, false);
       else if (norm) WD_BS(false, true, true);

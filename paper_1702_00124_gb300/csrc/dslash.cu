@@ -63,7 +63,9 @@ int hop(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, con
   if (in.fmt == WD_F64) s = hop_f64(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
   else if (in.fmt == WD_F32) s = hop_f32(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
   else if (in.fmt == WD_DD) s = hop_dd(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
-  else s = hop_h16(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
+  else if (in.fmt == WD_F16) s = hop_f16(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
+  else if (in.fmt == WD_BF16) s = hop_bf16(c, out_par, dag, in, out, y, alpha, norm_cg, in_cg);
+  else s = fail(WD_ERR_ARG, "hop: unknown field format");
   if (s != WD_OK) return s;
   prof_end(c, e0, hop_bytes(in.fmt, out.fmt, y != nullptr, gauge_link_bytes(c, in.fmt), c->g.Vh), in.fmt);
   return WD_OK;

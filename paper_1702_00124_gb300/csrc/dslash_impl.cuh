@@ -312,42 +312,15 @@ inline SpF64 sp64(const Field& f) { return SpF64{(double2*)f.data, f.stride}; }
 inline SpF32 sp32(const Field& f) { return SpF32{(float4*)f.data, f.stride}; }
 template <class H> inline Sp16<H> sp16(const Field& f) { return Sp16<H>{(uint4*)f.data, f.norm, f.stride}; }
 
-template <class T, class In, class Out, class Y>
-int hop_with_gauge(wd_ctx* c, int out_par, bool dag, In in, Out out, Y y, bool xpay, double alpha,
-                   bool norm_cg, bool in_cg, bool use64) {
-  Reduce red = reducer(c);
-  CGState* st = (norm_cg || in_cg) ? c->cgs : nullptr;
-  // tuning key: formats of in / out / y and the link storage
-  const long long base = ((long long)In::fmt * 8 + Out::fmt) * 8 + (xpay ? Y::fmt : 7);
-  const bool may_tune = !in_cg;
-  if constexpr (std::is_same<T, dd>::value) {
-    GDD G{c->gauge_dd, c->g.Vh};
-    HopArgs<In, Out, Y, GDD> a{c->g, out_par, in, out, y, G, alpha, red, st};
-    return launch_hop<T>(c, dag, xpay, norm_cg, base * 4 + 3, may_tune, a);
-  } else {
-  if (use64) {
-    GF64 G{c->gauge64, c->g.Vh};
-    HopArgs<In, Out, Y, GF64> a{c->g, out_par, in, out, y, G, alpha, red, st};
-    return launch_hop<T>(c, dag, xpay, norm_cg, base * 4 + 0, may_tune, a);
-  }
-  if (c->recon == WD_RECON_12) {
-    GF32R12 G{c->gauge32r12, c->g.Vh};
-    HopArgs<In, Out, Y, GF32R12> a{c->g, out_par, in, out, y, G, alpha, red, st};
-    return launch_hop<T>(c, dag, xpay, norm_cg, base * 4 + 2, may_tune, a);
-  }
-  GF32 G{c->gauge32, c->g.Vh};
-  HopArgs<In, Out, Y, GF32> a{c->g, out_par, in, out, y, G, alpha, red, st};
-  return launch_hop<T>(c, dag, xpay, norm_cg, base * 4 + 1, may_tune, a);
-  }
-}
-
 // per-family dispatchers (one translation unit each)
 int hop_f64(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
             double alpha, bool norm_cg, bool in_cg);
 int hop_f32(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
             double alpha, bool norm_cg, bool in_cg);
-int hop_h16(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
+int hop_f16(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
             double alpha, bool norm_cg, bool in_cg);
+int hop_bf16(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
+             double alpha, bool norm_cg, bool in_cg);
 int hop_dd(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
            double alpha, bool norm_cg, bool in_cg);
 inline SpDD spdd(const Field& f) { return SpDD{(float4*)f.data, f.stride}; }

@@ -16,11 +16,12 @@
 // 16^3 x 32 127 -> 111 (floor 93: 840 instructions x 33 ns on 608 schedulers),
 // 24^3 x 48 540 -> 518; from 32^4 on both take the same (808 and 810 us).
 //
-// FP32 and 16-bit, up to SPLIT_MAX_VH: there a hop takes as long as one
-// thread's eight dependent neighbour reads; here all eight are in flight at
-// once.  FP32 K_hat in a chain: 8^3 x 16 26.1 -> 19.7 us, 12^3 x 24 26.5 -> 27.0,
-// 16^4 28.0 -> 34.1 (the products' way through shared memory costs more than the
-// latency it hides).
+// FP32 and 16-bit, up to SPLIT_MAX_VH and SPLIT_MAX_VH_16: there a hop takes as long as
+// one thread's eight neighbour reads; here all eight are in flight at once.  K_hat in
+// a chain, the staged pipeline against this: FP32 (last hop with the Chebyshev
+// step) 4^4 12.5 -> 8.8 us, 8^3 x 16 14.4 -> 13.5, 12^4 16.8 -> 15.2, with
+// 18-real links 25.1 -> 15.1, 12^3 x 24 17.6 and 27.0; BF16 4^4 18.0 -> 14.7, 8^3 x 16 22.0 -> 21.4,
+// 8^2 x 12 x 16 22.5 and 27.3.
 #pragma once
 #include "dslash_staged.cuh"
 
@@ -96,15 +97,9 @@ template <bool DAG, class T> __device__ __forceinline__ cpx<T> split_sum_at(int 
   }
 }
 
-// operands of the Chebyshev step out = ca (v + cmu s - (y + alpha D in)) - cb sp
-struct SplitPoly {
-  SpF32 v, s, sp;
-  float ca, cmu, cb;
-};
-
 // EPI 0: out = D in; 1: out = y + alpha D in; 2: the Chebyshev step on that (FP32)
 template <class T, bool DAG, int EPI, bool NORM, class In, class Out, class Y, class G>
-__global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G> a, SplitPoly pe) {
+__global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G> a, HopPoly pe) {
   constexpr bool F64 = std::is_same<Out, SpF64>::value;
   constexpr bool WORDS = F64 || (std::is_same<Out, SpF32>::value && std::is_same<Y, SpF32>::value);
   static_assert(EPI != 2 || (WORDS && !F64), "the fused Chebyshev step is FP32");
@@ -235,15 +230,18 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
 // the lines lie between the last size that gains and the first that does not (above)
 constexpr long SPLIT_MAX_VH_F64 = 500000;
 constexpr long SPLIT_MAX_VH = 12288;
+constexpr long SPLIT_MAX_VH_16 = 4096;   // a 16-bit output is finished by one warp of the eight
 static_assert(SPLIT_MAX_VH_F64 / SPL_SITES < RED_MAX_BLOCKS, "a slot per block in the grid sum");
 
-inline bool split_eligible(const wd_ctx* c, bool f64) { return c->g.Vh <= (f64 ? SPLIT_MAX_VH_F64 : SPLIT_MAX_VH); }
+inline bool split_eligible(const wd_ctx* c, int fmt) {   // fmt of the input spinors
+  return c->g.Vh <= (fmt == WD_F64 ? SPLIT_MAX_VH_F64 : fmt == WD_F32 ? SPLIT_MAX_VH : SPLIT_MAX_VH_16);
+}
 
 template <class T, class In, class Out, class Y, class G>
 int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, Y, G>& a) {
   if (norm && (dag || !xpay)) return fail(WD_ERR_ARG, "hop: the |out|^2 epilogue exists for M_hat only");
   const int nb = nblocks(c->g.Vh, SPL_SITES);
-  const SplitPoly pe{};
+  const HopPoly pe{};
   // An early start puts a kernel's blocks where the one before has left room.  FP64
   // blocks fill the pipe of their SM, so between one block for every other SM
   // and two for each the early ones pile up on the idle SMs: K_hat at 8^3 x 16
@@ -263,23 +261,20 @@ int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, 
 }
 
 // FP32 arithmetic on the context's 12-real or 18-real links: eight threads per
-// site on small lattices, else the staged or the register-only kernel
-template <class In, class Out, class Y>
-int hop_r12(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, const Y& Yv, bool xpay, double alpha,
-            bool norm_cg, bool in_cg) {
-  if (!split_eligible(c, false)) return hop_staged(c, out_par, dag, I, O, Yv, xpay, alpha, norm_cg, in_cg);
-  HopArgs<In, Out, Y, GF32R12> a{c->g, out_par, I, O, Yv, GF32R12{c->gauge32r12, c->g.Vh}, alpha, reducer(c),
-                                 (norm_cg || in_cg) ? c->cgs : nullptr};
-  return hop_split<float>(c, dag, xpay, norm_cg, a);
+// site on small lattices, else the staged pipeline
+template <class In, class Out, class Y, class G>
+int hop_fp32(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, const Y& Yv, const G& gauge, bool xpay,
+             double alpha, bool norm_cg, bool in_cg) {
+  const HopArgs<In, Out, Y, G> a{c->g, out_par, I, O, Yv, gauge, alpha, reducer(c), (norm_cg || in_cg) ? c->cgs : nullptr};
+  if (split_eligible(c, In::fmt)) return hop_split<float>(c, dag, xpay, norm_cg, a);
+  return hop_staged(c, dag, xpay, norm_cg, a);
 }
 template <class In, class Out, class Y>
-int hop_r18(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, const Y& Yv, bool xpay, double alpha,
-            bool norm_cg, bool in_cg) {
-  if (!split_eligible(c, false))
-    return hop_with_gauge<float>(c, out_par, dag, I, O, Yv, xpay, alpha, norm_cg, in_cg, false);
-  HopArgs<In, Out, Y, GF32> a{c->g, out_par, I, O, Yv, GF32{c->gauge32, c->g.Vh}, alpha, reducer(c),
-                              (norm_cg || in_cg) ? c->cgs : nullptr};
-  return hop_split<float>(c, dag, xpay, norm_cg, a);
+int hop_links(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, const Y& Yv, bool xpay, double alpha,
+              bool norm_cg, bool in_cg) {
+  if (c->recon == WD_RECON_12)
+    return hop_fp32(c, out_par, dag, I, O, Yv, GF32R12{c->gauge32r12, c->g.Vh}, xpay, alpha, norm_cg, in_cg);
+  return hop_fp32(c, out_par, dag, I, O, Yv, GF32{c->gauge32, c->g.Vh}, xpay, alpha, norm_cg, in_cg);
 }
 
 }  // namespace wd

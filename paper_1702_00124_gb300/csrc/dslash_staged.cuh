@@ -1,74 +1,120 @@
-// Staged hopping stencil for 12-real FP32 links (Section 3.1 of the paper:
-// Wilson fermions, even-odd preconditioning), any spinor storage format.
+// Staged hopping stencil for FP32 links (Section 3.1 of the paper: Wilson
+// fermions, even-odd preconditioning), any spinor storage format.
 //
-// The register-only kernel holds a direction's neighbour loads in registers,
-// so at the register count that allows five 128-thread blocks per SM too few
-// bytes are in flight to keep HBM busy (long-scoreboard stalls dominate).
-// Here every thread runs its own software pipeline over the eight neighbour
-// directions: the three float4 of the link of direction D + NST are copied
-// global -> shared with cp.async.cg while direction D is computed, so NST
-// directions' links are in flight without holding registers.  A thread reads
-// only the shared words it copied itself, so no block barrier is needed; NST + 1
-// buffers make the buffer being refilled one whose values were consumed in the
-// previous step.  Neighbour spinors are read through L1 (each is read by eight
-// sites, several of them in the same block).
+// One thread per site.  A register-only kernel holds a direction's neighbour
+// loads in registers, so at the register count that fills an SM too few bytes are in
+// flight (long-scoreboard stalls dominate).  Here every thread runs its own
+// software pipeline over the eight neighbour directions: the link of direction
+// D + NST is copied global -> shared with cp.async while direction D is computed, so
+// NST directions' links are in flight without holding registers, and the neighbour
+// spinors of the next SA directions are in registers.  A thread reads only the
+// shared words it copied itself, so no block barrier is needed; NST + 1 buffers
+// make the buffer being refilled one whose values were consumed in the previous
+// step.  Neighbour spinors are read through L1 (each is read by eight sites, several
+// of them in the same block).
+//
+// How deep (hop_depth): a lattice of many waves of blocks is bound by HBM and wants
+// resident blocks; one that fits the SMs at once is bound by the chain of
+// eight neighbour reads, and registers that no second block would use hold more of them
+// in flight.  Per FP32 K_hat in a chain on 152 SMs, depth (NST, SA, blocks per SM):
+//                 blocks  (2,1,5)  (4,2,4)  (6,3,3)  (7,5,2)
+//   12^3 x 24        162    27.2     22.9     19.9     17.1 us
+//   16^4             256    26.6     22.9     19.7     17.3
+//   16^3 x 32        512    28.9     24.3     26.8     26.4
+//   16^2 x 32^2     1024    47.1     42.9     46.9     49.2
+//   24^4            1296    66.5     75.1     70.2     75.8
+//   32^3 x 64       8192     405      408      407      441
+// so: two blocks per SM if all fit, three if all fit, four while that takes no
+// more waves than the full occupancy.  16-bit spinors, (2,1,6) (4,3,4) (6,4,3): 12^3 x 24
+// 32.8, 25.5, 21.3; 16^3 x 32 38.8, 27.4, 30.2; 32^3 x 64 356, 388, 398.
 #pragma once
+#include <atomic>
+
 #include "dslash_impl.cuh"
 
 namespace wd {
 
-#ifndef WD_HOP_STAGES
-#define WD_HOP_STAGES 2
-#endif
-#ifndef WD_HOP_SPIN_AHEAD
-#define WD_HOP_SPIN_AHEAD 1
-#endif
-// resident 128-thread blocks per SM the register budget is set for: FP32
-// spinors five (96 registers), 16-bit spinors six (80 registers; their words
-// take half the registers).  Measured per hop at 32^3 x 64 in the K_hat chain:
-// FP32 0.1112 ms (five, with the look-ahead below) against 0.1163 (six) and
-// 0.1283 (seven); BF16 0.1070 ms (six) against 0.1104 (five).
-#ifndef WD_HOP_MINB_F32
-#define WD_HOP_MINB_F32 5
-#endif
-#ifndef WD_HOP_MINB_16
-#define WD_HOP_MINB_16 6
-#endif
-constexpr int HOP_NST = WD_HOP_STAGES;                 // link directions in flight
-// neighbour spinor of direction D + 1 loaded into registers while D is computed:
-// 0 never, 1 for FP32 spinors (0.1133 -> 0.1112 ms per hop; 16-bit spinors gain
-// nothing), 2 for every format
-template <class In> constexpr bool spin_ahead() {
-  return WD_HOP_SPIN_AHEAD >= 2 || (WD_HOP_SPIN_AHEAD == 1 && std::is_same<In, SpF32>::value);
-}
-template <class In> constexpr int hop_minb() {
-  return std::is_same<In, SpF32>::value ? WD_HOP_MINB_F32 : WD_HOP_MINB_16;
-}
-constexpr int HOP_MINB = WD_HOP_MINB_F32;              // FP32 kernels outside the template
-static_assert(HOP_NST >= 1 && HOP_NST <= 7, "one to seven directions in flight");
 constexpr int HOP_ST_THREADS = 128;
-constexpr size_t HOP_STAGE_SMEM = (size_t)(HOP_NST + 1) * 3 * HOP_ST_THREADS * sizeof(float4);
 
 __device__ __forceinline__ void cpa16(float4* sdst, const float4* gsrc) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
 
+__device__ __forceinline__ void cpa8(float2* sdst, const float2* gsrc) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cpa_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-template <int NST, bool DAG, class A>
+// a thread's link in a buffer [words][threads]: 12 reals as three 16-byte words,
+// 18 reals as nine 8-byte words
+template <class G> struct LinkBuf;
+template <> struct LinkBuf<GF32R12> {
+  using W = float4;
+  static constexpr int N = 3, NU = 6;
+  __device__ __forceinline__ static void copy(W* s, int nt, const W* g, long stride) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) cpa16(s + j * nt, g + j * stride);
+  }
+  __device__ __forceinline__ static void read(const W* s, int nt, cpx<float> (&U)[6]) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float4 v = s[j * nt];
+      U[2 * j] = {v.x, v.y};
+      U[2 * j + 1] = {v.z, v.w};
+    }
+  }
+  __device__ __forceinline__ static void mul(const cpx<float> (&U)[6], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
+    su3_mul_r12(U, h, o);
+  }
+  __device__ __forceinline__ static void dag_mul(const cpx<float> (&U)[6], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
+    su3_dag_mul_r12(U, h, o);
+  }
+};
+template <> struct LinkBuf<GF32> {
+  using W = float2;
+  static constexpr int N = 9, NU = 9;
+  __device__ __forceinline__ static void copy(W* s, int nt, const W* g, long stride) {
+#pragma unroll
+    for (int j = 0; j < 9; ++j) cpa8(s + j * nt, g + j * stride);
+  }
+  __device__ __forceinline__ static void read(const W* s, int nt, cpx<float> (&U)[9]) {
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      const float2 v = s[j * nt];
+      U[j] = {v.x, v.y};
+    }
+  }
+  __device__ __forceinline__ static void mul(const cpx<float> (&U)[9], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
+    su3_mul(U, h, o);
+  }
+  __device__ __forceinline__ static void dag_mul(const cpx<float> (&U)[9], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
+    su3_dag_mul(U, h, o);
+  }
+};
+template <class G> constexpr size_t hop_smem(int nst) {
+  return (size_t)(nst + 1) * LinkBuf<G>::N * HOP_ST_THREADS * sizeof(typename LinkBuf<G>::W);
+}
+
+template <int NST, int SA, bool DAG, class A>
 struct Staged {
+  using G = typename std::remove_cv<decltype(A::gauge)>::type;
+  using LB = LinkBuf<G>;
   static constexpr int NB = NST + 1;          // buffers
+  static_assert(NST >= 1 && NST <= 7 && SA >= 0 && SA <= 7, "one to seven directions in flight");
   const A& a;
   long cb;
   int c[4];
-  float4* buf;                                // [NB][3][blockDim.x]
+  float4* buf;                                // [NB][LB::N][threads]
   int tid, nt;
 
-  __device__ __forceinline__ float4* slot(int b, int k) const { return buf + (b * 3 + k) * nt + tid; }
+  __device__ __forceinline__ typename LB::W* slot(int b) const {
+    return reinterpret_cast<typename LB::W*>(buf) + b * LB::N * nt + tid;
+  }
 
   template <int D> __device__ __forceinline__ long nbr() const { return a.g.template nbr<D>((unsigned)cb, c); }
 
@@ -77,9 +123,7 @@ struct Staged {
       constexpr int MU = D >> 1;
       const int lpar = (D & 1) == 0 ? a.out_par : 1 - a.out_par;
       const long li = (D & 1) == 0 ? cb : nbr<D>();
-      const float4* q = a.gauge.p + ((long)(MU * 2 + lpar) * 3) * a.gauge.stride + li;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) cpa16(slot(D % NB, j), q + j * a.gauge.stride);
+      LB::copy(slot(D % NB), nt, a.gauge.p + ((long)(MU * 2 + lpar) * LB::N) * a.gauge.stride + li, a.gauge.stride);
     }
     cpa_commit();                              // possibly empty: keeps one group per step
   }
@@ -90,27 +134,29 @@ struct Staged {
     compute<D>(acc, s);
   }
 
-  // the same with the spinor of this direction loaded one step earlier (cur) and
-  // the next direction's issued now (nxt)
-  template <int D, class R> __device__ __forceinline__ void step_ahead(cpx<float> (&acc)[12], const R& cur,
-                                                                       R& nxt) const {
-    if constexpr (D + 1 < 8) a.in.loadRaw(nbr<D + 1>(), nxt);
-    cpx<float> s[12];
-    a.in.unpack(cur, s);
-    compute<D>(acc, s);
+  // the same with SA directions' spinors in flight: direction D + SA is requested, D used
+  template <int D, class R> __device__ __forceinline__ void first(R& r) const {
+    if constexpr (D < SA) {
+      a.in.loadRaw(nbr<D>(), r[D]);
+      first<D + 1>(r);
+    }
+  }
+  template <int D, class R> __device__ __forceinline__ void ahead(cpx<float> (&acc)[12], R& r) const {
+    if constexpr (D < 8) {
+      if constexpr (D + SA < 8) a.in.loadRaw(nbr<D + SA>(), r[(D + SA) % (SA + 1)]);
+      cpx<float> s[12];
+      a.in.unpack(r[D % (SA + 1)], s);
+      compute<D>(acc, s);
+      ahead<D + 1>(acc, r);
+    }
   }
 
   template <int D> __device__ __forceinline__ void compute(cpx<float> (&acc)[12], const cpx<float> (&s)[12]) const {
     constexpr int MU = D >> 1;
     constexpr bool FWD = (D & 1) == 0;
     cpa_wait<NST - 1>();                       // direction D has landed
-    cpx<float> U[6], h[6], u[6];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const float4 v = *slot(D % NB, j);
-      U[2 * j] = {v.x, v.y};
-      U[2 * j + 1] = {v.z, v.w};
-    }
+    cpx<float> U[LB::NU], h[6], u[6];
+    LB::read(slot(D % NB), nt, U);
     issue<D + NST>();                          // refills the buffer of direction D - 1
     constexpr int SF = DAG ? +1 : -1;
     constexpr int SG = FWD ? SF : -SF;
@@ -119,8 +165,8 @@ struct Staged {
 #pragma unroll
       for (int j = 0; j < 6; ++j) h[j] = mk<float>(-h[j].r, -h[j].i);
     }
-    if constexpr (FWD) su3_mul_r12(U, h, u);
-    else su3_dag_mul_r12(U, h, u);
+    if constexpr (FWD) LB::mul(U, h, u);
+    else LB::dag_mul(U, h, u);
     spin_accum<MU, SG, D == 0>(acc, u);        // direction 0 writes acc
   }
 
@@ -132,23 +178,12 @@ struct Staged {
     }
   }
 
-  __device__ __forceinline__ void run(cpx<float> (&acc)[12]) const {
-    prologue<0>();
-    run_after_prologue(acc);
-  }
   __device__ __forceinline__ void run_after_prologue(cpx<float> (&acc)[12]) const {
-    using In = typename std::remove_cv<decltype(a.in)>::type;
-    if constexpr (spin_ahead<In>()) {
-      typename In::Raw r0, r1;
-      a.in.loadRaw(nbr<0>(), r0);
-      step_ahead<0>(acc, r0, r1);
-      step_ahead<1>(acc, r1, r0);
-      step_ahead<2>(acc, r0, r1);
-      step_ahead<3>(acc, r1, r0);
-      step_ahead<4>(acc, r0, r1);
-      step_ahead<5>(acc, r1, r0);
-      step_ahead<6>(acc, r0, r1);
-      step_ahead<7>(acc, r1, r0);
+    if constexpr (SA > 0) {
+      using In = typename std::remove_cv<decltype(a.in)>::type;
+      typename In::Raw r[SA + 1];
+      first<0>(r);
+      ahead<0>(acc, r);
     } else {
       step<0>(acc);
       step<1>(acc);
@@ -162,14 +197,22 @@ struct Staged {
   }
 };
 
-template <bool DAG, bool XPAY, bool NORM, class In, class Out, class Y>
-__global__ void __launch_bounds__(HOP_ST_THREADS, hop_minb<In>()) k_hop_st(HopArgs<In, Out, Y, GF32R12> a) {
+// operands of the Chebyshev step out = ca (v + cmu s - (y + alpha D in)) - cb sp,
+// fused into the last hop of K_hat (FP32): saves the K s vector and a five-vector pass
+struct HopPoly {
+  SpF32 v, s, sp;
+  float ca, cmu, cb;
+};
+
+// EPI 0: out = D in; 1: out = y + alpha D in; 2: the Chebyshev step on that
+template <bool DAG, int EPI, bool NORM, int NST, int SA, int MINB, class In, class Out, class Y, class G>
+__global__ void __launch_bounds__(HOP_ST_THREADS, MINB) k_hop_st(HopArgs<In, Out, Y, G> a, HopPoly pe) {
   extern __shared__ float4 sbuf[];
   pdl_trigger();
   const long site = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool ok = site < a.g.Vh;
   const long cb = ok ? site : 0;               // a thread without a site repeats site 0 and stores nothing
-  Staged<HOP_NST, DAG, HopArgs<In, Out, Y, GF32R12>> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
+  Staged<NST, SA, DAG, HopArgs<In, Out, Y, G>> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
   a.g.coords(cb, a.out_par, S.c);
   S.template prologue<0>();                    // the links do not depend on the kernels before
   pdl_wait();
@@ -179,12 +222,22 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, hop_minb<In>()) k_hop_st(HopAr
   }
   cpx<float> acc[12];
   S.run_after_prologue(acc);
-  if constexpr (XPAY) {
+  if constexpr (EPI >= 1) {
     cpx<float> yv[12];
     a.y.template loadT<false>(cb, yv);
     const float al = (float)a.alpha;
 #pragma unroll
     for (int j = 0; j < 12; ++j) acc[j] = yv[j] + al * acc[j];
+  }
+  if constexpr (EPI == 2) {
+    cpx<float> x[12], q[12];
+    pe.v.template loadT<false>(cb, x);
+    pe.s.template loadT<false>(cb, q);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) acc[j] = x[j] + pe.cmu * q[j] - acc[j];
+    pe.sp.template loadT<false>(cb, q);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) acc[j] = pe.ca * acc[j] - pe.cb * q[j];
   }
   double part[1] = {0.0};
   if constexpr (NORM) { if (ok) part[0] = site_norm2(acc); }
@@ -202,22 +255,74 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, hop_minb<In>()) k_hop_st(HopAr
   }
 }
 
-// Launch of the staged stencil for the context's 12-real FP32 links.
-template <class In, class Out, class Y>
-int hop_staged(wd_ctx* c, int out_par, bool dag, const In& I, const Out& O, const Y& Yv, bool xpay, double alpha,
-               bool norm_cg, bool in_cg) {
+// Resident blocks per SM that the pipeline's depth is chosen for (table at the top):
+// 2, 3, 4 or the full occupancy
+inline int hop_depth(const wd_ctx* c, int full) {
+  const int nb = nblocks(c->g.Vh, HOP_ST_THREADS), n = c->nsm > 0 ? c->nsm : 1;
+  if (nb <= 2 * n) return 2;
+  if (nb <= 3 * n) return 3;
+  return (nb + 4 * n - 1) / (4 * n) <= (nb + full * n - 1) / (full * n) ? 4 : full;
+}
+
+template <bool DAG, int EPI, bool NORM, int NST, int SA, int MINB, class In, class Out, class Y, class G>
+void hop_st_go(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {
+  auto k = k_hop_st<DAG, EPI, NORM, NST, SA, MINB, In, Out, Y, G>;
+  constexpr size_t sm = hop_smem<G>(NST);
+  if constexpr (sm > 47 * 1024) {              // above 48 KB (with the grid sum's) a kernel has to ask, once per device
+    static std::atomic<unsigned long long> asked{0};
+    const unsigned long long bit = 1ull << (c->device & 63);
+    if ((asked.load() & bit) == 0 || c->device >= 64) {
+      (void)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);   // a failure shows at the launch
+      asked.fetch_or(bit);
+    }
+  }
+  pdl_launch(k, nblocks(c->g.Vh, HOP_ST_THREADS), HOP_ST_THREADS, sm, c->stream, a, pe);
+}
+template <bool DAG, int EPI, bool NORM, class In, class Out, class Y, class G>
+void hop_st_depth(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {
+  if constexpr (std::is_same<G, GF32>::value) {
+    // 18 reals: 9 KB a buffer, 55 KB a block at NST = 5
+    if constexpr (std::is_same<In, SpF32>::value) {
+      switch (hop_depth(c, 5)) {
+        case 2: hop_st_go<DAG, EPI, NORM, 5, 5, 2>(c, a, pe); break;
+        case 3: hop_st_go<DAG, EPI, NORM, 4, 3, 3>(c, a, pe); break;
+        case 4: hop_st_go<DAG, EPI, NORM, 4, 2, 4>(c, a, pe); break;
+        default: hop_st_go<DAG, EPI, NORM, 2, 1, 5>(c, a, pe);
+      }
+    } else {
+      if (hop_depth(c, 5) <= 4) hop_st_go<DAG, EPI, NORM, 4, 3, 4>(c, a, pe);
+      else hop_st_go<DAG, EPI, NORM, 2, 1, 5>(c, a, pe);
+    }
+  } else if constexpr (std::is_same<In, SpF32>::value) {
+    switch (hop_depth(c, 5)) {
+      case 2: hop_st_go<DAG, EPI, NORM, 6, 5, 2>(c, a, pe); break;
+      case 3: hop_st_go<DAG, EPI, NORM, 6, 3, 3>(c, a, pe); break;
+      case 4: hop_st_go<DAG, EPI, NORM, 4, 2, 4>(c, a, pe); break;
+      default: hop_st_go<DAG, EPI, NORM, 2, 1, 5>(c, a, pe);
+    }
+  } else {
+    switch (hop_depth(c, 6)) {
+      case 2:
+      case 3: hop_st_go<DAG, EPI, NORM, 6, 4, 3>(c, a, pe); break;
+      case 4: hop_st_go<DAG, EPI, NORM, 4, 3, 4>(c, a, pe); break;
+      default: hop_st_go<DAG, EPI, NORM, 2, 1, 6>(c, a, pe);
+    }
+  }
+}
+
+// Launch of the staged stencil on the links G of the context
+template <class In, class Out, class Y, class G>
+int hop_staged(wd_ctx* c, bool dag, bool xpay, bool norm_cg, const HopArgs<In, Out, Y, G>& a) {
   if (norm_cg && nblocks(c->g.Vh, 64) > RED_MAX_BLOCKS) return fail(WD_ERR_ARG, "lattice too large for one reduction grid");
   if (norm_cg && (dag || !xpay)) return fail(WD_ERR_ARG, "hop: the |out|^2 epilogue exists for M_hat only");
-  CGState* st = (norm_cg || in_cg) ? c->cgs : nullptr;
-  HopArgs<In, Out, Y, GF32R12> a{c->g, out_par, I, O, Yv, GF32R12{c->gauge32r12, c->g.Vh}, alpha, reducer(c), st};
-  const int nb = nblocks(c->g.Vh, HOP_ST_THREADS);
+  const HopPoly pe{};
   if (!dag) {
-    if (!xpay) pdl_launch(k_hop_st<false, false, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
-    else if (!norm_cg) pdl_launch(k_hop_st<false, true, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
-    else pdl_launch(k_hop_st<false, true, true, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
+    if (!xpay) hop_st_depth<false, 0, false>(c, a, pe);
+    else if (!norm_cg) hop_st_depth<false, 1, false>(c, a, pe);
+    else hop_st_depth<false, 1, true>(c, a, pe);
   } else {
-    if (!xpay) pdl_launch(k_hop_st<true, false, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
-    else pdl_launch(k_hop_st<true, true, false, In, Out, Y>, nb, HOP_ST_THREADS, HOP_STAGE_SMEM, c->stream, a);
+    if (!xpay) hop_st_depth<true, 0, false>(c, a, pe);
+    else hop_st_depth<true, 1, false>(c, a, pe);
   }
   WD_CHECK_LAUNCH();
   return WD_OK;
