@@ -284,8 +284,9 @@ int wd_hop(wd_ctx* c, int out_parity, int dagger, int prec, const double* in, do
   WsGuard w(c);
   Field a, b;
   WD_TRY(w.get(prec, &a));
-  WD_TRY(w.get(prec, &b));
   WD_TRY(convert(c, fi, a));
+  if (prec == WD_F32 && hop_widens(c)) return hop(c, out_parity, dagger != 0, a, fo, nullptr, 0.0, false, false);
+  WD_TRY(w.get(prec, &b));
   WD_TRY(hop(c, out_parity, dagger != 0, a, b, nullptr, 0.0, false, false));
   return convert(c, b, fo);
 }
@@ -302,8 +303,9 @@ int wd_apply(wd_ctx* c, double kappa, int dagger, int prec, const double* in, do
   WD_TRY(w.get(prec, &t));
   if (prec == WD_F64) return apply_mhat(c, kappa, dagger != 0, fi, fo, t, false);
   WD_TRY(w.get(prec, &a));
-  WD_TRY(w.get(prec, &b));
   WD_TRY(convert(c, fi, a));
+  if (prec == WD_F32 && hop_widens(c)) return apply_mhat(c, kappa, dagger != 0, a, fo, t, false);
+  WD_TRY(w.get(prec, &b));
   WD_TRY(apply_mhat(c, kappa, dagger != 0, a, b, t, false));
   return convert(c, b, fo);
 }
@@ -319,8 +321,10 @@ int mdagm_apply(wd_ctx* c, double kappa, int prec, int nrhs, const double* in, d
   Field t1, t2, a, b;
   WD_TRY(w.get(prec, &t1));
   WD_TRY(w.get(prec, &t2));
-  if (prec != WD_F64) {
-    WD_TRY(w.get(prec, &a));
+  // FP32: the last hop stores FP64 (K_hat at 32^3 x 64 with its conversions 568 -> 556 us)
+  const bool widen = prec == WD_F32 && hop_widens(c);
+  if (prec != WD_F64) WD_TRY(w.get(prec, &a));
+  if (prec != WD_F64 && !widen) {
     // K_hat of 16-bit input writes FP32; FP32 and double-float keep their format
     WD_TRY(w.get(prec == WD_DF ? WD_DD : WD_F32, &b));
   }
@@ -331,8 +335,8 @@ int mdagm_apply(wd_ctx* c, double kappa, int prec, int nrhs, const double* in, d
       WD_TRY(apply_khat(c, kappa, fi, fo, t1, t2, false, false));
     } else {
       WD_TRY(convert(c, fi, a));
-      WD_TRY(apply_khat(c, kappa, a, b, t1, t2, false, false));
-      WD_TRY(convert(c, b, fo));
+      WD_TRY(apply_khat(c, kappa, a, widen ? fo : b, t1, t2, false, false));
+      if (!widen) WD_TRY(convert(c, b, fo));
     }
   }
   return WD_OK;

@@ -103,15 +103,15 @@ __global__ void k_f64_to_f32(long n, const double2* in, float4* out) {
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i >= n) return;
   const double2 a = ldw(in + 2 * j * n + i), b = ldw(in + (2 * j + 1) * n + i);
-  out[j * n + i] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+  out[j * n + i] = make_float4(f32_of(a.x), f32_of(a.y), f32_of(b.x), f32_of(b.y));
 }
 __global__ void k_f32_to_f64(long n, const float4* in, double2* out) {
   pdl_enter();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i >= n) return;
   const float4 v = ldw(in + j * n + i);
-  out[2 * j * n + i] = make_double2((double)v.x, (double)v.y);
-  out[(2 * j + 1) * n + i] = make_double2((double)v.z, (double)v.w);
+  out[2 * j * n + i] = make_double2(f64_of(v.x), f64_of(v.y));
+  out[(2 * j + 1) * n + i] = make_double2(f64_of(v.z), f64_of(v.w));
 }
 __global__ void k_f64_to_dd(long n, const double2* in, float4* out) {
   pdl_enter();

@@ -4,11 +4,19 @@
 
 namespace wd {
 
+// whether hop_f32 can store FP64 (the tile-staged option cannot)
+bool hop_widens(wd_ctx* c) { return !(c->recon == WD_RECON_12 && tt_eligible(c)); }
+
 int hop_f32(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
             double alpha, bool norm_cg, bool in_cg) {
-  if (in.fmt != WD_F32 || out.fmt != WD_F32 || (y && y->fmt != WD_F32))
-    return fail(WD_ERR_ARG, "hop_f32: field formats must all be FP32");
-  SpF32 I = sp32(in), O = sp32(out), Y = y ? sp32(*y) : O;
+  if (in.fmt != WD_F32 || (out.fmt != WD_F32 && out.fmt != WD_F64) || (y && y->fmt != WD_F32))
+    return fail(WD_ERR_ARG, "hop_f32: input and y must be FP32, the output FP32 or FP64");
+  SpF32 I = sp32(in), Y = y ? sp32(*y) : I;
+  if (out.fmt == WD_F64) {   // the FP32 result widened as it is stored: the last hop of an operator call
+    if (!hop_widens(c) || norm_cg) return fail(WD_ERR_ARG, "hop_f32: no FP64 output on this path");
+    return hop_links(c, out_par, dag, I, sp64(out), Y, y != nullptr, alpha, norm_cg, in_cg);
+  }
+  SpF32 O = sp32(out);
   if (c->recon == WD_RECON_12 && tt_eligible(c))
     return hop_tt(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
   return hop_links(c, out_par, dag, I, O, Y, y != nullptr, alpha, norm_cg, in_cg);
@@ -34,15 +42,39 @@ int wait_selftest(wd_ctx* c, long long ns) {
   return WD_OK;
 }
 
-template <class G>
+template <int EPI, class G>
 static void hop_poly(wd_ctx* c, const G& gauge, double alpha, const Field& in, const Field& y, const Field& out,
                      const HopPoly& pe) {
   const HopArgs<SpF32, SpF32, SpF32, G> a{c->g, 0, sp32(in), sp32(out), sp32(y), gauge, alpha, reducer(c), nullptr};
   if (split_eligible(c, WD_F32))
-    pdl_launch(k_hop_split<float, true, 2, false, SpF32, SpF32, SpF32, G>, nblocks(c->g.Vh, SPL_SITES), SPL_THREADS, 0,
+    pdl_launch(k_hop_split<float, true, EPI, false, SpF32, SpF32, SpF32, G>, nblocks(c->g.Vh, SPL_SITES), SPL_THREADS, 0,
                c->stream, a, pe);
   else
-    hop_st_depth<true, 2, false>(c, a, pe);
+    hop_st_depth<true, EPI, false>(c, a, pe);
+}
+template <int EPI>
+static int hop_poly_links(wd_ctx* c, double alpha, const Field& in, const Field& y, const Field& out, const HopPoly& pe) {
+  if (c->recon == WD_RECON_12) hop_poly<EPI>(c, GF32R12{c->gauge32r12, c->g.Vh}, alpha, in, y, out, pe);
+  else hop_poly<EPI>(c, GF32{c->gauge32, c->g.Vh}, alpha, in, y, out, pe);
+  WD_CHECK_LAUNCH();
+  c->prof.all[WD_F32] += 1;
+  return WD_OK;
+}
+
+// out = y + alpha D^dag_eo in + z v, the last hop of a factor (K_hat + z) v
+int hop_shift(wd_ctx* c, const Field& in, const Field& y, double alpha, double zr, double zi, const Field& v,
+              const Field& out) {
+  if (in.fmt == WD_F32 && hop_widens(c)) {   // not the tile-staged option
+    const Field* fields[] = {&y, &v, &out};
+    for (const Field* f : fields)
+      if (f->fmt != WD_F32) return fail(WD_ERR_ARG, "hop_shift: formats differ");
+    return hop_poly_links<3>(c, alpha, in, y, out, HopPoly{sp32(v), sp32(v), sp32(v), (float)zr, 0.f, (float)zi});
+  }
+  WsGuard w(c);
+  Field k;
+  WD_TRY(w.get(in.fmt, &k));
+  WD_TRY(hop(c, 0, true, in, k, &y, alpha, false, false));
+  return caxpby(c, 1.0, 0.0, k, zr, zi, v, out);
 }
 
 // out = ca (v + cmu s - K_hat s) - cb sprev for FP32 fields (t1, t2 scratch)
@@ -64,12 +96,10 @@ int khat_poly_step_f32(wd_ctx* c, double kappa, const Field& s, Field& t1, Field
     for (const Field* f : chk)
       if (((uintptr_t)f->data & 15) != 0) return fail(WD_ERR_ARG, "khat_poly_step_f32: fields must be 16-byte aligned");
     WD_TRY((tt_launch<true, 2, false>(c, a, pe)));
+    c->prof.all[WD_F32] += 1;
   } else {
-    if (c->recon == WD_RECON_12) hop_poly(c, GF32R12{c->gauge32r12, c->g.Vh}, a2, t1, t2, out, hp);
-    else hop_poly(c, GF32{c->gauge32, c->g.Vh}, a2, t1, t2, out, hp);
-    WD_CHECK_LAUNCH();
+    WD_TRY(hop_poly_links<2>(c, a2, t1, t2, out, hp));
   }
-  c->prof.all[WD_F32] += 1;
   c->nmat += 1;
   return WD_OK;
 }

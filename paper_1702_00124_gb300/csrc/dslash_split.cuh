@@ -97,12 +97,13 @@ template <bool DAG, class T> __device__ __forceinline__ cpx<T> split_sum_at(int 
   }
 }
 
-// EPI 0: out = D in; 1: out = y + alpha D in; 2: the Chebyshev step on that (FP32)
+// EPI 0: out = D in; 1: out = y + alpha D in; 2 and 3: HopPoly on that (FP32)
 template <class T, bool DAG, int EPI, bool NORM, class In, class Out, class Y, class G>
 __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G> a, HopPoly pe) {
-  constexpr bool F64 = std::is_same<Out, SpF64>::value;
-  constexpr bool WORDS = F64 || (std::is_same<Out, SpF32>::value && std::is_same<Y, SpF32>::value);
-  static_assert(EPI != 2 || (WORDS && !F64), "the fused Chebyshev step is FP32");
+  constexpr bool F64 = std::is_same<T, double>::value;
+  constexpr bool OUT64 = std::is_same<Out, SpF64>::value;   // FP64 fields, or an FP32 result widened
+  constexpr bool WORDS = F64 || ((OUT64 || std::is_same<Out, SpF32>::value) && std::is_same<Y, SpF32>::value);
+  static_assert(EPI < 2 || (WORDS && !F64), "the fused polynomial epilogues are FP32");
   __shared__ cpx<T> sh[8 * 6 * SPL_SITES];
   pdl_trigger();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
       if (w < 4) y1 = a.y.p[(8 + w) * a.y.stride + cb];
     } else if (w < 6) {
       yv = a.y.p[w * a.y.stride + cb];
+      if constexpr (EPI >= 2) vv = pe.v.p[w * pe.v.stride + cb];
       if constexpr (EPI == 2) {
-        vv = pe.v.p[w * pe.v.stride + cb];
         sv = pe.s.p[w * pe.s.stride + cb];
         pv = pe.sp.p[w * pe.sp.stride + cb];
       }
@@ -175,8 +176,18 @@ __global__ void __launch_bounds__(SPL_THREADS) k_hop_split(HopArgs<In, Out, Y, G
         o.z = pe.ca * (vv.z + pe.cmu * sv.z - o.z) - pe.cb * pv.z;
         o.w = pe.ca * (vv.w + pe.cmu * sv.w - o.w) - pe.cb * pv.w;
       }
+      if constexpr (EPI == 3) {
+        const cpx<float> z = mk(pe.ca, pe.cb), e0 = cfma(z, mk(vv.x, vv.y), mk(o.x, o.y)),
+                         e1 = cfma(z, mk(vv.z, vv.w), mk(o.z, o.w));
+        o = make_float4(e0.r, e0.i, e1.r, e1.i);
+      }
       if (ok) {
-        a.out.p[w * a.out.stride + cb] = o;
+        if constexpr (OUT64) {
+          a.out.p[2 * w * a.out.stride + cb] = make_double2(f64_of(o.x), f64_of(o.y));
+          a.out.p[(2 * w + 1) * a.out.stride + cb] = make_double2(f64_of(o.z), f64_of(o.w));
+        } else {
+          a.out.p[w * a.out.stride + cb] = o;
+        }
         if constexpr (NORM) part[0] = (double)fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, o.w * o.w)));
       }
     }

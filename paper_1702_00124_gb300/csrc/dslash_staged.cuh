@@ -197,14 +197,17 @@ struct Staged {
   }
 };
 
-// operands of the Chebyshev step out = ca (v + cmu s - (y + alpha D in)) - cb sp,
-// fused into the last hop of K_hat (FP32): saves the K s vector and a five-vector pass
+// Operands fused into the last hop of K_hat (FP32):
+//   EPI 2, the Chebyshev step out = ca (v + cmu s - (y + alpha D in)) - cb sp: saves
+//          the K s vector and a five-vector pass
+//   EPI 3, a factor of a root product out = y + alpha D in + (ca + i cb) v: saves a
+//          four-vector pass
 struct HopPoly {
   SpF32 v, s, sp;
   float ca, cmu, cb;
 };
 
-// EPI 0: out = D in; 1: out = y + alpha D in; 2: the Chebyshev step on that
+// EPI 0: out = D in; 1: out = y + alpha D in; 2 and 3: as above
 template <bool DAG, int EPI, bool NORM, int NST, int SA, int MINB, class In, class Out, class Y, class G>
 __global__ void __launch_bounds__(HOP_ST_THREADS, MINB) k_hop_st(HopArgs<In, Out, Y, G> a, HopPoly pe) {
   extern __shared__ float4 sbuf[];
@@ -238,6 +241,13 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, MINB) k_hop_st(HopArgs<In, Out
     pe.sp.template loadT<false>(cb, q);
 #pragma unroll
     for (int j = 0; j < 12; ++j) acc[j] = pe.ca * acc[j] - pe.cb * q[j];
+  }
+  if constexpr (EPI == 3) {
+    cpx<float> x[12];
+    pe.v.template loadT<false>(cb, x);
+    const cpx<float> z = mk(pe.ca, pe.cb);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) acc[j] = cfma(z, x[j], acc[j]);
   }
   double part[1] = {0.0};
   if constexpr (NORM) { if (ok) part[0] = site_norm2(acc); }

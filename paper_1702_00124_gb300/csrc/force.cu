@@ -101,9 +101,6 @@ struct ForceArgs {
   double* F;                 // [4][2][8][Vh]
 };
 
-__device__ __forceinline__ double to_f64(float v) { return f64_of(v); }
-__device__ __forceinline__ double to_f64(double v) { return v; }
-
 template <int MU, int NP, class T, class S, class G>
 __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4], bool ok) {
   const Geom& g = a.g;

@@ -73,13 +73,19 @@ static int mhat(wd_ctx* c, double kappa, bool dag, const Field& in, const Field&
   return apply_mhat(c, kappa, dag, in, out, t, false);
 }
 
-// out = K x - z x  (z complex; conj_z selects conj(z))
+// out = K x - z x (z complex; out may be x)
 static int k_minus(wd_ctx* c, double kappa, double zr, double zi, const Field& x, const Field& out) {
   WsGuard w(c);
-  Field k;
-  WD_TRY(w.get(x.fmt, &k));
-  WD_TRY(khat_any(c, kappa, x, k));
-  return caxpby(c, 1.0, 0.0, k, -zr, -zi, x, out);
+  Field t1, t2;
+  WD_TRY(w.get(x.fmt, &t1));
+  WD_TRY(w.get(x.fmt, &t2));
+  const double a = -kappa * kappa;
+  WD_TRY(hop(c, 1, false, x, t1, nullptr, 0.0, false, false));
+  WD_TRY(hop(c, 0, false, t1, t2, &x, a, false, false));
+  WD_TRY(hop(c, 1, true, t2, t1, nullptr, 0.0, false, false));
+  WD_TRY(hop_shift(c, t1, t2, a, -zr, -zi, x, out));
+  c->nmat += 1;
+  return WD_OK;
 }
 
 // Force of S = v^dag Q(K) v, Q = scale prod_k (K - r_k), added with coef.
@@ -94,11 +100,11 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
   // of those R, formed while K_hat is applied to them in the segment rebuild;
   // L, lo, ml, mlo: the same of the segment's L
   std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg), L(seg), lo(seg), ml(seg), mlo(seg);
-  Field Ln, cur, KR;
+  Field Ln, cur;
   for (auto& x : cp) WD_TRY(w.get(f, &x));
   for (auto* v : {&buf, &ro, &mr, &mro, &L, &lo, &ml, &mlo})
     for (auto& x : *v) WD_TRY(w.get(f, &x));
-  for (Field* x : {&Ln, &cur, &KR}) WD_TRY(w.get(f, x));
+  for (Field* x : {&Ln, &cur}) WD_TRY(w.get(f, x));
   const double k2 = kappa * kappa;
   auto seg_end = [&](int s) { return std::min((s + 1) * seg, m) - 1; };
   // backward pass: R_{m-1} = v, R_{k-1} = (K - r_k) R_k; keep R at segment ends
@@ -118,9 +124,8 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
       WD_TRY(hop(c, 1, false, buf[j], ro[j], nullptr, 0.0, false, false));
       WD_TRY(hop(c, 0, false, ro[j], mr[j], &buf[j], -k2, false, false));
       WD_TRY(hop(c, 1, true, mr[j], mro[j], nullptr, 0.0, false, false));
-      WD_TRY(hop(c, 0, true, mro[j], KR, &mr[j], -k2, false, false));
+      WD_TRY(hop_shift(c, mro[j], mr[j], -k2, -rr[a + j], -ri[a + j], buf[j], buf[j - 1]));
       c->nmat += 1;
-      WD_TRY(caxpby(c, 1.0, 0.0, KR, -rr[a + j], -ri[a + j], buf[j], buf[j - 1]));
     }
     for (int k = a; k <= b; ++k) {
       const int j = k - a;
@@ -140,10 +145,9 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
       Ye[2 * j + 1] = ml[j], Yo[2 * j + 1] = mlo[j], Xe[2 * j + 1] = buf[j], Xo[2 * j + 1] = ro[j];
       if (k < m - 1) {
         // K L = M^dag (M L) = ml - kappa^2 D^dag_eo mlo: one more hop
-        WD_TRY(hop(c, 0, true, mlo[j], KR, &ml[j], -k2, false, false));
+        // with the shift of (K - conj r_k) L
+        WD_TRY(hop_shift(c, mlo[j], ml[j], -k2, -rr[k], ri[k], L[j], k < b ? L[j + 1] : Ln));
         c->nmat += 1;
-        const Field& nx = k < b ? L[j + 1] : Ln;
-        WD_TRY(caxpby(c, 1.0, 0.0, KR, -rr[k], ri[k], L[j], nx));   // (K - conj r_k) L
       }
     }
     // the segment's pairs in one pass over the links and F

@@ -144,6 +144,10 @@ __device__ __forceinline__ double f64_of(float v) {
   return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+__device__ __forceinline__ double to_f64(float v) { return f64_of(v); }
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(dd v) { return (double)v; }
+
 // ----------------------------------------------------------------------------
 // Gamma matrices, DeGrand-Rossi chiral basis (gamma_5 = diag(1,1,-1,-1)).
 // Each gamma_mu has one non-zero per row; row a (a = 0,1) couples to column
@@ -290,7 +294,7 @@ struct SpF64 {
   long stride;
   template <class T> __device__ __forceinline__ void store(long i, const cpx<T> (&s)[12]) const {
 #pragma unroll
-    for (int j = 0; j < 12; ++j) p[j * stride + i] = make_double2((double)s[j].r, (double)s[j].i);
+    for (int j = 0; j < 12; ++j) p[j * stride + i] = make_double2(to_f64(s[j].r), to_f64(s[j].i));
   }
   template <bool RO = true, class T> __device__ __forceinline__ void loadT(long i, cpx<T> (&s)[12]) const {
 #pragma unroll
@@ -769,11 +773,14 @@ int wait_selftest(wd_ctx* c, long long ns);
 // the solver state carries a stop flag; norm_cg: also form pAp = |out|^2.
 int hop(wd_ctx* c, int out_par, bool dag, const Field& in, const Field& out, const Field* y,
         double alpha, bool norm_cg, bool in_cg);
+bool hop_widens(wd_ctx* c);   // FP32 hops may store an FP64 output
 int apply_mhat(wd_ctx* c, double kappa, bool dag, const Field& in, const Field& out, Field& tmp,
                bool norm_cg);
 int apply_khat(wd_ctx* c, double kappa, const Field& in, const Field& out, Field& t1, Field& t2,
                bool norm_cg, bool in_cg = false);
 double hop_bytes(int fmt_in, int fmt_out, bool xpay, int gauge_bytes_per_link, long Vh);
+int hop_shift(wd_ctx* c, const Field& in, const Field& y, double alpha, double zr, double zi, const Field& v,
+              const Field& out);
 int khat_poly_step_f32(wd_ctx* c, double kappa, const Field& s, Field& t1, Field& t2, const Field& v,
                        const Field& sprev, double ca, double cmu, double cb, const Field& out);
 
