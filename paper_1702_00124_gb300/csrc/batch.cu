@@ -500,6 +500,65 @@ __global__ void k_slot(long Vh, int nr, int r, float4* il, double2* f64, int dir
   }
 }
 
+// Word by word (blockIdx.y or a stride loop over the six FP32 words of a site), one
+// system: the start of a solve and the two ends of a reliable update.  Their sums go to
+// the batch's pinned array, so that the host waits once for all systems of a pass.
+
+// r = p = b, increment = 0, |b|^2
+__global__ void __launch_bounds__(256) k_sys_start(long Vh, int nr, int rs, const double2* b, float4* R, float4* P,
+                                                   float4* X, Reduce red) {
+  double v[1] = {0.0};
+  for (long k = (long)blockIdx.x * 256 + threadIdx.x; k < 6 * Vh; k += (long)gridDim.x * 256) {
+    const long j = k / Vh, i = k - j * Vh, e = (j * Vh + i) * nr + rs;
+    const double2 c0 = __ldg(b + 2 * j * Vh + i), c1 = __ldg(b + (2 * j + 1) * Vh + i);
+    const float4 w = make_float4(f32_of(c0.x), f32_of(c0.y), f32_of(c1.x), f32_of(c1.y));
+    R[e] = w;
+    P[e] = w;
+    X[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = fma(c0.y, c0.y, fma(c0.x, c0.x, v[0]));
+    v[0] = fma(c1.y, c1.y, fma(c1.x, c1.x, v[0]));
+  }
+  grid_sum_hl<1>(red, v);
+}
+// x += increment, increment = 0; xd (or null) = x in double-float
+__global__ void __launch_bounds__(256) k_sys_fold(long Vh, int nr, int rs, float4* X, double2* x, float4* xd) {
+  const long i = (long)blockIdx.x * 256 + threadIdx.x, j = blockIdx.y;
+  if (i >= Vh) return;
+  const long e = (j * Vh + i) * nr + rs, c0 = 2 * j * Vh + i, c1 = c0 + Vh;
+  const float4 w = X[e];
+  double2 a = x[c0], b = x[c1];
+  a = make_double2(a.x + f64_of(w.x), a.y + f64_of(w.y));
+  b = make_double2(b.x + f64_of(w.z), b.y + f64_of(w.w));
+  X[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  x[c0] = a;
+  x[c1] = b;
+  if (xd != nullptr) {
+    const dd ar(a.x), ai(a.y), br(b.x), bi(b.y);
+    xd[c0] = make_float4(ar.hi, ar.lo, ai.hi, ai.lo);
+    xd[c1] = make_float4(br.hi, br.lo, bi.hi, bi.lo);
+  }
+}
+// r = b - A x in FP64, stored in FP32, and |r|^2; A x FP64 or double-float
+template <class W>
+__global__ void __launch_bounds__(256) k_sys_resid(long Vh, int nr, int rs, const double2* b, const W* ax, float4* R,
+                                                   Reduce red) {
+  double v[1] = {0.0};
+  auto get = [](const W& w) -> double2 {
+    if constexpr (std::is_same<W, float4>::value) return make_double2((double)dd(w.x, w.y), (double)dd(w.z, w.w));
+    else return w;
+  };
+  for (long k = (long)blockIdx.x * 256 + threadIdx.x; k < 6 * Vh; k += (long)gridDim.x * 256) {
+    const long j = k / Vh, i = k - j * Vh, c0 = 2 * j * Vh + i, c1 = c0 + Vh;
+    const double2 b0 = __ldg(b + c0), b1 = __ldg(b + c1), a0 = get(ax[c0]), a1 = get(ax[c1]);
+    const double2 r0 = make_double2(b0.x - a0.x, b0.y - a0.y), r1 = make_double2(b1.x - a1.x, b1.y - a1.y);
+    R[(j * Vh + i) * nr + rs] = make_float4(f32_of(r0.x), f32_of(r0.y), f32_of(r1.x), f32_of(r1.y));
+    v[0] = fma(r0.y, r0.y, fma(r0.x, r0.x, v[0]));
+    v[0] = fma(r1.y, r1.y, fma(r1.x, r1.x, v[0]));
+  }
+  grid_sum_hl<1>(red, v);
+}
+inline int sys_blocks(long Vh) { return (int)std::min<long>(8 * 152, (6 * Vh + 255) / 256); }
+
 // p_s = r_s + beta p_s for one system
 __global__ void k_slot_pupdate(long Vh, int nr, int r, float4* p, const float4* rr, float beta) {
   const long cb = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -532,6 +591,7 @@ struct wd_batch {
   double* partial = nullptr;
   CGState* st_d = nullptr;
   CGState* st_h = nullptr;       // pinned
+  double* sum_h = nullptr;       // pinned, two doubles per system: |b|^2 or |r|^2 as hi + lo
   cudaStream_t stream = nullptr; // capture-capable stream
   bool own_stream = false;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
@@ -811,6 +871,7 @@ int wd_batch_create(wd_ctx* const* ctxs, int nlat, const double* kappas, const i
   cudaError_t e = cudaMalloc(&b->lat_d, sizeof(BLat) * nlat);
   if (e == cudaSuccess) e = cudaMalloc(&b->st_d, sizeof(CGState) * b->S);
   if (e == cudaSuccess) e = cudaMallocHost(&b->st_h, sizeof(CGState) * b->S);
+  if (e == cudaSuccess) e = cudaMallocHost(&b->sum_h, sizeof(double) * 2 * b->S);
   if (e == cudaSuccess) e = cudaMemset(b->st_d, 0, sizeof(CGState) * b->S);
   if (e == cudaSuccess) e = cudaMalloc(&b->gbar, sizeof(GridBar));
   if (e == cudaSuccess) e = cudaMalloc(&b->kerr, sizeof(unsigned));
@@ -843,6 +904,7 @@ int wd_batch_destroy(wd_batch* b) {
   cudaFree(b->gbar);
   cudaFree(b->kerr);
   if (b->st_h) cudaFreeHost(b->st_h);
+  if (b->sum_h) cudaFreeHost(b->sum_h);
   if (b->own_stream) {
     cudaStreamDestroy(b->stream);
     cudaEventDestroy(b->ev_in);
@@ -889,14 +951,16 @@ int wd_batch_cg(wd_batch* b, const double* const* bvec, double* const* x, const 
     nmat0[l] = c->nmat;
     for (int r = 0; r < L.nr; ++r) {
       const long off = (long)r * 24 * L.g.Vh;
-      Field bf = wrap_f64(c, bvec[l] + off), xf = wrap_f64(c, x[l] + off);
-      WD_TRY(zero(c, xf));
-      WD_TRY(norm2(c, bf, &bb[L.sys0 + r]));
-      WD_TRY(b_slot(b, l, r, BF_R, const_cast<double*>(bvec[l]) + off, 1));
-      WD_TRY(b_slot(b, l, r, BF_P, const_cast<double*>(bvec[l]) + off, 1));
-      WD_TRY(b_slot(b, l, r, BF_X, nullptr, 2));
+      WD_CUDA(cudaMemsetAsync(x[l] + off, 0, sizeof(double) * 24 * L.g.Vh, b->stream));
+      k_sys_start<<<sys_blocks(L.g.Vh), 256, 0, b->stream>>>(
+          L.g.Vh, L.nr, r, (const double2*)(bvec[l] + off), L.f[BF_R], L.f[BF_P], L.f[BF_X],
+          Reduce{c->red_partial, c->red_counter, b->sum_h + 2 * (L.sys0 + r)});
+      b->launches += 1;
     }
   }
+  WD_CUDA(cudaGetLastError());
+  WD_CUDA(cudaStreamSynchronize(b->stream));
+  for (int s = 0; s < b->S; ++s) bb[s] = b->sum_h[2 * s];
   for (int s = 0; s < b->S; ++s) {
     CGState& S = b->st_h[s];
     S = CGState{};
@@ -955,67 +1019,70 @@ int wd_batch_cg(wd_batch* b, const double* const* bvec, double* const* x, const 
       WD_TRY(b_leave(b));
       return fail(WD_ERR_TIMEOUT, "wd_batch_cg: a grid-barrier wait of the persistent kernel expired");
     }
+    // reliable updates of the systems that stopped, in FP64 on their own lattices: every
+    // system's kernels are queued before the host waits once for all the sums
     bool all_done = true, changed = false;
+    std::vector<std::pair<int, int>> upd;   // (lattice, rhs)
+    if (b->own_stream) {   // the contexts' stream works on what the batch stream produced
+      WD_CUDA(cudaEventRecord(b->ev_out, b->stream));
+      WD_CUDA(cudaStreamWaitEvent(b->ctx[0]->stream, b->ev_out, 0));
+    }
     for (int l = 0; l < nlat && status == WD_OK; ++l) {
       const BLat& L = b->lat_h[l];
       wd_ctx* c = b->ctx[l];
       for (int r = 0; r < L.nr; ++r) {
         const int sidx = L.sys0 + r;
-        CGState& S = b->st_h[sidx];
+        const CGState& S = b->st_h[sidx];
         if (S.flag == FLAG_DONE) continue;
         if (S.flag & FLAG_NAN) { status = fail(WD_ERR_NAN, "wd_batch_cg: non-finite value"); break; }
         if (S.flag == 0) { all_done = false; continue; }
-        // reliable update of this system in FP64 on its own lattice
-        const long off = (long)r * 24 * L.g.Vh;
-        Field xf = wrap_f64(c, x[l] + off), bf = wrap_f64(c, bvec[l] + off);
+        const long Vh = L.g.Vh, off = (long)r * 24 * Vh;
+        Field xf = wrap_f64(c, x[l] + off);
+        // K_hat x in double-float when the lattice's context selects it (as the
+        // single-system solver's true residual): FP64-class accuracy on the FP32
+        // pipes, b, x, r and the norm stay FP64
+        const bool df = c->resid_dd && c->gauge_dd;
         WsGuard w(c);
-        Field t, rr, t1, t2;
-        WD_TRY(w.get(WD_F64, &t));
-        WD_TRY(w.get(WD_F64, &rr));
-        WD_TRY(w.get(WD_F64, &t1));
-        WD_TRY(w.get(WD_F64, &t2));
-        WD_TRY(b_slot(b, l, r, BF_X, (double*)t.data, 0));
-        WD_TRY(b_slot(b, l, r, BF_X, nullptr, 2));
-        if (b->own_stream) {   // the context stream works on what the batch stream produced
-          WD_CUDA(cudaEventRecord(b->ev_out, b->stream));
-          WD_CUDA(cudaStreamWaitEvent(c->stream, b->ev_out, 0));
-        }
-        WD_TRY(axpby(c, 1.0, xf, 1.0, t, xf));
-        if (c->resid_dd && c->gauge_dd) {
-          // K_hat x in double-float when the lattice's context selects it (as
-          // the single-system solver's true residual): FP64-class accuracy on
-          // the FP32 pipes, b, x, r and the norm stay FP64
-          Field xd, td, d1, d2;
-          WD_TRY(w.get(WD_DD, &xd));
-          WD_TRY(w.get(WD_DD, &td));
-          WD_TRY(w.get(WD_DD, &d1));
-          WD_TRY(w.get(WD_DD, &d2));
-          WD_TRY(convert(c, xf, xd));
-          WD_TRY(apply_khat(c, L.kappa, xd, td, d1, d2, false, false));
-          WD_TRY(convert(c, td, t));
-        } else {
-          WD_TRY(apply_khat(c, L.kappa, xf, t, t1, t2, false, false));
-        }
-        WD_TRY(axpby(c, 1.0, bf, -1.0, t, rr));
-        double rr2;
-        WD_TRY(norm2(c, rr, &rr2));
-        info[sidx].reliable_updates += 1;
-        info[sidx].iters = S.iter;
-        info[sidx].true_rel_resid = std::sqrt(rr2 / bb[sidx]);
-        changed = true;
-        if (!std::isfinite(rr2)) { status = fail(WD_ERR_NAN, "wd_batch_cg: non-finite residual"); break; }
-        if (rr2 <= S.stop_rr) { S.flag = FLAG_DONE; continue; }
-        if (S.flag & FLAG_MAXITER) { status = fail(WD_ERR_NOCONV, "wd_batch_cg: maxiter reached"); break; }
-        all_done = false;
-        WD_TRY(b_slot(b, l, r, BF_R, (double*)rr.data, 1));
-        const double beta = rr2 / S.rr_old;
-        k_slot_pupdate<<<nblocks(L.g.Vh, 128), 128, 0, b->stream>>>(L.g.Vh, L.nr, r, L.f[BF_P], L.f[BF_R],
-                                                                    (float)beta);
-        b->launches += 1;
-        S.rr = rr2;
-        S.upd_rr = std::max(delta * delta * rr2, S.stop_rr);
-        S.flag = 0;
+        Field xd, t, t1, t2;
+        WD_TRY(w.get(df ? WD_DD : WD_F64, &t));
+        WD_TRY(w.get(df ? WD_DD : WD_F64, &t1));
+        WD_TRY(w.get(df ? WD_DD : WD_F64, &t2));
+        if (df) WD_TRY(w.get(WD_DD, &xd));
+        k_sys_fold<<<dim3(nblocks(Vh, 256), 6), 256, 0, c->stream>>>(Vh, L.nr, r, L.f[BF_X], (double2*)xf.data,
+                                                                     df ? (float4*)xd.data : nullptr);
+        WD_TRY(apply_khat(c, L.kappa, df ? xd : xf, t, t1, t2, false, false));
+        const Reduce red{c->red_partial, c->red_counter, b->sum_h + 2 * sidx};
+        if (df)
+          k_sys_resid<<<sys_blocks(Vh), 256, 0, c->stream>>>(Vh, L.nr, r, (const double2*)(bvec[l] + off),
+                                                             (const float4*)t.data, L.f[BF_R], red);
+        else
+          k_sys_resid<<<sys_blocks(Vh), 256, 0, c->stream>>>(Vh, L.nr, r, (const double2*)(bvec[l] + off),
+                                                             (const double2*)t.data, L.f[BF_R], red);
+        b->launches += 2;
+        WD_CUDA(cudaGetLastError());
+        upd.push_back({l, r});
       }
+    }
+    if (!upd.empty()) WD_CUDA(cudaStreamSynchronize(b->ctx[0]->stream));
+    for (size_t k = 0; k < upd.size(); ++k) {
+      const BLat& L = b->lat_h[upd[k].first];
+      const int r = upd[k].second, sidx = L.sys0 + r;
+      CGState& S = b->st_h[sidx];
+      const double rr2 = b->sum_h[2 * sidx];
+      info[sidx].reliable_updates += 1;
+      info[sidx].iters = S.iter;
+      info[sidx].true_rel_resid = std::sqrt(rr2 / bb[sidx]);
+      changed = true;
+      if (!std::isfinite(rr2)) { status = fail(WD_ERR_NAN, "wd_batch_cg: non-finite residual"); break; }
+      if (rr2 <= S.stop_rr) { S.flag = FLAG_DONE; continue; }
+      if (S.flag & FLAG_MAXITER) { status = fail(WD_ERR_NOCONV, "wd_batch_cg: maxiter reached"); break; }
+      all_done = false;
+      const double beta = rr2 / S.rr_old;
+      k_slot_pupdate<<<nblocks(L.g.Vh, 128), 128, 0, b->stream>>>(L.g.Vh, L.nr, r, L.f[BF_P], L.f[BF_R], (float)beta);
+      b->launches += 1;
+      S.rr = rr2;
+      S.upd_rr = std::max(delta * delta * rr2, S.stop_rr);
+      S.flag = 0;
     }
     if (status != WD_OK) break;
     if (changed) WD_CUDA(cudaMemcpyAsync(b->st_d, b->st_h, sizeof(CGState) * b->S, cudaMemcpyHostToDevice, b->stream));
