@@ -90,7 +90,7 @@ __device__ __forceinline__ void outer_acc(cpx<T> (&A)[9], const cpx<T> (&h)[6], 
 // Measured at 16^3 x 32 (FP32): the kernel before it (one thread per site, two products
 // per pair, F updated for every pair of pairs) 94 us per root, 16 roots 1.51 ms; the
 // whole polynomial force of degree 16 3.02 -> 2.39 ms.
-constexpr int F_MAXP = 16;   // pairs per launch
+constexpr int F_MAXP = 2 * FORCE_ROOTS;   // pairs per launch
 template <class S, class G>
 struct ForceArgs {
   Geom g;

@@ -98,13 +98,24 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
   WsGuard w(c);
   // buf: the R of one segment; ro / mr / mro: D_oe R, M_hat R and D^dag_oe M_hat R
   // of those R, formed while K_hat is applied to them in the segment rebuild;
-  // L, lo, ml, mlo: the same of the segment's L
+  // L, lo, ml, mlo: the same of a group of up to nl of its L, whose outer products
+  // go out in one launch.  Where memory is short the group shrinks, down to one root
+  // (nseg + 4 seg + 6 vectors in all, one launch per root)
   std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg), L(seg), lo(seg), ml(seg), mlo(seg);
   Field Ln, cur;
   for (auto& x : cp) WD_TRY(w.get(f, &x));
-  for (auto* v : {&buf, &ro, &mr, &mro, &L, &lo, &ml, &mlo})
+  for (auto* v : {&buf, &ro, &mr, &mro})
     for (auto& x : *v) WD_TRY(w.get(f, &x));
-  for (Field* x : {&Ln, &cur}) WD_TRY(w.get(f, x));
+  for (Field* x : {&Ln, &cur, &L[0], &lo[0], &ml[0], &mlo[0]}) WD_TRY(w.get(f, x));
+  int nl = 1;
+  for (; nl < std::min(seg, FORCE_ROOTS); ++nl) {
+    bool ok = true;
+    for (Field* x : {&L[nl], &lo[nl], &ml[nl], &mlo[nl]}) ok = ok && w.get(f, x) == WD_OK;
+    if (!ok) {
+      cudaGetLastError();                      // out of memory: handled here
+      break;
+    }
+  }
   const double k2 = kappa * kappa;
   auto seg_end = [&](int s) { return std::min((s + 1) * seg, m) - 1; };
   // backward pass: R_{m-1} = v, R_{k-1} = (K - r_k) R_k; keep R at segment ends
@@ -115,7 +126,7 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
   }
   // forward pass over k with L_k; R_k rebuilt from the segment's checkpoint
   WD_TRY(convert(c, v, L[0]));
-  std::vector<Field> Ye(2 * seg), Yo(2 * seg), Xe(2 * seg), Xo(2 * seg);
+  std::vector<Field> Ye(2 * nl), Yo(2 * nl), Xe(2 * nl), Xo(2 * nl);
   for (int s = 0; s < nseg; ++s) {
     const int a = s * seg, b = seg_end(s);
     WD_TRY(convert(c, cp[s], buf[b - a]));
@@ -128,31 +139,34 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
       c->nmat += 1;
     }
     for (int k = a; k <= b; ++k) {
-      const int j = k - a;
+      const int j = k - a, i = j % nl;         // place in the segment, in the group
+      const bool last = i == nl - 1 || k == b;
       // lo = D_oe L, ml = M_hat L, mlo = D^dag_oe ml (the odd halves of L~ and
       // (M L)~), and the same for R (kept from the rebuild except for its
       // first vector)
-      WD_TRY(hop(c, 1, false, L[j], lo[j], nullptr, 0.0, false, false));
-      WD_TRY(hop(c, 0, false, lo[j], ml[j], &L[j], -k2, false, false));
-      WD_TRY(hop(c, 1, true, ml[j], mlo[j], nullptr, 0.0, false, false));
+      WD_TRY(hop(c, 1, false, L[i], lo[i], nullptr, 0.0, false, false));
+      WD_TRY(hop(c, 0, false, lo[i], ml[i], &L[i], -k2, false, false));
+      WD_TRY(hop(c, 1, true, ml[i], mlo[i], nullptr, 0.0, false, false));
       if (j == 0) {
         WD_TRY(hop(c, 1, false, buf[0], ro[0], nullptr, 0.0, false, false));
         WD_TRY(hop(c, 0, false, ro[0], mr[0], &buf[0], -k2, false, false));
         WD_TRY(hop(c, 1, true, mr[0], mro[0], nullptr, 0.0, false, false));
       }
       // Re((M R)~^dag dD L~) and Re((M L)~^dag dD R~)
-      Ye[2 * j] = mr[j], Yo[2 * j] = mro[j], Xe[2 * j] = L[j], Xo[2 * j] = lo[j];
-      Ye[2 * j + 1] = ml[j], Yo[2 * j + 1] = mlo[j], Xe[2 * j + 1] = buf[j], Xo[2 * j + 1] = ro[j];
+      Ye[2 * i] = mr[j], Yo[2 * i] = mro[j], Xe[2 * i] = L[i], Xo[2 * i] = lo[i];
+      Ye[2 * i + 1] = ml[i], Yo[2 * i + 1] = mlo[i], Xe[2 * i + 1] = buf[j], Xo[2 * i + 1] = ro[j];
       if (k < m - 1) {
         // K L = M^dag (M L) = ml - kappa^2 D^dag_eo mlo: one more hop
         // with the shift of (K - conj r_k) L
-        WD_TRY(hop_shift(c, mlo[j], ml[j], -k2, -rr[k], ri[k], L[j], k < b ? L[j + 1] : Ln));
+        WD_TRY(hop_shift(c, mlo[i], ml[i], -k2, -rr[k], ri[k], L[i], last ? Ln : L[i + 1]));
         c->nmat += 1;
       }
+      if (last) {
+        // the group's pairs in one pass over the links and F
+        WD_TRY(force_pairs(c, -coef * scale * k2, i + 1, Ye.data(), Yo.data(), Xe.data(), Xo.data(), F));
+        std::swap(L[0], Ln);
+      }
     }
-    // the segment's pairs in one pass over the links and F
-    WD_TRY(force_pairs(c, -coef * scale * k2, b - a + 1, Ye.data(), Yo.data(), Xe.data(), Xo.data(), F));
-    std::swap(L[0], Ln);
   }
   return WD_OK;
 }

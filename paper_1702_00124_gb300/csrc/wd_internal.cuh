@@ -824,6 +824,7 @@ int gaussian_draw_k(wd_ctx* c, int what, int parity, uint64_t seed, uint64_t str
 // force layer (force.cu)
 int force_outer(wd_ctx* c, double coef, const Field& Ye, const Field& Yo, const Field& Xe,
                 const Field& Xo, double* F, int prec);
+constexpr int FORCE_ROOTS = 8;   // groups of two pairs that one launch takes
 int force_pairs(wd_ctx* c, double coef, int n, const Field* Ye, const Field* Yo, const Field* Xe, const Field* Xo,
                 double* F);
 
