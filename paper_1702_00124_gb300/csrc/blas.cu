@@ -23,7 +23,10 @@ constexpr int BL_THREADS = 256;
 // plain load (not the read-only path: see pdl_wait)
 template <class W> __device__ __forceinline__ W ldw(const W* p) { return *p; }
 
-constexpr int SUM_BLOCKS = 8 * 152;   // eight blocks per SM: a full GB300
+// Eight blocks per SM, a full GB300.  FP64 CG at 16^3 x 32 with 152 / 304 / 608 / 1216 /
+// 2432 blocks: 43.1 / 42.5 / 42.1 / 41.8 / 42.2 ms; BF16 CG at 12^3 x 24: 5.09 / 5.07 /
+// 5.01 / 5.03 / 5.11 ms (fewer leave each thread a longer chain, more lengthen the last pass)
+constexpr int SUM_BLOCKS = 8 * 152;
 
 
 size_t field_bytes(int fmt, long Vh) {
