@@ -105,8 +105,6 @@ template <int MU, int NP, class T, class S, class G>
 __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4], bool ok) {
   const Geom& g = a.g;
   const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
-  cpx<T> U[9];
-  a.gauge.load(MU, par, cb, U);
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int i = 0; i < a.n; ++i) {
     cpx<T> A[9];
@@ -127,7 +125,8 @@ __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, lon
       half_of<MU, +1>(s, k);
       outer_acc(A, h, k);
     }
-    cpx<T> W[9];
+    cpx<T> U[9], W[9];
+    a.gauge.load(MU, par, cb, U);
     mat_mul(U, A, W);
     T f[8];
     proj_ta(W, f);
@@ -143,8 +142,13 @@ __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, lon
   }
 }
 
+// Two FP32 pairs: latency of the spinor reads, so five blocks per SM (96 registers, 14
+// words spilled).  16 roots at 16^3 x 32, whole force: link kept over the groups, 138
+// registers 2.10 ms; link read again per group (L1), 110 registers 2.05 ms; this 2.00 ms.
+// One pair takes 108 registers; FP64 is bound by its arithmetic.
+template <class T, int NP> constexpr int force_blocks() { return sizeof(T) == 4 && NP == 2 ? 5 : 1; }
 template <class T, int NP, class S, class G>
-__global__ void __launch_bounds__(F_THREADS) k_force(ForceArgs<S, G> a) {
+__global__ void __launch_bounds__(F_THREADS, force_blocks<T, NP>()) k_force(ForceArgs<S, G> a) {
   const int lane = threadIdx.x & 31, mu = threadIdx.x >> 5;
   const int par = blockIdx.y;
   const long site = (long)blockIdx.x * 32 + lane;
