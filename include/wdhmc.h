@@ -77,9 +77,10 @@ enum wd_recon { WD_RECON_18 = 0, WD_RECON_12 = 1 };
 /* Kernel of the FP32/FP16/BF16 hopping stencil with 12-real links (Section 3.1;
  * a kernel choice, the arithmetic is the same):
  *   WD_STENCIL_THREAD  (default) one thread per output site, each thread
- *                      copying its own links two directions ahead into shared
- *                      memory (cp.async) and its next neighbour spinor into
- *                      registers;
+ *                      copying its own links two or more directions ahead into
+ *                      shared memory (cp.async) and its next neighbour spinors
+ *                      into registers; small lattices take eight threads per
+ *                      site, one per direction;
  *   WD_STENCIL_TILE    one persistent block per SM; a producer warp copies the
  *                      links and neighbour-spinor faces of 512-site tiles, one
  *                      direction at a time, into a ring of shared-memory stages
@@ -88,8 +89,8 @@ enum wd_recon { WD_RECON_18 = 0, WD_RECON_12 = 1 };
  *                      memory.  Used where the lattice allows it (Lx/2 a
  *                      multiple of 4 that divides 512 in at most 32 x rows, Vh a
  *                      multiple of 512), elsewhere the thread kernel runs.  At
- *                      32^3 x 64 it takes 0.70 ms per FP32 K_hat against 0.54 ms
- *                      for the thread kernel. */
+ *                      32^3 x 64 it takes 0.70 ms per FP32 K_hat where the thread
+ *                      kernel took 0.54 ms. */
 enum wd_stencil { WD_STENCIL_THREAD = 0, WD_STENCIL_TILE = 1 };
 
 /* Pseudofermion term kinds (Section 2; Section 4.1):
@@ -180,11 +181,12 @@ int wd_kernel_status(wd_ctx* ctx, unsigned* word);
  * wd_kernel_status returns WD_ERR_TIMEOUT (and clears the word).  Nothing else
  * of the context changes.  WD_ERR_ARG for a bound outside the range. */
 int wd_selftest_wait_timeout(wd_ctx* ctx, long long timeout_ns);
-/* Launch-shape autotuner of the hop kernels (no counterpart in the paper; on
- * by default): the first launch
+/* Launch-shape autotuner of the register-only hop kernel (no counterpart in
+ * the paper; on by default), which serves FP64 lattices above 500,000 sites per
+ * parity; every other hop takes its shape from the lattice.  The first launches
  * of each (formats, link storage, dagger, epilogue) outside a queued CG chunk
- * times the candidate block sizes and register caps on the context stream and
- * keeps the fastest for the context's volume.  enable: 1 on, 0 off, -1 leave;
+ * time the candidate block sizes and register caps on the context stream, and the
+ * tuner keeps the fastest for the context's volume.  enable: 1 on, 0 off, -1 leave;
  * *n_tuned (may be NULL) = number of tuned keys. */
 int wd_set_autotune(wd_ctx* ctx, int enable, int* n_tuned);
 /* The index-th tuned entry (no counterpart in the paper; WD_ERR_ARG when
@@ -236,7 +238,7 @@ int mdagm_apply(wd_ctx* ctx, double kappa, int prec, int nrhs, const double* in,
 /* Solve A x = b on even sites, A = K_hat(kappa) (Section 2: K inverted by an
  * iterative solver such as CG), or A = K_hat P(K_hat) when filt != NULL (the
  * [P(K) K]^-1 of the filtered action S_PF, Section 2).  x is the initial guess
- * on entry.  Mixed precision (p->prec != WD_F64) runs the bulk in that
+ * on entry; where |x|^2 = 0 the solve starts from r = b without applying A.  Mixed precision (p->prec != WD_F64) runs the bulk in that
  * precision and recomputes the residual in FP64 (reliable updates).
  * WD_ERR_NOCONV at maxiter, WD_ERR_NAN on a non-finite value. */
 int cg_solve(wd_ctx* ctx, double kappa, const wd_poly* filt, const double* b, double* x,

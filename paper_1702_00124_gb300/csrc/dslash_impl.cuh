@@ -205,8 +205,9 @@ __global__ void __launch_bounds__(MAXT) k_hop(HopArgs<In, Out, Y, G> a) {
   }
 }
 
-// Launch-shape autotuner.  Candidates: block sizes 128 and 64 with the kernel
-// compiled for at most 128 threads (FP32: 86-88 registers, no spills), and
+// Launch-shape autotuner of k_hop (FP64 lattices above SPLIT_MAX_VH_F64; the other
+// kernels take their shape from the number of blocks).  Candidates: block sizes 128 and 64 with the kernel
+// compiled for at most 128 threads, and
 // 256 with a kernel compiled for 256 threads (the compiler then takes up to
 // 255 registers).  Register caps below the compiler's choice spill and lost
 // 4-5 % inside the trajectory, so none is a candidate.  The first launches of

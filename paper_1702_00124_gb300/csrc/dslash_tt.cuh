@@ -25,8 +25,8 @@
 // them, and the consumers read at shared-memory latency.
 //
 // Measured at 32^3 x 64 (FP32 K_hat, links 12 reals): 0.70 ms per application
-// against 0.54 ms for the per-thread staged kernel (dslash_staged.cuh), which
-// stays the default.  With 256-site tiles (8 consumer warps, six 36 KB stages)
+// against 0.54 ms for the per-thread staged kernel of the time (dslash_staged.cuh;
+// 0.41 ms without the conversions today), which stays the default.  With 256-site tiles (8 consumer warps, six 36 KB stages)
 // it took 0.98 ms; ncu showed DRAM traffic equal to the algorithmic bytes but
 // DRAM only 35 % busy, 14 % of warps active and the consumers stalled on the
 // stage barriers: the ring fills at about 37 GB/s per SM.  A producer of two
