@@ -20,6 +20,20 @@ int cuda_fail(cudaError_t e, const char* what) {
   return fail(WD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// A launch recorded by a stream capture runs later, in the graph: the write still
+// needs a plain launch of its own on the stream, and one in every capture.
+bool links_fence(wd_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(c->stream, &st, &id) == cudaSuccess && st == cudaStreamCaptureStatusActive) {
+    const bool first = c->links_capture != id;
+    c->links_capture = id;
+    return first;
+  }
+  c->links_new = false;
+  return true;
+}
+
 int ws_get(wd_ctx* c, int fmt, Field* f) {
   for (size_t i = 0; i < c->pool.size(); ++i) {
     if (!c->pool_used[i] && c->pool[i].fmt == fmt) {
@@ -228,6 +242,7 @@ int wd_volume(const wd_ctx* c, long long out[2]) {
 int wd_gauge_load(wd_ctx* c, const double* U_lex) {
   CHECK_CTX(c);
   CHECK_PTR(U_lex);
+  links_written(c);
   WD_TRY(pack_k(c, false, 4, 9, 2, -1, U_lex, (double*)c->gauge64));
   WD_TRY(gauge_lowprec_k(c));
   c->have_gauge = true;

@@ -144,25 +144,25 @@ int convert(wd_ctx* c, const Field& in, const Field& out) {
   const dim3 g6(nblocks(n, BL_THREADS), 6);
   const int fi = in.fmt, fo = out.fmt;
   if (fi == WD_F64 && fo == WD_F64) {
-    pdl_launch(k_copy<double2>, n12, BL_THREADS, 0, c->stream, 12 * n, (const double2*)in.data, (double2*)out.data);
+    pdl_launch(c, k_copy<double2>, n12, BL_THREADS, 0, 12 * n, (const double2*)in.data, (double2*)out.data);
   } else if (fi == WD_DD && fo == WD_DD) {
-    pdl_launch(k_copy<float4>, n12, BL_THREADS, 0, c->stream, 12 * n, (const float4*)in.data, (float4*)out.data);
+    pdl_launch(c, k_copy<float4>, n12, BL_THREADS, 0, 12 * n, (const float4*)in.data, (float4*)out.data);
   } else if (fi == WD_F32 && fo == WD_F32) {
-    pdl_launch(k_copy<float4>, nblocks(6 * n, BL_THREADS), BL_THREADS, 0, c->stream, 6 * n, (const float4*)in.data,
-                                                                             (float4*)out.data);
+    pdl_launch(c, k_copy<float4>, nblocks(6 * n, BL_THREADS), BL_THREADS, 0, 6 * n, (const float4*)in.data,
+               (float4*)out.data);
   } else if (fi == WD_F64 && fo == WD_F32) {
-    pdl_launch(k_f64_to_f32, g6, BL_THREADS, 0, c->stream, n, (const double2*)in.data, (float4*)out.data);
+    pdl_launch(c, k_f64_to_f32, g6, BL_THREADS, 0, n, (const double2*)in.data, (float4*)out.data);
   } else if (fi == WD_F32 && fo == WD_F64) {
-    pdl_launch(k_f32_to_f64, g6, BL_THREADS, 0, c->stream, n, (const float4*)in.data, (double2*)out.data);
+    pdl_launch(c, k_f32_to_f64, g6, BL_THREADS, 0, n, (const float4*)in.data, (double2*)out.data);
   } else if (fi == WD_F64 && fo == WD_DD) {
-    pdl_launch(k_f64_to_dd, n12, BL_THREADS, 0, c->stream, 12 * n, (const double2*)in.data, (float4*)out.data);
+    pdl_launch(c, k_f64_to_dd, n12, BL_THREADS, 0, 12 * n, (const double2*)in.data, (float4*)out.data);
   } else if (fi == WD_DD && fo == WD_F64) {
-    pdl_launch(k_dd_to_f64, n12, BL_THREADS, 0, c->stream, 12 * n, (const float4*)in.data, (double2*)out.data);
+    pdl_launch(c, k_dd_to_f64, n12, BL_THREADS, 0, 12 * n, (const float4*)in.data, (double2*)out.data);
   } else {
     return with_fmt(in, [&](auto I) {
       return with_fmt(out, [&](auto O) {
         using T = typename Pick<decltype(I), decltype(O)>::T;
-        pdl_launch(k_convert<T, decltype(I), decltype(O)>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, I, O);
+        pdl_launch(c, k_convert<T, decltype(I), decltype(O)>, nblocks(n, BL_THREADS), BL_THREADS, 0, n, I, O);
         WD_CHECK_LAUNCH();
         return (int)WD_OK;
       });
@@ -216,18 +216,18 @@ static void axpby_words(wd_ctx* c, double ar, double ai, const Field& x, double 
   const long m = nwords<F>(c->g.Vh);
   const int nb = nblocks(m, BL_THREADS);
   if (ai == 0.0 && bi == 0.0)
-    pdl_launch(k_axpby<F, true>, nb, BL_THREADS, 0, c->stream, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
+    pdl_launch(c, k_axpby<F, true>, nb, BL_THREADS, 0, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
                                                        (const W*)y.data, (W*)out.data);
   else
-    pdl_launch(k_axpby<F, false>, nb, BL_THREADS, 0, c->stream, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
+    pdl_launch(c, k_axpby<F, false>, nb, BL_THREADS, 0, m, T(ar), T(ai), (const W*)x.data, T(br), T(bi),
                                                         (const W*)y.data, (W*)out.data);
 }
 template <class H>
 static void axpby_16(wd_ctx* c, double ar, double ai, const Field& x, double br, double bi, const Field& y,
                      const Field& out) {
   const long n = c->g.Vh;
-  pdl_launch(k_caxpby<float, Sp16<H>>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, (float)ar, (float)ai, sp16<H>(x), (float)br,
-                                                                        (float)bi, sp16<H>(y), sp16<H>(out));
+  pdl_launch(c, k_caxpby<float, Sp16<H>>, nblocks(n, BL_THREADS), BL_THREADS, 0, n, (float)ar, (float)ai, sp16<H>(x), (float)br,
+               (float)bi, sp16<H>(y), sp16<H>(out));
 }
 
 int caxpby(wd_ctx* c, double ar, double ai, const Field& x, double br, double bi, const Field& y,
@@ -311,14 +311,14 @@ int dot(wd_ctx* c, const Field& a, const Field& b, double* re, double* im) {
   const long n = c->g.Vh;
   WD_TRY(check_sum(c));
   if (a.fmt == WD_F64 && b.fmt == WD_F64) {
-    pdl_launch(k_dot64, sum_blocks(12 * n), BL_THREADS, 0, c->stream, 12 * n, (const double2*)a.data, (const double2*)b.data,
-                                                              reducer_host(c));
+    pdl_launch(c, k_dot64, sum_blocks(12 * n), BL_THREADS, 0, 12 * n, (const double2*)a.data, (const double2*)b.data,
+               reducer_host(c));
     WD_CHECK_LAUNCH();
   } else {
     WD_TRY(with_fmt(a, [&](auto A) {
       return with_fmt(b, [&](auto B) {
         using T = typename Pick<decltype(A), decltype(B)>::T;
-        pdl_launch(k_dot<T, decltype(A), decltype(B)>, nblocks(n, BL_THREADS), BL_THREADS, 0, c->stream, n, A, B, reducer_host(c));
+        pdl_launch(c, k_dot<T, decltype(A), decltype(B)>, nblocks(n, BL_THREADS), BL_THREADS, 0, n, A, B, reducer_host(c));
         WD_CHECK_LAUNCH();
         return (int)WD_OK;
       });
@@ -336,11 +336,11 @@ int dot_hl(wd_ctx* c, const Field& a, const Field& b, double re[2]) {
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
   if (a.data == b.data) {
-    pdl_launch(k_norm64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, reducer_host(c));
+    pdl_launch(c, k_norm64, sum_blocks(n), BL_THREADS, 0, n, (const double2*)a.data, reducer_host(c));
     WD_CHECK_LAUNCH();
     return fetch_host(c, 2, re);
   }
-  pdl_launch(k_dot64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, (const double2*)b.data, reducer_host(c));
+  pdl_launch(c, k_dot64, sum_blocks(n), BL_THREADS, 0, n, (const double2*)a.data, (const double2*)b.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   double v[4];
   WD_TRY(fetch_host(c, 4, v));
@@ -366,7 +366,7 @@ int norm2_any(wd_ctx* c, const Field& b, const Field& x, double* bb, bool* nonze
   if (b.fmt != WD_F64 || x.fmt != WD_F64) return fail(WD_ERR_ARG, "norm2_any: FP64 fields");
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
-  pdl_launch(k_norm_any, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const double2*)x.data,
+  pdl_launch(c, k_norm_any, sum_blocks(n), BL_THREADS, 0, n, (const double2*)b.data, (const double2*)x.data,
              reducer_host(c));
   WD_CHECK_LAUNCH();
   double v[4];
@@ -380,7 +380,7 @@ int norm2(wd_ctx* c, const Field& a, double* out) {
   if (a.fmt != WD_F64) return dot(c, a, a, out, nullptr);
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
-  pdl_launch(k_norm64, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)a.data, reducer_host(c));
+  pdl_launch(c, k_norm64, sum_blocks(n), BL_THREADS, 0, n, (const double2*)a.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   return fetch_host(c, 1, out);
 }
@@ -413,11 +413,11 @@ int residual(wd_ctx* c, const Field& b, const Field& t, const Field& r, double* 
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
   if (t.fmt == WD_F64)
-    pdl_launch(k_resid<SpF64>, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const double2*)t.data,
-                                                                (double2*)r.data, reducer_host(c));
+    pdl_launch(c, k_resid<SpF64>, sum_blocks(n), BL_THREADS, 0, n, (const double2*)b.data, (const double2*)t.data,
+               (double2*)r.data, reducer_host(c));
   else
-    pdl_launch(k_resid<SpDD>, sum_blocks(n), BL_THREADS, 0, c->stream, n, (const double2*)b.data, (const float4*)t.data,
-                                                               (double2*)r.data, reducer_host(c));
+    pdl_launch(c, k_resid<SpDD>, sum_blocks(n), BL_THREADS, 0, n, (const double2*)b.data, (const float4*)t.data,
+               (double2*)r.data, reducer_host(c));
   WD_CHECK_LAUNCH();
   return fetch_host(c, 1, rr);
 }
@@ -449,9 +449,9 @@ int fold(wd_ctx* c, const Field& s, const Field& x) {
   const long n = c->g.Vh;
   if (x.fmt != WD_F64 || (s.fmt != WD_F64 && s.fmt != WD_F32)) return fail(WD_ERR_ARG, "fold: x FP64, s FP32 or FP64");
   if (s.fmt == WD_F32)
-    pdl_launch(k_fold32, dim3(nblocks(n, BL_THREADS), 6), BL_THREADS, 0, c->stream, n, (float4*)s.data, (double2*)x.data);
+    pdl_launch(c, k_fold32, dim3(nblocks(n, BL_THREADS), 6), BL_THREADS, 0, n, (float4*)s.data, (double2*)x.data);
   else
-    pdl_launch(k_fold64, nblocks(12 * n, BL_THREADS), BL_THREADS, 0, c->stream, 12 * n, (double2*)s.data, (double2*)x.data);
+    pdl_launch(c, k_fold64, nblocks(12 * n, BL_THREADS), BL_THREADS, 0, 12 * n, (double2*)s.data, (double2*)x.data);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(BL_THREADS) k_cg_update(long n, typename Words
 // 16-bit p (scaled per site) with FP32 x, r, Ap: one 16-byte word of p, two of the others
 template <class P>
 __global__ void __launch_bounds__(BL_THREADS) k_cg_update16(long Vh, float4* x, P p, float4* r, const float4* ap,
-                                                            CGState* st, Reduce red) {
+               CGState* st, Reduce red) {
   pdl_enter();
   if (st->flag != 0) return;
   const float al = (float)st->alpha;
@@ -595,21 +595,21 @@ int cg_update(wd_ctx* c, const Field& x, const Field& r, const Field& p, const F
     return fail(WD_ERR_ARG, "cg_update: x, r, Ap must share FP64 or FP32");
   if (x.fmt == WD_F64 && p.fmt == WD_F64) {
     const long m = nwords<SpF64>(n);
-    pdl_launch(k_cg_update<SpF64>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (double2*)x.data, (const double2*)p.data,
-                                                                    (double2*)r.data, (const double2*)Ap.data, c->cgs,
-                                                                    reducer(c));
+    pdl_launch(c, k_cg_update<SpF64>, sum_blocks(m), BL_THREADS, 0, m, (double2*)x.data, (const double2*)p.data,
+               (double2*)r.data, (const double2*)Ap.data, c->cgs,
+               reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_F32) {
     const long m = nwords<SpF32>(n);
-    pdl_launch(k_cg_update<SpF32>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (float4*)x.data, (const float4*)p.data,
-                                                                    (float4*)r.data, (const float4*)Ap.data, c->cgs,
-                                                                    reducer(c));
+    pdl_launch(c, k_cg_update<SpF32>, sum_blocks(m), BL_THREADS, 0, m, (float4*)x.data, (const float4*)p.data,
+               (float4*)r.data, (const float4*)Ap.data, c->cgs,
+               reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_F16) {
-    pdl_launch(k_cg_update16<Sp16<__half>>, sum_blocks(3 * n), BL_THREADS, 0, c->stream, n, (float4*)x.data, sp16<__half>(p), (float4*)r.data,
-                                                                   (const float4*)Ap.data, c->cgs, reducer(c));
+    pdl_launch(c, k_cg_update16<Sp16<__half>>, sum_blocks(3 * n), BL_THREADS, 0, n, (float4*)x.data, sp16<__half>(p), (float4*)r.data,
+               (const float4*)Ap.data, c->cgs, reducer(c));
   } else if (x.fmt == WD_F32 && p.fmt == WD_BF16) {
-    pdl_launch(k_cg_update16<Sp16<__nv_bfloat16>>, sum_blocks(3 * n), BL_THREADS, 0, c->stream, n, (float4*)x.data, sp16<__nv_bfloat16>(p),
-                                                                   (float4*)r.data, (const float4*)Ap.data, c->cgs,
-                                                                   reducer(c));
+    pdl_launch(c, k_cg_update16<Sp16<__nv_bfloat16>>, sum_blocks(3 * n), BL_THREADS, 0, n, (float4*)x.data, sp16<__nv_bfloat16>(p),
+               (float4*)r.data, (const float4*)Ap.data, c->cgs,
+               reducer(c));
   } else {
     return fail(WD_ERR_ARG, "cg_update: p must be FP64 with FP64 fields, else FP32 or 16-bit");
   }
@@ -621,16 +621,16 @@ int cg_pupdate(wd_ctx* c, const Field& r, const Field& p) {
   const long n = c->g.Vh;
   if (r.fmt == WD_F64 && p.fmt == WD_F64) {
     const long m = nwords<SpF64>(n);
-    pdl_launch(k_cg_pupdate_w<SpF64>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, (const double2*)r.data,
-                                                                                (double2*)p.data, c->cgs);
+    pdl_launch(c, k_cg_pupdate_w<SpF64>, nblocks(m, BL_THREADS), BL_THREADS, 0, m, (const double2*)r.data,
+               (double2*)p.data, c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_F32) {
     const long m = nwords<SpF32>(n);
-    pdl_launch(k_cg_pupdate_w<SpF32>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, (const float4*)r.data,
-                                                                                (float4*)p.data, c->cgs);
+    pdl_launch(c, k_cg_pupdate_w<SpF32>, nblocks(m, BL_THREADS), BL_THREADS, 0, m, (const float4*)r.data,
+               (float4*)p.data, c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_F16) {
-    pdl_launch(k_cg_pupdate<float, SpF32, Sp16<__half>>, nblocks(n, 128), 128, 0, c->stream, n, sp32(r), sp16<__half>(p), c->cgs);
+    pdl_launch(c, k_cg_pupdate<float, SpF32, Sp16<__half>>, nblocks(n, 128), 128, 0, n, sp32(r), sp16<__half>(p), c->cgs);
   } else if (r.fmt == WD_F32 && p.fmt == WD_BF16) {
-    pdl_launch(k_cg_pupdate<float, SpF32, Sp16<__nv_bfloat16>>, nblocks(n, 128), 128, 0, c->stream, n, sp32(r), sp16<__nv_bfloat16>(p), c->cgs);
+    pdl_launch(c, k_cg_pupdate<float, SpF32, Sp16<__nv_bfloat16>>, nblocks(n, 128), 128, 0, n, sp32(r), sp16<__nv_bfloat16>(p), c->cgs);
   } else {
     return fail(WD_ERR_ARG, "cg_pupdate: r must be FP64 or FP32, p of its format or 16-bit");
   }
@@ -643,12 +643,12 @@ int cg_dot_pap(wd_ctx* c, const Field& p, const Field& Ap) {
     return fail(WD_ERR_ARG, "cg_dot_pap: p and Ap must share FP64 or FP32");
   if (p.fmt == WD_F64) {
     const long m = nwords<SpF64>(c->g.Vh);
-    pdl_launch(k_cg_dot_pap<SpF64>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (const double2*)p.data, (const double2*)Ap.data,
-                                                                     c->cgs, reducer(c));
+    pdl_launch(c, k_cg_dot_pap<SpF64>, sum_blocks(m), BL_THREADS, 0, m, (const double2*)p.data, (const double2*)Ap.data,
+               c->cgs, reducer(c));
   } else {
     const long m = nwords<SpF32>(c->g.Vh);
-    pdl_launch(k_cg_dot_pap<SpF32>, sum_blocks(m), BL_THREADS, 0, c->stream, m, (const float4*)p.data, (const float4*)Ap.data,
-                                                                     c->cgs, reducer(c));
+    pdl_launch(c, k_cg_dot_pap<SpF32>, sum_blocks(m), BL_THREADS, 0, m, (const float4*)p.data, (const float4*)Ap.data,
+               c->cgs, reducer(c));
   }
   WD_CHECK_LAUNCH();
   return WD_OK;
@@ -681,9 +681,9 @@ static void poly_step_words(wd_ctx* c, double a, double mu, double b, const Fiel
   using T = typename Words<F>::T;
   using W = typename Words<F>::W;
   const long m = nwords<F>(c->g.Vh);
-  pdl_launch(k_poly_step<F>, nblocks(m, BL_THREADS), BL_THREADS, 0, c->stream, m, T(a), T(mu), T(b), (const W*)v.data,
-                                                                       (const W*)s.data, (const W*)Ks.data,
-                                                                       (const W*)sprev.data, (W*)out.data);
+  pdl_launch(c, k_poly_step<F>, nblocks(m, BL_THREADS), BL_THREADS, 0, m, T(a), T(mu), T(b), (const W*)v.data,
+               (const W*)s.data, (const W*)Ks.data,
+               (const W*)sprev.data, (W*)out.data);
 }
 int poly_step(wd_ctx* c, double a, double mu, double b, const Field& v, const Field& s,
               const Field& Ks, const Field& sprev, const Field& out) {

@@ -236,7 +236,7 @@ static int hop_dd_launch(wd_ctx* c, const HopArgs<SpDD, SpDD, SpDD, GDD>& a) {
   // early starts pile FP32-bound blocks up on idle SMs as they do FP64-bound ones (dslash_split.cuh)
   const bool early = 2 * nb <= c->nsm || nb >= 2 * c->nsm;
   WD_CUDA(cudaFuncSetAttribute(k_hop_dd<DAG, XPAY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-  pdl_launch_if(early, k_hop_dd<DAG, XPAY>, nb, 256, sm, c->stream, a);
+  pdl_launch_if(c, early, k_hop_dd<DAG, XPAY>, nb, 256, sm, a);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }

@@ -47,8 +47,8 @@ static void hop_poly(wd_ctx* c, const G& gauge, double alpha, const Field& in, c
                      const HopPoly& pe) {
   const HopArgs<SpF32, SpF32, SpF32, G> a{c->g, 0, sp32(in), sp32(out), sp32(y), gauge, alpha, reducer(c), nullptr};
   if (split_eligible(c, WD_F32))
-    pdl_launch(k_hop_split<float, true, EPI, false, SpF32, SpF32, SpF32, G>, nblocks(c->g.Vh, SPL_SITES), SPL_THREADS, 0,
-               c->stream, a, pe);
+    pdl_launch(c, k_hop_split<float, true, EPI, false, SpF32, SpF32, SpF32, G>, nblocks(c->g.Vh, SPL_SITES), SPL_THREADS,
+               0, a, pe);
   else
     hop_st_depth<true, EPI, false>(c, a, pe);
 }

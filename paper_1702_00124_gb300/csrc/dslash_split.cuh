@@ -260,12 +260,12 @@ int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, 
   // and 96.8, 16^3 x 32 (2048) 437 and 426.
   const bool early = !std::is_same<T, double>::value || 2 * nb <= c->nsm || nb >= 2 * c->nsm;
   if (!dag) {
-    if (!xpay) pdl_launch_if(early, k_hop_split<T, false, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
-    else if (!norm) pdl_launch_if(early, k_hop_split<T, false, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
-    else pdl_launch_if(early, k_hop_split<T, false, 1, true, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
+    if (!xpay) pdl_launch_if(c, early, k_hop_split<T, false, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
+    else if (!norm) pdl_launch_if(c, early, k_hop_split<T, false, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
+    else pdl_launch_if(c, early, k_hop_split<T, false, 1, true, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
   } else {
-    if (!xpay) pdl_launch_if(early, k_hop_split<T, true, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
-    else pdl_launch_if(early, k_hop_split<T, true, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, c->stream, a, pe);
+    if (!xpay) pdl_launch_if(c, early, k_hop_split<T, true, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
+    else pdl_launch_if(c, early, k_hop_split<T, true, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
   }
   WD_CHECK_LAUNCH();
   return WD_OK;

@@ -286,7 +286,7 @@ void hop_st_go(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {
       asked.fetch_or(bit);
     }
   }
-  pdl_launch(k, nblocks(c->g.Vh, HOP_ST_THREADS), HOP_ST_THREADS, sm, c->stream, a, pe);
+  pdl_launch(c, k, nblocks(c->g.Vh, HOP_ST_THREADS), HOP_ST_THREADS, sm, a, pe);
 }
 template <bool DAG, int EPI, bool NORM, class In, class Out, class Y, class G>
 void hop_st_depth(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {

@@ -230,6 +230,7 @@ __global__ void __launch_bounds__(H_THREADS) k_step_T(Geom g, const double* P, d
 
 int step_T_k(wd_ctx* c, const double* P, double eps) {
   const long n = 8 * c->g.Vh;
+  links_written(c);
   k_step_T<<<nblocks(n, H_THREADS), H_THREADS, 0, c->stream>>>(c->g, P, eps, c->gauge64, c->gauge32,
                                                                 c->gauge32r12, c->gauge_dd);
   WD_CHECK_LAUNCH();

@@ -123,6 +123,7 @@ __global__ void k_gauge_lowprec(long n9, long Vh, const double2* U64, float2* U3
 
 int gauge_lowprec_k(wd_ctx* c) {
   const long n = 8 * c->g.Vh;
+  links_written(c);
   k_gauge_lowprec<<<nblocks(n, 128), 128, 0, c->stream>>>(n, c->g.Vh, c->gauge64, c->gauge32, c->gauge32r12,
                                                           c->gauge_dd);
   WD_CHECK_LAUNCH();

@@ -66,7 +66,7 @@ int launch(cudaStream_t s, const Geom& g, int out_par, const double2* gauge, con
   // caller's own kernels may write the links it reads
   auto k = k_hop_split<double, DAG, XPAY ? 1 : 0, false, SpF64, SpF64, SpF64, GF64>;
   if (first) k<<<nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s>>>(a, HopPoly{});
-  else pdl_launch(k, nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s, a, HopPoly{});
+  else launch_early(true, k, nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s, a, HopPoly{});
   WD_CUDA(cudaGetLastError());
   return WD_OK;
 }

@@ -238,16 +238,17 @@ struct Geom {
 // Programmatic dependent launch.  A chain of small kernels on one stream is
 // spaced by the launch latency: 4.1 us a kernel launched plainly, 1.35 us when a
 // kernel may start while its predecessor drains (GB300, chains of 128 x 128
-// threads).  The FP32 and 16-bit stencils on 12-real links, the eight-threads-per-site
-// stencil and the vector kernels call pdl_enter (or pdl_trigger at the top and pdl_wait)
-// and are launched by pdl_launch.  The register-only, double-float, force and batched
-// kernels are not: they run for tens of microseconds and lose more to plain
-// loads than the overlap gains (18-real FP32 K_hat at 32^3 x 64 680 -> 813 us,
-// double-float 2345 -> 2494 us).
+// threads).  The staged stencil (FP32 and 16-bit spinors, both link storages), the
+// eight-threads-per-site stencils (FP64, FP32, 16-bit, double-float) and the vector kernels
+// call pdl_enter (or pdl_trigger at the top and pdl_wait) and are launched by pdl_launch.
+// The register-only FP64, tile, force, link-update and batched kernels are not.
 //   - Before pdl_wait a kernel reads nothing but its arguments and the link copies.
 //     Links are written by kernels that never trigger (k_step_T, k_pack,
-//     k_gauge_lowprec) and by copies, so a kernel that starts after them,
-//     or after a kernel that did, finds them complete.
+//     k_gauge_lowprec).  A kernel that starts early after one of these starts when its
+//     blocks are done, but its writes are promised to be visible only after pdl_wait.  So
+//     those writers call links_written, and the next launch of the context that could start
+//     early is a plain one, which starts when all before it is done and visible;
+//     every kernel behind that one starts later still.
 //   - pdl_wait returns when every earlier kernel of the stream has completed: each
 //     of them has waited for its own predecessor.  Spinors, sums and the solver
 //     state are read after it, by plain loads (loadT<false>; a read-only load could
@@ -260,7 +261,7 @@ __device__ __forceinline__ void pdl_enter() {
   pdl_wait();
 }
 template <class... P, class... A>
-inline void pdl_launch_if(bool early, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
+inline void launch_early(bool early, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -272,10 +273,6 @@ inline void pdl_launch_if(bool early, void (*k)(P...), dim3 grid, dim3 block, si
   cfg.attrs = at;
   cfg.numAttrs = early ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);   // the caller checks cudaGetLastError
-}
-template <class... P, class... A>
-inline void pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
-  pdl_launch_if(true, k, grid, block, smem, s, a...);
 }
 
 // ----------------------------------------------------------------------------
@@ -689,6 +686,8 @@ struct wd_ctx {
   int device = 0;
   int recon = WD_RECON_18;
   bool have_gauge = false;
+  bool links_new = false;           // links written since the last plain launch by pdl_launch
+  unsigned long long links_capture = 0;   // stream capture that holds a plain launch after the write
   // gauge copies
   double2* gauge64 = nullptr;       // [4][2][9][Vh]
   float2* gauge32 = nullptr;        // [4][2][9][Vh]
@@ -720,6 +719,22 @@ struct wd_ctx {
 };
 
 namespace wd {
+
+// launches on the context's stream that may start early (above); plain where links are new
+bool links_fence(wd_ctx* c);   // new links: whether this launch has to be the plain one (api.cu)
+inline void links_written(wd_ctx* c) {   // before the launch that writes them
+  c->links_new = true;
+  c->links_capture = 0;
+}
+template <class... P, class... A>
+inline void pdl_launch_if(wd_ctx* c, bool early, void (*k)(P...), dim3 grid, dim3 block, size_t smem, A... a) {
+  const bool plain = c->links_new && links_fence(c);
+  launch_early(early && !plain, k, grid, block, smem, c->stream, a...);
+}
+template <class... P, class... A>
+inline void pdl_launch(wd_ctx* c, void (*k)(P...), dim3 grid, dim3 block, size_t smem, A... a) {
+  pdl_launch_if(c, true, k, grid, block, smem, a...);
+}
 
 // error reporting (thread local message)
 void set_error(const std::string& msg);
