@@ -61,10 +61,13 @@ static int hop_poly_links(wd_ctx* c, double alpha, const Field& in, const Field&
   return WD_OK;
 }
 
-// out = y + alpha D^dag_eo in + z v, the last hop of a factor (K_hat + z) v
+// whether hop_shift is one launch on fields of the format (it takes a vector of its own if not)
+bool hop_shift_fused(wd_ctx* c, int fmt) { return fmt == WD_F32 && hop_widens(c); }   // not the tile-staged option
+
+// out = y + alpha D^dag_eo in + z v, the last hop of a factor (K_hat + z) v; out may be v
 int hop_shift(wd_ctx* c, const Field& in, const Field& y, double alpha, double zr, double zi, const Field& v,
               const Field& out) {
-  if (in.fmt == WD_F32 && hop_widens(c)) {   // not the tile-staged option
+  if (hop_shift_fused(c, in.fmt)) {
     const Field* fields[] = {&y, &v, &out};
     for (const Field* f : fields)
       if (f->fmt != WD_F32) return fail(WD_ERR_ARG, "hop_shift: formats differ");

@@ -88,48 +88,73 @@ static int k_minus(wd_ctx* c, double kappa, double zr, double zi, const Field& x
   return WD_OK;
 }
 
-// Force of S = v^dag Q(K) v, Q = scale prod_k (K - r_k), added with coef.
+// Force of S = v^dag Q(K) v, Q = scale prod_k (K - r_k), added with coef.  v is used up;
+// scratch64 (or null): an FP64 vector of the caller's that is free meanwhile.
 static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, const std::vector<double>& ri,
-                      double scale, const Field& v, double coef, double* F) {
+                      double scale, const Field& v, const Field* scratch64, double coef, double* F) {
   const int m = (int)rr.size();
   const int f = v.fmt;
   const int seg = std::max(1, (int)std::ceil(std::sqrt((double)m)));
   const int nseg = (m + seg - 1) / seg;
+  // The outer products of a group of roots go out in one launch, which reads and writes
+  // F once.  Memory: no more than one root per launch takes (nseg + 4 seg + 7 vectors and
+  // three inside k_minus), for what the pool takes it keeps: as many roots share a launch as
+  // the vectors that are free at the time hold (16 roots: 3, 1, 3, 1, 4, 4).  Whole force of
+  // 16 roots at 16^3 x 32 (FP32): one launch for each checkpoint segment, with vectors
+  // of its own (15 more), 1.99 ms; 1, 2, 1, 2, 2, ... roots 2.18 ms; this 2.06 ms.
+  // `spare` holds the vectors not in use: cp, the R at the segments' ends; buf, ro, mr, mro,
+  // the R of one segment with D_oe R, M_hat R and D^dag_oe M_hat R, formed while K_hat
+  // is applied to them in the segment's rebuild; L, lo, ml, mlo, the same of a group of L.
   WsGuard w(c);
-  // buf: the R of one segment; ro / mr / mro: D_oe R, M_hat R and D^dag_oe M_hat R
-  // of those R, formed while K_hat is applied to them in the segment rebuild;
-  // L, lo, ml, mlo: the same of a group of up to nl of its L, whose outer products
-  // go out in one launch.  Where memory is short the group shrinks, down to one root
-  // (nseg + 4 seg + 6 vectors in all, one launch per root)
-  std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg), L(seg), lo(seg), ml(seg), mlo(seg);
-  Field Ln, cur;
-  for (auto& x : cp) WD_TRY(w.get(f, &x));
-  for (auto* v : {&buf, &ro, &mr, &mro})
-    for (auto& x : *v) WD_TRY(w.get(f, &x));
-  for (Field* x : {&Ln, &cur, &L[0], &lo[0], &ml[0], &mlo[0]}) WD_TRY(w.get(f, x));
-  int nl = 1;
-  for (; nl < std::min(seg, FORCE_ROOTS); ++nl) {
-    bool ok = true;
-    for (Field* x : {&L[nl], &lo[nl], &ml[nl], &mlo[nl]}) ok = ok && w.get(f, x) == WD_OK;
-    if (!ok) {
-      cudaGetLastError();                      // out of memory: handled here
-      break;
-    }
-  }
+  std::vector<Field> spare(nseg + 4 * seg + 7);
+  for (auto& x : spare) WD_TRY(w.get(f, &x));
+  auto take = [&] {
+    const Field x = spare.back();
+    spare.pop_back();
+    return x;
+  };
+  std::vector<Field> cp(nseg), buf(seg), ro(seg), mr(seg), mro(seg);
+  Field L[FORCE_ROOTS], lo[FORCE_ROOTS], ml[FORCE_ROOTS], mlo[FORCE_ROOTS];
+  Field Ye[2 * FORCE_ROOTS], Yo[2 * FORCE_ROOTS], Xe[2 * FORCE_ROOTS], Xo[2 * FORCE_ROOTS];
   const double k2 = kappa * kappa;
   auto seg_end = [&](int s) { return std::min((s + 1) * seg, m) - 1; };
   // backward pass: R_{m-1} = v, R_{k-1} = (K - r_k) R_k; keep R at segment ends
+  const Field cur = take();
   WD_TRY(convert(c, v, cur));
   for (int s = nseg - 1, k = m - 1; k >= 0; --k) {
-    if (s >= 0 && k == seg_end(s)) { WD_TRY(convert(c, cur, cp[s])); --s; }
+    if (s >= 0 && k == seg_end(s)) {
+      cp[s] = take();
+      WD_TRY(convert(c, cur, cp[s]));
+      --s;
+    }
     if (k > 0) WD_TRY(k_minus(c, kappa, rr[k], ri[k], cur, cur));
   }
+  spare.push_back(cur);
+  // k_minus is done: its three vectors (one stays for hop_shift where that needs it), scratch64
+  for (int i = m == 1 ? 0 : hop_shift_fused(c, f) ? 3 : 2; i > 0; --i) {
+    Field x;
+    WD_TRY(w.get(f, &x));
+    spare.push_back(x);
+  }
+  if (scratch64 != nullptr) {
+    Field x = *scratch64;
+    x.fmt = f;
+    spare.push_back(x);
+    if (f == WD_F32) {
+      x.data = (char*)x.data + field_bytes(WD_F32, c->g.Vh);
+      spare.push_back(x);
+    }
+  }
   // forward pass over k with L_k; R_k rebuilt from the segment's checkpoint
-  WD_TRY(convert(c, v, L[0]));
-  std::vector<Field> Ye(2 * nl), Yo(2 * nl), Xe(2 * nl), Xo(2 * nl);
+  L[0] = v;
   for (int s = 0; s < nseg; ++s) {
     const int a = s * seg, b = seg_end(s);
-    WD_TRY(convert(c, cp[s], buf[b - a]));
+    for (int j = 0; j <= b - a; ++j) {
+      buf[j] = j == b - a ? cp[s] : take();
+      ro[j] = take();
+      mr[j] = take();
+      mro[j] = take();
+    }
     // R_{a+j-1} = (K - r_{a+j}) R_{a+j}, keeping the hops of each K R_{a+j}
     for (int j = b - a; j >= 1; --j) {
       WD_TRY(hop(c, 1, false, buf[j], ro[j], nullptr, 0.0, false, false));
@@ -138,34 +163,46 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
       WD_TRY(hop_shift(c, mro[j], mr[j], -k2, -rr[a + j], -ri[a + j], buf[j], buf[j - 1]));
       c->nmat += 1;
     }
-    for (int k = a; k <= b; ++k) {
-      const int j = k - a, i = j % nl;         // place in the segment, in the group
-      const bool last = i == nl - 1 || k == b;
-      // lo = D_oe L, ml = M_hat L, mlo = D^dag_oe ml (the odd halves of L~ and
-      // (M L)~), and the same for R (kept from the rebuild except for its
-      // first vector)
-      WD_TRY(hop(c, 1, false, L[i], lo[i], nullptr, 0.0, false, false));
-      WD_TRY(hop(c, 0, false, lo[i], ml[i], &L[i], -k2, false, false));
-      WD_TRY(hop(c, 1, true, ml[i], mlo[i], nullptr, 0.0, false, false));
-      if (j == 0) {
-        WD_TRY(hop(c, 1, false, buf[0], ro[0], nullptr, 0.0, false, false));
-        WD_TRY(hop(c, 0, false, ro[0], mr[0], &buf[0], -k2, false, false));
-        WD_TRY(hop(c, 1, true, mr[0], mro[0], nullptr, 0.0, false, false));
+    WD_TRY(hop(c, 1, false, buf[0], ro[0], nullptr, 0.0, false, false));
+    WD_TRY(hop(c, 0, false, ro[0], mr[0], &buf[0], -k2, false, false));
+    WD_TRY(hop(c, 1, true, mr[0], mro[0], nullptr, 0.0, false, false));
+    for (int k = a; k <= b;) {
+      // n roots: three vectors for the first, four for each one after it
+      const int n = std::min({FORCE_ROOTS, b - k + 1, ((int)spare.size() + 1) / 4});
+      for (int i = 0; i < n; ++i) {
+        const int j = k - a + i;               // place in the segment
+        // L_k = (K - conj r_{k-1}) L_{k-1}, K L = M^dag (M L) = ml - kappa^2 D^dag_eo mlo: one
+        // more hop, with the shift
+        if (i > 0) {
+          L[i] = take();
+          WD_TRY(hop_shift(c, mlo[i - 1], ml[i - 1], -k2, -rr[k + i - 1], ri[k + i - 1], L[i - 1], L[i]));
+          c->nmat += 1;
+        }
+        // lo = D_oe L, ml = M_hat L, mlo = D^dag_oe ml: the odd halves of L~ and (M L)~
+        lo[i] = take();
+        ml[i] = take();
+        mlo[i] = take();
+        WD_TRY(hop(c, 1, false, L[i], lo[i], nullptr, 0.0, false, false));
+        WD_TRY(hop(c, 0, false, lo[i], ml[i], &L[i], -k2, false, false));
+        WD_TRY(hop(c, 1, true, ml[i], mlo[i], nullptr, 0.0, false, false));
+        // Re((M R)~^dag dD L~) and Re((M L)~^dag dD R~)
+        Ye[2 * i] = mr[j], Yo[2 * i] = mro[j], Xe[2 * i] = L[i], Xo[2 * i] = lo[i];
+        Ye[2 * i + 1] = ml[i], Yo[2 * i + 1] = mlo[i], Xe[2 * i + 1] = buf[j], Xo[2 * i + 1] = ro[j];
       }
-      // Re((M R)~^dag dD L~) and Re((M L)~^dag dD R~)
-      Ye[2 * i] = mr[j], Yo[2 * i] = mro[j], Xe[2 * i] = L[i], Xo[2 * i] = lo[i];
-      Ye[2 * i + 1] = ml[i], Yo[2 * i + 1] = mlo[i], Xe[2 * i + 1] = buf[j], Xo[2 * i + 1] = ro[j];
-      if (k < m - 1) {
-        // K L = M^dag (M L) = ml - kappa^2 D^dag_eo mlo: one more hop
-        // with the shift of (K - conj r_k) L
-        WD_TRY(hop_shift(c, mlo[i], ml[i], -k2, -rr[k], ri[k], L[i], last ? Ln : L[i + 1]));
+      // the group's pairs in one pass over the links and F
+      WD_TRY(force_pairs(c, -coef * scale * k2, n, Ye, Yo, Xe, Xo, F));
+      const Field last = L[n - 1];
+      if (k + n < m) {                         // the next group's first L, in place
+        WD_TRY(hop_shift(c, mlo[n - 1], ml[n - 1], -k2, -rr[k + n - 1], ri[k + n - 1], last, last));
         c->nmat += 1;
       }
-      if (last) {
-        // the group's pairs in one pass over the links and F
-        WD_TRY(force_pairs(c, -coef * scale * k2, i + 1, Ye.data(), Yo.data(), Xe.data(), Xo.data(), F));
-        std::swap(L[0], Ln);
+      for (int i = 0; i < n; ++i) {
+        const int j = k - a + i;
+        for (const Field& x : {buf[j], ro[j], mr[j], mro[j], lo[i], ml[i], mlo[i]}) spare.push_back(x);
+        if (i + 1 < n) spare.push_back(L[i]);
       }
+      L[0] = last;
+      k += n;
     }
   }
   return WD_OK;
@@ -326,8 +363,9 @@ int term_heatbath(wd_ctx* c, const wd_term& t, const Field& chi, const wd_cg_par
 
 // Force from a given solution X (and Y = M_hat X, or nullptr to form it):
 // no solve.  POLY and RATIO ignore X and Y.  f = FP64 or FP32 arithmetic.
-int term_force_xy(wd_ctx* c, const wd_term& t, const Field& phi, const Field* X, const Field* Y, int f,
-                  double coef, double* F) {
+// scratch64: an FP64 vector that POLY and RATIO may use, or nullptr.
+int term_force_xy(wd_ctx* c, const wd_term& t, const Field& phi, const Field* X, const Field* Y, const Field* scratch64,
+                  int f, double coef, double* F) {
   WsGuard w(c);
   Field Xf, Yf, phif;
   switch (t.kind) {
@@ -351,14 +389,14 @@ int term_force_xy(wd_ctx* c, const wd_term& t, const Field& phi, const Field* X,
       WD_TRY(poly_coef(t.poly, &pc));
       WD_TRY(w.get(f, &phif));
       WD_TRY(convert(c, phi, phif));
-      return poly_force(c, t.kappa, pc.zr, pc.zi, pc.scale, phif, coef, F);
+      return poly_force(c, t.kappa, pc.zr, pc.zi, pc.scale, phif, scratch64, coef, F);
     }
     case WD_TERM_RATIO: {
       PolyCoef q;
       WD_TRY(ratio_coef(t.poly, t.poly_lo, &q));
       WD_TRY(w.get(f, &phif));
       WD_TRY(convert(c, phi, phif));
-      return poly_force(c, t.kappa, q.zr, q.zi, q.scale, phif, coef, F);
+      return poly_force(c, t.kappa, q.zr, q.zi, q.scale, phif, scratch64, coef, F);
     }
     case WD_TERM_FILTERED: {
       PolyCoef pc;
@@ -368,7 +406,7 @@ int term_force_xy(wd_ctx* c, const wd_term& t, const Field& phi, const Field* X,
       std::vector<double> rr(1, 0.0), ri(1, 0.0);
       rr.insert(rr.end(), pc.zr.begin(), pc.zr.end());
       ri.insert(ri.end(), pc.zi.begin(), pc.zi.end());
-      return poly_force(c, t.kappa, rr, ri, pc.scale, Xf, -coef, F);
+      return poly_force(c, t.kappa, rr, ri, pc.scale, Xf, nullptr, -coef, F);
     }
   }
   return fail(WD_ERR_ARG, "unknown term kind");
@@ -386,13 +424,13 @@ int term_force(wd_ctx* c, const wd_term& t, const Field& phi, const wd_cg_params
       if (t.kind == WD_TERM_PLAIN) WD_TRY(convert(c, phi, b));
       else WD_TRY(mhat(c, t.kappa_h, true, phi, b));
       WD_TRY(solve(c, t.kappa, nullptr, b, X, p));
-      return term_force_xy(c, t, phi, &X, nullptr, f, coef, F);
+      return term_force_xy(c, t, phi, &X, nullptr, nullptr, f, coef, F);
     case WD_TERM_POLY:
     case WD_TERM_RATIO:
-      return term_force_xy(c, t, phi, nullptr, nullptr, f, coef, F);
+      return term_force_xy(c, t, phi, nullptr, nullptr, &X, f, coef, F);
     case WD_TERM_FILTERED:
       WD_TRY(solve(c, t.kappa, &t.poly, phi, X, p));
-      return term_force_xy(c, t, phi, &X, nullptr, f, coef, F);
+      return term_force_xy(c, t, phi, &X, nullptr, nullptr, f, coef, F);
   }
   return fail(WD_ERR_ARG, "unknown term kind");
 }
@@ -577,7 +615,7 @@ int fermion_force_xy(wd_ctx* c, const wd_term* term, const double* phi, const do
   if (!c->have_gauge) return fail(WD_ERR_STATE, "no gauge field loaded");
   Field fx = wrap_f64(c, X), fy = wrap_f64(c, Y);
   const bool useY = Y != nullptr && (term->kind == WD_TERM_PLAIN || term->kind == WD_TERM_HASENBUSCH);
-  return term_force_xy(c, *term, wrap_f64(c, phi), X ? &fx : nullptr, useY ? &fy : nullptr, prec, coef, F);
+  return term_force_xy(c, *term, wrap_f64(c, phi), X ? &fx : nullptr, useY ? &fy : nullptr, nullptr, prec, coef, F);
 }
 
 int pf_heatbath(wd_ctx* c, const wd_term* term, const double* chi, const wd_cg_params* p, double* phi) {
