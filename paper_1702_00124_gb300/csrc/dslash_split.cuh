@@ -253,12 +253,7 @@ int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, 
   if (norm && (dag || !xpay)) return fail(WD_ERR_ARG, "hop: the |out|^2 epilogue exists for M_hat only");
   const int nb = nblocks(c->g.Vh, SPL_SITES);
   const HopPoly pe{};
-  // An early start puts a kernel's blocks where the one before has left room.  FP64
-  // blocks fill the pipe of their SM, so between one block for every other SM
-  // and two for each the early ones pile up on the idle SMs: K_hat at 8^3 x 16
-  // (128 blocks) 49.6 us, early 91.7; 4^4 (4) 47.6 and 36.0, 12^4 (324) 106.9
-  // and 96.8, 16^3 x 32 (2048) 437 and 426.
-  const bool early = !std::is_same<T, double>::value || 2 * nb <= c->nsm || nb >= 2 * c->nsm;
+  const bool early = !std::is_same<T, double>::value || early_gains(nb, c->nsm);
   if (!dag) {
     if (!xpay) pdl_launch_if(c, early, k_hop_split<T, false, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
     else if (!norm) pdl_launch_if(c, early, k_hop_split<T, false, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);

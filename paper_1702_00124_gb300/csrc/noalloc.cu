@@ -39,9 +39,11 @@ static __device__ __align__(256) double2 g_noalloc_scratch[2 * 12 * NOALLOC_MAX_
 
 std::mutex g_noalloc_mutex;
 double2* g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
+int g_noalloc_nsm[NOALLOC_MAX_DEVICES] = {};
 
-// Device address of the scratch array on the current device (looked up once).
-int scratch_address(double2** out) {
+// Device address of the scratch array on the current device and its number of SMs
+// (looked up once).
+int scratch_address(double2** out, int* nsm) {
   int dev = 0;
   WD_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return fail(WD_ERR_ARG, "mdagm_apply_noalloc: device index out of range");
@@ -50,23 +52,22 @@ int scratch_address(double2** out) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
+    WD_CUDA(cudaDeviceGetAttribute(&g_noalloc_nsm[dev], cudaDevAttrMultiProcessorCount, dev));
     g_noalloc_ptr[dev] = static_cast<double2*>(p);
   }
   *out = g_noalloc_ptr[dev];
+  *nsm = g_noalloc_nsm[dev];
   return WD_OK;
 }
 
 template <bool DAG, bool XPAY>
 int launch(cudaStream_t s, const Geom& g, int out_par, const double2* gauge, const double2* in, double2* out,
-           const double2* y, double alpha, bool first = false) {
+           const double2* y, double alpha, bool early) {
   using A = HopArgs<SpF64, SpF64, SpF64, GF64>;
   SpF64 I{const_cast<double2*>(in), g.Vh}, O{out, g.Vh}, Y{const_cast<double2*>(y ? y : in), g.Vh};
   A a{g, out_par, I, O, Y, GF64{gauge, g.Vh}, alpha, Reduce{nullptr, nullptr, nullptr}, nullptr};
-  // the first of the four hops starts after everything before it on the stream: the
-  // caller's own kernels may write the links it reads
   auto k = k_hop_split<double, DAG, XPAY ? 1 : 0, false, SpF64, SpF64, SpF64, GF64>;
-  if (first) k<<<nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s>>>(a, HopPoly{});
-  else launch_early(true, k, nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s, a, HopPoly{});
+  launch_early(early, k, nblocks(g.Vh, SPL_SITES), SPL_THREADS, 0, s, a, HopPoly{});
   WD_CUDA(cudaGetLastError());
   return WD_OK;
 }
@@ -91,7 +92,8 @@ extern "C" int mdagm_apply_noalloc(const int dims[4], const double* gauge_eo, do
     return fail(WD_ERR_ARG, "mdagm_apply_noalloc: lattice has more than 32768 sites per parity "
                             "(the fixed scratch size); use mdagm_apply with a context instead");
   double2* scratch = nullptr;
-  WD_TRY(scratch_address(&scratch));
+  int nsm = 0;
+  WD_TRY(scratch_address(&scratch, &nsm));
   double2* t1 = scratch;                   // odd sites
   double2* t2 = scratch + 12 * g.Vh;       // even sites
   const cudaStream_t s = (cudaStream_t)stream;
@@ -99,9 +101,12 @@ extern "C" int mdagm_apply_noalloc(const int dims[4], const double* gauge_eo, do
   const double2* x = (const double2*)in;
   double2* y = (double2*)out;
   const double a = -kappa * kappa;
-  WD_TRY((launch<false, false>(s, g, 1, G, x, t1, nullptr, 0.0, true)));   // t1 = D_oe x
-  WD_TRY((launch<false, true>(s, g, 0, G, t1, t2, x, a)));           // t2 = x - k^2 D_eo t1 = M_hat x
-  WD_TRY((launch<true, false>(s, g, 1, G, t2, t1, nullptr, 0.0)));   // t1 = D^dag_oe t2
-  WD_TRY((launch<true, true>(s, g, 0, G, t1, y, t2, a)));            // out = M_hat^dag t2
+  // the first of the four hops starts after everything before it on the stream: the
+  // caller's own kernels may write the links it reads
+  const bool early = early_gains(nblocks(g.Vh, SPL_SITES), nsm);
+  WD_TRY((launch<false, false>(s, g, 1, G, x, t1, nullptr, 0.0, false)));   // t1 = D_oe x
+  WD_TRY((launch<false, true>(s, g, 0, G, t1, t2, x, a, early)));           // t2 = x - k^2 D_eo t1 = M_hat x
+  WD_TRY((launch<true, false>(s, g, 1, G, t2, t1, nullptr, 0.0, early)));   // t1 = D^dag_oe t2
+  WD_TRY((launch<true, true>(s, g, 0, G, t1, y, t2, a, early)));            // out = M_hat^dag t2
   return WD_OK;
 }
