@@ -234,7 +234,7 @@ static int hop_dd_launch(wd_ctx* c, const HopArgs<SpDD, SpDD, SpDD, GDD>& a) {
   constexpr int sm = (8 * 6 * 32 + 9 * 256) * (int)sizeof(float4);   // 61 KB: three blocks per SM
   const int nb = nblocks(c->g.Vh, 32);
   WD_CUDA(cudaFuncSetAttribute(k_hop_dd<DAG, XPAY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-  pdl_launch_if(c, early_gains(nb, c->nsm), k_hop_dd<DAG, XPAY>, nb, 256, sm, a);
+  pdl_launch_if(c, early_gains_dd(nb, c->nsm), k_hop_dd<DAG, XPAY>, nb, 256, sm, a);
   WD_CHECK_LAUNCH();
   return WD_OK;
 }

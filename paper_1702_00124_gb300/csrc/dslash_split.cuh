@@ -253,7 +253,7 @@ int hop_split(wd_ctx* c, bool dag, bool xpay, bool norm, const HopArgs<In, Out, 
   if (norm && (dag || !xpay)) return fail(WD_ERR_ARG, "hop: the |out|^2 epilogue exists for M_hat only");
   const int nb = nblocks(c->g.Vh, SPL_SITES);
   const HopPoly pe{};
-  const bool early = !std::is_same<T, double>::value || early_gains(nb, c->nsm);
+  const bool early = !std::is_same<T, double>::value || early_gains_f64(nb, c->nsm);
   if (!dag) {
     if (!xpay) pdl_launch_if(c, early, k_hop_split<T, false, 0, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);
     else if (!norm) pdl_launch_if(c, early, k_hop_split<T, false, 1, false, In, Out, Y, G>, nb, SPL_THREADS, 0, a, pe);

@@ -103,7 +103,7 @@ extern "C" int mdagm_apply_noalloc(const int dims[4], const double* gauge_eo, do
   const double a = -kappa * kappa;
   // the first of the four hops starts after everything before it on the stream: the
   // caller's own kernels may write the links it reads
-  const bool early = early_gains(nblocks(g.Vh, SPL_SITES), nsm);
+  const bool early = early_gains_f64(nblocks(g.Vh, SPL_SITES), nsm);
   WD_TRY((launch<false, false>(s, g, 1, G, x, t1, nullptr, 0.0, false)));   // t1 = D_oe x
   WD_TRY((launch<false, true>(s, g, 0, G, t1, t2, x, a, early)));           // t2 = x - k^2 D_eo t1 = M_hat x
   WD_TRY((launch<true, false>(s, g, 1, G, t2, t1, nullptr, 0.0, early)));   // t1 = D^dag_oe t2

@@ -275,11 +275,16 @@ inline void launch_early(bool early, void (*k)(P...), dim3 grid, dim3 block, siz
   (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);   // the caller checks cudaGetLastError
 }
 // Whether a stencil of nb blocks that fill the pipe of their SM (FP64, double-float) gains
-// by an early start, which puts a kernel's blocks where the one before has left room:
-// between one block for every other SM and two for each the early ones pile up on the
-// idle SMs.  FP64 K_hat, plain and early: 8^3 x 16 (128 blocks) 49.6 and 91.7 us; 4^4 (4)
-// 47.6 and 36.0, 12^4 (324) 106.9 and 96.8, 16^3 x 32 (2048) 437 and 426.
-inline bool early_gains(int nb, int nsm) { return 2 * nb <= nsm || nb >= 2 * nsm; }
+// by an early start, which puts a kernel's blocks where the ones before have left room.
+// FP64: while the blocks of three kernels in flight find an SM each, and where they go round
+// the SMs twice; in between the early ones share SMs whose neighbours idle.  Double-float
+// blocks leave their SM enough room for a second: only between half a block and one
+// per SM does nothing come of it.  K_hat in us, plain / early:
+//   blocks          4          48         64         128        152-160     192        256        304        320        2048
+//   FP64         49 / 37    49 / 38    49 / 73    49 / 94    78 / 96    81 / 79    82 / 98    82 / 70   107 / 99   446 / 439
+//   double-float 29 / 18    29 / 22    29 / 22    30 / 31    37 / 32    37 / 34    39 / 34    39 / 35    43 / 35   156 / 143
+inline bool early_gains_f64(int nb, int nsm) { return 3 * nb <= nsm || nb >= 2 * nsm; }
+inline bool early_gains_dd(int nb, int nsm) { return 2 * nb <= nsm || nb > nsm; }
 
 // ----------------------------------------------------------------------------
 // spinor storage formats
