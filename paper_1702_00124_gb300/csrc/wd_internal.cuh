@@ -592,7 +592,8 @@ struct Sum2 {
 };
 __device__ __forceinline__ Sum2 sum2_add(Sum2 a, double s, double c) {
   const double t = a.s + s, z = t - a.s;
-  return {t, a.c + (((a.s - (t - z)) + (s - z)) + c)};
+  const double e = isfinite(t) ? (a.s - (t - z)) + (s - z) : 0.0;   // a sum that overflows stays infinite
+  return {t, a.c + (e + c)};
 }
 template <int NV> __device__ __forceinline__ void grid_sum_hl(const Reduce& r, double (&v)[NV]) {
   __shared__ double sh[NV * 32];
@@ -636,7 +637,7 @@ template <int NV> __device__ __forceinline__ void grid_sum_hl(const Reduce& r, d
   for (int k = 0; k < NV; ++k) {
     const double h = a[k].s + a[k].c;
     r.out[k] = h;
-    r.out[NV + k] = (a[k].s - h) + a[k].c;
+    r.out[NV + k] = isfinite(h) ? (a[k].s - h) + a[k].c : 0.0;
   }
   *r.counter = 0u;
 }
