@@ -85,7 +85,8 @@ __device__ __forceinline__ void outer_acc(cpx<T> (&A)[9], const cpx<T> (&h)[6], 
 // roots goes out in one launch.
 //
 // Block: 32 sites of one parity x 4 directions, one warp a direction, so that
-// a site's own spinors are read once from L2 and three times from L1.
+// a site's own spinors are read once from L2 and three times from L1.  One FP32 pair
+// on all but small lattices: k_force_site below.
 //
 // Measured at 16^3 x 32 (FP32): the kernel before it (one thread per site, two products
 // per pair, F updated for every pair of pairs) 94 us per root, 16 roots 1.51 ms; the
@@ -145,7 +146,7 @@ __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, lon
 // Two FP32 pairs: latency of the spinor reads, so five blocks per SM (96 registers, 14
 // words spilled).  16 roots at 16^3 x 32, whole force: link kept over the groups, 138
 // registers 2.10 ms; link read again per group (L1), 110 registers 2.05 ms; this 2.00 ms.
-// One pair takes 108 registers; FP64 is bound by its arithmetic.
+// One FP32 pair, on small lattices, takes 154 registers; FP64 is bound by its arithmetic.
 template <class T, int NP> constexpr int force_blocks() { return sizeof(T) == 4 && NP == 2 ? 5 : 1; }
 template <class T, int NP, class S, class G>
 __global__ void __launch_bounds__(F_THREADS, force_blocks<T, NP>()) k_force(ForceArgs<S, G> a) {
@@ -162,6 +163,58 @@ __global__ void __launch_bounds__(F_THREADS, force_blocks<T, NP>()) k_force(Forc
     case 2: force_dir<2, NP, T>(a, par, cb, c, ok); break;
     default: force_dir<3, NP, T>(a, par, cb, c, ok); break;
   }
+}
+
+// One FP32 pair: one thread per site, the directions in turn.  Its own X and Y stay in
+// registers (the warps per direction above read them four times) and 128 sites share
+// their neighbours through L1; four blocks per SM (128 registers).  Derivative, sums and
+// results are bit for bit those of k_force.  Latency of the spinor reads bounds it on small
+// lattices, HBM on large ones: links, X, Y and F move 2.1 GB at 32^3 x 64, 0.31 ms.
+// One call of the force from given X and Y (two conversions, two hops, this), k_force -> this:
+// 12^3 x 24 33 -> 25 us, 16^3 x 32 94 -> 66, 24^4 243 -> 180, 24^3 x 48 467 -> 331, 32^3 x 64
+// 1413 -> 958 (five blocks per SM 1003, no bound 1087).  From one block per SM on (156 blocks
+// 24.0 -> 21.2 us); 8^3 x 16, 64 blocks, 17.1 -> 18.8.
+template <int MU, class S, class G>
+__device__ __forceinline__ void force_site_dir(const ForceArgs<S, G>& a, int par, long cb, const int (&c)[4],
+                                               const cpx<float> (&Xs)[12], const cpx<float> (&Ys)[12]) {
+  const Geom& g = a.g;
+  const long nb = g.template nbr<2 * MU>((unsigned)cb, c);
+  cpx<float> A[9], s[12], h[6], k[6];
+#pragma unroll
+  for (int j = 0; j < 9; ++j) A[j] = mk<float>(0, 0);
+  (par ? a.Xe[0] : a.Xo[0]).loadT(nb, s);
+  half_of<MU, -1>(s, h);
+  half_of<MU, -1>(Ys, k);
+  outer_acc(A, h, k);
+  (par ? a.Ye[0] : a.Yo[0]).loadT(nb, s);
+  half_of<MU, +1>(s, h);
+  half_of<MU, +1>(Xs, k);
+  outer_acc(A, h, k);
+  cpx<float> U[9], W[9];
+  a.gauge.load(MU, par, cb, U);
+  mat_mul(U, A, W);
+  float f[8];
+  proj_ta(W, f);
+  const double coef = (MU == 3 && c[3] == g.L[3] - 1) ? -a.coef : a.coef;
+  double* F = a.F + ((long)(MU * 2 + par) * 8) * g.Vh + cb;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) F[q * g.Vh] = fma(coef, to_f64(f[q]), F[q * g.Vh]);
+}
+template <class S, class G>
+__global__ void __launch_bounds__(F_THREADS, 4) k_force_site(ForceArgs<S, G> a) {
+  const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= 2 * a.g.Vh) return;
+  const int par = (int)(tid / a.g.Vh);
+  const long cb = tid - par * a.g.Vh;
+  int c[4];
+  a.g.coords(cb, par, c);
+  cpx<float> Xs[12], Ys[12];
+  (par ? a.Xo[0] : a.Xe[0]).loadT(cb, Xs);
+  (par ? a.Yo[0] : a.Ye[0]).loadT(cb, Ys);
+  force_site_dir<0>(a, par, cb, c, Xs, Ys);
+  force_site_dir<1>(a, par, cb, c, Xs, Ys);
+  force_site_dir<2>(a, par, cb, c, Xs, Ys);
+  force_site_dir<3>(a, par, cb, c, Xs, Ys);
 }
 
 template <class T, int NP, class S, class G>
@@ -183,8 +236,15 @@ static void force_launch(wd_ctx* c, const G& gauge, double coef, int n, const Fi
       a.Xe[p] = S{(P)Xe[s].data, Vh};
       a.Xo[p] = S{(P)Xo[s].data, Vh};
     }
-    k_force<T, NP><<<dim3(nblocks(Vh, 32), 2), F_THREADS, 0, c->stream>>>(a);
     c->launches += 1;
+    if constexpr (NP == 1 && sizeof(T) == 4) {
+      const int nb = nblocks(2 * Vh, F_THREADS);
+      if (a.n == 1 && nb >= c->nsm) {          // a block for every SM
+        k_force_site<<<nb, F_THREADS, 0, c->stream>>>(a);
+        continue;
+      }
+    }
+    k_force<T, NP><<<dim3(nblocks(Vh, 32), 2), F_THREADS, 0, c->stream>>>(a);
   }
 }
 
