@@ -138,7 +138,11 @@ __device__ __forceinline__ void b_block_partial(const BArgs& a, int vb, float (&
 
 // One direction of the hop for RPT right-hand sides of one site: the link is
 // loaded and rebuilt once and applied to the RPT neighbour spinors (consecutive
-// in the interleaved layout).
+// in the interleaved layout).  Products in two chains: with 18-real links a chain of six
+// left the compiler 90 registers' worth of loads in flight and the default shape (128 items, one
+// right-hand side per thread) 7 to 10 % behind separately rounded products.  wd_batch_mdagm,
+// separate / one chain / two chains: 18 reals, 4 x 8^3 x 16 x 2 sides 99.5 / 107.7 / 99.4 us,
+// 3 x 12^3 x 24 x 2 150 / 164 / 142, 6 x 16^3 x 32 x 4 1338 / 1366 / 1138; 12 reals, the last 1123 / 1051 / 976.
 template <int MU, bool DAG, int RPT, bool COH, class G>
 __device__ __forceinline__ void bhop_dir(const Geom& g, int par, long cb, const int (&c)[4], const float4* in,
                                          long stride, int nr, int r0, const G& gauge, cpx<float> (&acc)[RPT][12]) {
@@ -162,11 +166,11 @@ __device__ __forceinline__ void bhop_dir(const Geom& g, int par, long cb, const 
         for (int j = 0; j < 6; ++j) h[j] = mk<float>(-h[j].r, -h[j].i);
       }
       if (fwd) {
-        su3_mul(U, h, u);
+        su3_mul_2c(U, h, u);
         if constexpr (MU == 0) spin_accum<MU, SF, true>(acc[k], u);   // the first direction writes acc
         else spin_accum<MU, SF>(acc[k], u);
       } else {
-        su3_dag_mul(U, h, u);
+        su3_dag_mul_2c(U, h, u);
         spin_accum<MU, -SF>(acc[k], u);
       }
     }
