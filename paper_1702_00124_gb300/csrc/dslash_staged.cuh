@@ -16,17 +16,24 @@
 // How deep (hop_depth): a lattice of many waves of blocks is bound by HBM and wants
 // resident blocks; one that fits the SMs at once is bound by the chain of
 // eight neighbour reads, and registers that no second block would use hold more of them
-// in flight.  Per FP32 K_hat in a chain on 152 SMs, depth (NST, SA, blocks per SM):
-//                 blocks  (2,1,5)  (4,2,4)  (6,3,3)  (7,5,2)
-//   12^3 x 24        162    27.2     22.9     19.9     17.1 us
-//   16^4             256    26.6     22.9     19.7     17.3
-//   16^3 x 32        512    28.9     24.3     26.8     26.4
-//   16^2 x 32^2     1024    47.1     42.9     46.9     49.2
-//   24^4            1296    66.5     75.1     70.2     75.8
-//   32^3 x 64       8192     405      408      407      441
-// so: two blocks per SM if all fit, three if all fit, four while that takes no
-// more waves than the full occupancy.  16-bit spinors, (2,1,6) (4,3,4) (6,4,3): 12^3 x 24
-// 32.8, 25.5, 21.3; 16^3 x 32 38.8, 27.4, 30.2; 32^3 x 64 356, 388, 398.
+// in flight.  K_hat in a chain on 152 SMs, its conversion from FP64 included, us, by depth
+// (NST, SA, blocks per SM), FP32 spinors:
+//                       12 reals                           18 reals
+//                 blocks (2,1,5) (4,2,4) (6,3,3) (6,5,2)   (2,1,5) (4,2,4) (4,3,3) (5,5,2)
+//   12^3 x 24        162   32.5    27.5    25.7    21.5      42.4    32.3    28.5    21.3
+//   16^4             256   32.7    27.0    26.2    22.6      41.7    30.7    28.7    21.9
+//   16^3 x 24        384   34.0    30.2    26.0    29.2      44.3    34.6    29.0    33.5
+//   16^3 x 32        512   36.1    31.9    35.4    34.7      47.5    37.7    42.0    37.8
+//   18x22x20x26      805   55.9    53.2    52.6    53.5      85.5    77.4    72.2    73.2
+//   20x22x24x26     1073   69.9    67.1    72.6    76.2     107.4   100.3   100.8   105.4
+//   24^4            1296   83.5    92.7    90.1    98.1     118.4   124.4   115.0   123.2
+//   24^3 x 48       2592    171     176     178     193       229     225     215     225
+//   32^3 x 64       8192    485     485     497     555       644     639     611     660
+// so: two blocks per SM if all fit, three if all fit; with 12 reals four while that takes
+// no more waves than the full occupancy; with 18 reals (9 KB a buffer) four if all fit, else three.
+// 16-bit spinors, (2,1,6) (4,3,4) (6,4,3) on 12 reals: 12^3 x 24 34.2, 32.7, 29.2; 16^3 x 32
+// 43.2, 35.6, 37.6; 24^4 80.3, 83.3, 83.7; 32^3 x 64 445, 464, 481; (2,1,5) (4,3,4) on 18 reals:
+// 12^3 x 24 37.2, 36.4; 16^3 x 32 43.7, 37.3; 24^4 107, 115; 32^3 x 64 569, 577.
 #pragma once
 #include <atomic>
 
@@ -266,11 +273,12 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, MINB) k_hop_st(HopArgs<In, Out
 }
 
 // Resident blocks per SM that the pipeline's depth is chosen for (table at the top):
-// 2, 3, 4 or the full occupancy
+// 2, 3, 4 or the full occupancy; full = 0: not beyond one wave of four, else three
 inline int hop_depth(const wd_ctx* c, int full) {
   const int nb = nblocks(c->g.Vh, HOP_ST_THREADS), n = c->nsm > 0 ? c->nsm : 1;
   if (nb <= 2 * n) return 2;
   if (nb <= 3 * n) return 3;
+  if (full == 0) return nb <= 4 * n ? 4 : 3;
   return (nb + 4 * n - 1) / (4 * n) <= (nb + full * n - 1) / (full * n) ? 4 : full;
 }
 
@@ -291,13 +299,12 @@ void hop_st_go(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {
 template <bool DAG, int EPI, bool NORM, class In, class Out, class Y, class G>
 void hop_st_depth(wd_ctx* c, const HopArgs<In, Out, Y, G>& a, const HopPoly& pe) {
   if constexpr (std::is_same<G, GF32>::value) {
-    // 18 reals: 9 KB a buffer, 55 KB a block at NST = 5
+    // 55 KB a block at NST = 5
     if constexpr (std::is_same<In, SpF32>::value) {
-      switch (hop_depth(c, 5)) {
+      switch (hop_depth(c, 0)) {
         case 2: hop_st_go<DAG, EPI, NORM, 5, 5, 2>(c, a, pe); break;
-        case 3: hop_st_go<DAG, EPI, NORM, 4, 3, 3>(c, a, pe); break;
         case 4: hop_st_go<DAG, EPI, NORM, 4, 2, 4>(c, a, pe); break;
-        default: hop_st_go<DAG, EPI, NORM, 2, 1, 5>(c, a, pe);
+        default: hop_st_go<DAG, EPI, NORM, 4, 3, 3>(c, a, pe);
       }
     } else {
       if (hop_depth(c, 5) <= 4) hop_st_go<DAG, EPI, NORM, 4, 3, 4>(c, a, pe);
