@@ -16,14 +16,19 @@ namespace wd {
 // 1.97 -> 0.44 ms (2.4 GB, 0.36 ms at the copy peak).
 // The lexicographic side needs 8-byte alignment only; VEC: elements of the EO side
 // move as 16-byte words.
+// The shapes are compile-time constants: with run-time divisors the index arithmetic of
+// algebra fields, whose elements are one double, cost more than the old strides at
+// some sizes.  Algebra pack / unpack in us, one site per thread, run-time shapes, constants: 16^3 x 32
+// 23.1 / 23.1, 24.9 / 25.7, 13.2 / 14.8; 18 x 22 x 20 x 26 34.7 / 36.5, 37.2 / 39.6, 23.2 / 25.1;
+// 24^3 x 48 138 / 240, 107 / 112, 66 / 70.  Links 16^3 x 32 with the FP32 copies 62.0, 59.7, 51.9.
 constexpr int PACK_S = 64, PACK_THREADS = 256;
+constexpr int pack_pitch(int d, int c) { return d + (c == 2 ? 2 : 1 - (d & 1)); }   // doubles of a site in shared memory
 
-template <int C, bool VEC, bool UNPACK>
-__global__ void __launch_bounds__(PACK_THREADS) k_pack(Geom g, int nchunk, int W, int parity, const double* src,
-                                                       double* dst) {
+template <int C, int NOUTER, int NCHUNK, bool VEC, bool UNPACK>
+__global__ void __launch_bounds__(PACK_THREADS) k_pack(Geom g, int parity, const double* src, double* dst) {
   extern __shared__ double2 pack_sh[];
   double* sh = reinterpret_cast<double*>(pack_sh);   // [PACK_S][P]
-  const int D = W * C, P = D + (C == 2 ? 2 : 1 - (D & 1));
+  constexpr int W = NOUTER * NCHUNK, D = W * C, P = pack_pitch(D, C);
   const long lex0 = (long)blockIdx.x * PACK_S;
   const int n = (int)(g.V - lex0 < PACK_S ? g.V - lex0 : PACK_S), half = n / 2;   // V is even
   const int npar = parity >= 0 ? 1 : 2;
@@ -42,11 +47,11 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack(Geom g, int nchunk, int W
     __syncthreads();
   }
   for (int e = threadIdx.x; e < npar * W * half; e += PACK_THREADS) {
-    const int q = e / half, k = e - q * half;
+    const int q = half == PACK_S / 2 ? e / (PACK_S / 2) : e / half, k = e - q * half;
     const int p = q / W, w = q - p * W;
     const int par = parity >= 0 ? parity : p;
-    const int o = w / nchunk, j = w - o * nchunk;
-    const long base = parity >= 0 ? w : (long)(o * 2 + par) * nchunk + j;
+    const int o = w / NCHUNK, j = w - o * NCHUNK;
+    const long base = parity >= 0 ? w : (long)(o * 2 + par) * NCHUNK + j;
     const long eo = (base * g.Vh + (lex0 >> 1) + k) * C;
     double* at = sh + site_of(k, par) * P + w * C;
     if constexpr (VEC) {
@@ -76,21 +81,28 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack(Geom g, int nchunk, int W
   }
 }
 
-template <int C, bool VEC>
-static void pack_launch(wd_ctx* c, bool unpack, int nouter, int nchunk, int parity, const double* src, double* dst) {
-  const int W = nouter * nchunk, D = W * C;
-  const size_t sm = sizeof(double) * PACK_S * (D + (C == 2 ? 2 : 1 - (D & 1)));   // links: 37.9 KB
+template <int C, int NOUTER, int NCHUNK, bool VEC>
+static void pack_launch(wd_ctx* c, bool unpack, int parity, const double* src, double* dst) {
+  constexpr size_t sm = sizeof(double) * PACK_S * pack_pitch(NOUTER * NCHUNK * C, C);   // links: 37.9 KB
   const int nb = (int)((c->g.V + PACK_S - 1) / PACK_S);
-  if (unpack) k_pack<C, VEC, true><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, nchunk, W, parity, src, dst);
-  else k_pack<C, VEC, false><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, nchunk, W, parity, src, dst);
+  if (unpack) k_pack<C, NOUTER, NCHUNK, VEC, true><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, parity, src, dst);
+  else k_pack<C, NOUTER, NCHUNK, VEC, false><<<nb, PACK_THREADS, sm, c->stream>>>(c->g, parity, src, dst);
 }
 
 int pack_k(wd_ctx* c, bool unpack, int nouter, int nchunk, int chunk, int parity, const double* src,
            double* dst) {
   const bool aligned = ((uintptr_t)(unpack ? src : dst) & 15) == 0;   // the EO side
-  if (chunk == 2 && aligned) pack_launch<2, true>(c, unpack, nouter, nchunk, parity, src, dst);
-  else if (chunk == 2) pack_launch<2, false>(c, unpack, nouter, nchunk, parity, src, dst);
-  else pack_launch<1, false>(c, unpack, nouter, nchunk, parity, src, dst);
+  if (nouter == 4 && nchunk == 9 && chunk == 2) {            // links
+    if (aligned) pack_launch<2, 4, 9, true>(c, unpack, parity, src, dst);
+    else pack_launch<2, 4, 9, false>(c, unpack, parity, src, dst);
+  } else if (nouter == 1 && nchunk == 12 && chunk == 2) {    // spinors
+    if (aligned) pack_launch<2, 1, 12, true>(c, unpack, parity, src, dst);
+    else pack_launch<2, 1, 12, false>(c, unpack, parity, src, dst);
+  } else if (nouter == 4 && nchunk == 8 && chunk == 1) {     // algebra fields
+    pack_launch<1, 4, 8, false>(c, unpack, parity, src, dst);
+  } else {
+    return fail(WD_ERR_ARG, "pack: unknown field shape");
+  }
   WD_CHECK_LAUNCH();
   return WD_OK;
 }
