@@ -15,8 +15,9 @@
 // Bound by the FP64 pipe: 472 bytes a link would take 0.58 ms at 32^3 x 64, about 400
 // FP64 instructions a link (33 ns each on 608 schedulers, 32 links) 5.3 ms.
 // Measured 7.55 ms with whole matrices, divisions and square roots; 5.62 ms with two
-// rows and Newton steps from FP32 seeds; 5.35 ms with the FP32 copies rounded by
-// integer operations.
+// rows and Newton steps from FP32 seeds; 5.36 ms with the FP32 copies rounded by
+// integer operations; 5.44 ms with the square root and the quotient of the
+// exponential corrected by their residuals.
 //
 // Random numbers: Philox4x64-10 (Salmon, Moraes, Dror, Shaw, SC'11) with key
 // (seed, 0) and counter (j, stream, 0, 0); the four words of block j give
@@ -54,16 +55,17 @@ __device__ __forceinline__ double sinc_series(double y) {
 }
 
 // 1/sqrt(x) and 1/x for x > 0 within FP32's range: an FP32 seed (relative error
-// about 1e-7) and two Newton steps, each squaring the error.  GB300 runs FP64 at
-// 1/64 of the FP32 rate; the division and square root of the language cost several
-// times as many FP64 instructions.
+// about 1e-7) and two Newton steps, each squaring the error.  The last step adds a
+// correction to the iterate, so that the result carries its own rounding and little of the step's.
+// GB300 runs FP64 at 1/64 of the FP32 rate; the division and square root of the
+// language cost several times as many FP64 instructions.
 __device__ __forceinline__ bool beyond_seed(double x) { return __double2hiint(x) >= 0x46000000; }   // x > 1e29, inf, NaN
 __device__ __forceinline__ double rsqrt_newton(double x) {
   if (beyond_seed(x)) return 1.0 / sqrt(x);
   double y = (double)rsqrtf((float)x);
   const double hx = 0.5 * x;
 #pragma unroll
-  for (int it = 0; it < 2; ++it) y = y * fma(-hx, y * y, 1.5);
+  for (int it = 0; it < 2; ++it) y = fma(y, fma(-hx * y, y, 0.5), y);
   return y;
 }
 __device__ __forceinline__ double rcp_newton(double x) {
@@ -99,8 +101,14 @@ __device__ __forceinline__ void cayley_hamilton_rows(double q00, double q11, dou
     const bool neg = c0 < 0;
     const double t3 = c1 * (1.0 / 3.0);
     const double y = rsqrt_newton(t3);             // 1 / sqrt(c1 / 3)
-    const double st3 = t3 * y;
-    double r = 0.5 * fabs(c0) * (y * y * y);       // |c0| / (2 (c1/3)^{3/2})
+    double st3 = t3 * y;                           // sqrt(c1 / 3), corrected by its residual
+    st3 = fma(fma(-st3, st3, t3), 0.5 * y, st3);
+    // r = |c0| / (2 (c1/3)^{3/2}), the quotient corrected the same way.  Links after a step of
+    // eps against 128-bit arithmetic, rms, with square root and divisions / uncorrected / this:
+    // eps 0.1 9.3e-17 / 7.3e-17 / 7.3e-17, 2 2.38e-16 / 2.89e-16 / 2.31e-16, 3 3.44e-16 / 4.20e-16 / 3.44e-16
+    const double y3 = y * y * y, q0 = 0.5 * fabs(c0);
+    double r = q0 * y3;
+    r = fma(fma(-t3 * st3, r, q0), y3, r);
     r = r > 1.0 ? 1.0 : r;
     // cs = cos(th/3), th = acos(r) in [0, pi/2]: the root of 4 cs^3 - 3 cs = r
     // in [cos(pi/6), 1], where the derivative 12 cs^2 - 3 lies in [6, 9]; an
