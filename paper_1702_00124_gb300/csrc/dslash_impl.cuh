@@ -68,30 +68,23 @@ __device__ __forceinline__ void su3_dag_mul(const cpx<T> (&U)[9], const cpx<T> (
       o[3 * a + c] = cfma_c(U[6 + c], h[3 * a + 2], cfma_c(U[3 + c], h[3 * a + 1], cmul_c(U[c], h[3 * a])));
 }
 
-// The same with every real component as the difference (or sum) of two chains of three
-// products: one operation more than one chain of six and half its length, for a kernel
-// with few warps in flight (batched hop).
+// The same with every real component as the difference or sum of two chains of three
+// products (dot3, dot3_c): one operation more than one chain of six and half its length, for
+// kernels with few warps in flight (batched hop).
 template <class T>
 __device__ __forceinline__ void su3_mul_2c(const cpx<T> (&U)[9], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const cpx<T> u0 = U[3 * c], u1 = U[3 * c + 1], u2 = U[3 * c + 2], v0 = h[3 * a], v1 = h[3 * a + 1], v2 = h[3 * a + 2];
-      o[3 * a + c] = {fma_t(u2.r, v2.r, fma_t(u1.r, v1.r, u0.r * v0.r)) - fma_t(u2.i, v2.i, fma_t(u1.i, v1.i, u0.i * v0.i)),
-                      fma_t(u2.r, v2.i, fma_t(u1.r, v1.i, u0.r * v0.i)) + fma_t(u2.i, v2.r, fma_t(u1.i, v1.r, u0.i * v0.r))};
-    }
+    for (int c = 0; c < 3; ++c)
+      o[3 * a + c] = dot3(U[3 * c], h[3 * a], U[3 * c + 1], h[3 * a + 1], U[3 * c + 2], h[3 * a + 2]);
 }
 template <class T>
 __device__ __forceinline__ void su3_dag_mul_2c(const cpx<T> (&U)[9], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const cpx<T> u0 = U[c], u1 = U[3 + c], u2 = U[6 + c], v0 = h[3 * a], v1 = h[3 * a + 1], v2 = h[3 * a + 2];
-      o[3 * a + c] = {fma_t(u2.r, v2.r, fma_t(u1.r, v1.r, u0.r * v0.r)) + fma_t(u2.i, v2.i, fma_t(u1.i, v1.i, u0.i * v0.i)),
-                      fma_t(u2.r, v2.i, fma_t(u1.r, v1.i, u0.r * v0.i)) - fma_t(u2.i, v2.r, fma_t(u1.i, v1.r, u0.i * v0.r))};
-    }
+    for (int c = 0; c < 3; ++c) o[3 * a + c] = dot3_c(U[c], h[3 * a], U[3 + c], h[3 * a + 1], U[6 + c], h[3 * a + 2]);
 }
 
 // The same from rows 0 and 1 of U alone (12-real links): an entry of row 2 is

@@ -35,12 +35,19 @@ __device__ __forceinline__ void proj_ta(const cpx<T> (&W)[9], T (&f)[8]) {
   f[7] = -h * (W[0].i + W[4].i - (T)2 * W[8].i) * (T)0.57735026918962576451;
 }
 
+// 3 x 3 products.  FP32: two chains of three per component, which keep the rounding of the
+// separately rounded products before them (against FP64, 16^3 x 32: gauge force 7.17e-8, one
+// chain of six 7.47e-8, two of three 7.19e-8; Hasenbusch force 1.026e-6, 1.088e-6, 1.035e-6).  FP64: one chain
+// of six, the fewest operations on the pipe that bounds it.
 template <class T>
 __device__ __forceinline__ void mat_mul(const cpx<T> (&A)[9], const cpx<T> (&B)[9], cpx<T> (&C)[9]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) C[3 * i + j] = cfma(A[3 * i + 2], B[6 + j], cfma(A[3 * i + 1], B[3 + j], cmul(A[3 * i], B[j])));
+    for (int j = 0; j < 3; ++j) {
+      if constexpr (sizeof(T) == 4) C[3 * i + j] = dot3(A[3 * i], B[j], A[3 * i + 1], B[3 + j], A[3 * i + 2], B[6 + j]);
+      else C[3 * i + j] = cfma(A[3 * i + 2], B[6 + j], cfma(A[3 * i + 1], B[3 + j], cmul(A[3 * i], B[j])));
+    }
 }
 // C = A B^dag
 template <class T>
@@ -48,8 +55,11 @@ __device__ __forceinline__ void mat_mul_nd(const cpx<T> (&A)[9], const cpx<T> (&
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      C[3 * i + j] = cfma_c(B[3 * j + 2], A[3 * i + 2], cfma_c(B[3 * j + 1], A[3 * i + 1], cmul_c(B[3 * j], A[3 * i])));
+    for (int j = 0; j < 3; ++j) {
+      if constexpr (sizeof(T) == 4)
+        C[3 * i + j] = dot3_c(B[3 * j], A[3 * i], B[3 * j + 1], A[3 * i + 1], B[3 * j + 2], A[3 * i + 2]);
+      else C[3 * i + j] = cfma_c(B[3 * j + 2], A[3 * i + 2], cfma_c(B[3 * j + 1], A[3 * i + 1], cmul_c(B[3 * j], A[3 * i])));
+    }
 }
 // C = A^dag B
 template <class T>
@@ -57,7 +67,10 @@ __device__ __forceinline__ void mat_mul_dn(const cpx<T> (&A)[9], const cpx<T> (&
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) C[3 * i + j] = cfma_c(A[6 + i], B[6 + j], cfma_c(A[3 + i], B[3 + j], cmul_c(A[i], B[j])));
+    for (int j = 0; j < 3; ++j) {
+      if constexpr (sizeof(T) == 4) C[3 * i + j] = dot3_c(A[i], B[j], A[3 + i], B[3 + j], A[6 + i], B[6 + j]);
+      else C[3 * i + j] = cfma_c(A[6 + i], B[6 + j], cfma_c(A[3 + i], B[3 + j], cmul_c(A[i], B[j])));
+    }
 }
 
 // h_a(X) for the projector (1 + SG g_mu): 2 x 3 complex
@@ -73,6 +86,15 @@ __device__ __forceinline__ void outer_acc(cpx<T> (&A)[9], const cpx<T> (&h)[6], 
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) A[3 * i + j] = cfma_c(k[3 + j], h[3 + i], cfma_c(k[j], h[i], A[3 * i + j]));
+}
+
+// A += sum_a h_a k_a^dag with the sum formed by itself, so that A1 and A2^dag round apart
+template <class T>
+__device__ __forceinline__ void outer_apart(cpx<T> (&A)[9], const cpx<T> (&h)[6], const cpx<T> (&k)[6]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) A[3 * i + j] = A[3 * i + j] + cfma_c(k[3 + j], h[3 + i], cmul_c(k[j], h[i]));
 }
 
 // F += coef sum_i dRe(Y_i^dag D X_i) over n groups of NP (Y, X) pairs.
@@ -124,7 +146,8 @@ __device__ __forceinline__ void force_dir(const ForceArgs<S, G>& a, int par, lon
       half_of<MU, +1>(s, h);
       (par ? a.Xo[p] : a.Xe[p]).loadT(cb, s);
       half_of<MU, +1>(s, k);
-      outer_acc(A, h, k);
+      if constexpr (NP == 1 && sizeof(T) == 4) outer_apart(A, h, k);
+      else outer_acc(A, h, k);
     }
     cpx<T> U[9], W[9];
     a.gauge.load(MU, par, cb, U);
@@ -189,7 +212,7 @@ __device__ __forceinline__ void force_site_dir(const ForceArgs<S, G>& a, int par
   (par ? a.Ye[0] : a.Yo[0]).loadT(nb, s);
   half_of<MU, +1>(s, h);
   half_of<MU, +1>(Xs, k);
-  outer_acc(A, h, k);
+  outer_apart(A, h, k);
   cpx<float> U[9], W[9];
   a.gauge.load(MU, par, cb, U);
   mat_mul(U, A, W);
@@ -295,11 +318,12 @@ __device__ __forceinline__ void step(const Geom& g, int (&c)[4], int mu, int d) 
   c[mu] = v < 0 ? v + g.L[mu] : (v >= g.L[mu] ? v - g.L[mu] : v);
 }
 
-// One thread per site, every direction in turn.  Measured at 32^3 x 64 (FP32): 1.60 ms,
-// 1.26 ms with the products as FMA chains.  One warp per direction with the planes
-// unrolled took 1.39 ms (links of 18 reals: three at a time fill the registers).
+// One thread per site, every direction in turn, FP32 at four blocks per SM (128 registers).
+// Measured at 32^3 x 64 (FP32): 1.58 ms, 1.26 ms with the products as chains of six, 1.33 ms with two
+// chains of three (1.55 ms without the register bound: 136, three blocks).  One warp per direction
+// with the planes unrolled took 1.39 ms (links of 18 reals: three at a time fill the registers).
 template <class T, class G>
-__global__ void __launch_bounds__(F_THREADS) k_gauge_force(Geom g, G gauge, double coef, double* F) {
+__global__ void __launch_bounds__(F_THREADS, sizeof(T) == 4 ? 4 : 1) k_gauge_force(Geom g, G gauge, double coef, double* F) {
   const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= 2 * g.Vh) return;
   const int par = (int)(tid / g.Vh);
