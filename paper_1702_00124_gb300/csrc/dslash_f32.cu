@@ -71,7 +71,13 @@ int hop_shift(wd_ctx* c, const Field& in, const Field& y, double alpha, double z
     const Field* fields[] = {&y, &v, &out};
     for (const Field* f : fields)
       if (f->fmt != WD_F32) return fail(WD_ERR_ARG, "hop_shift: formats differ");
-    return hop_poly_links<3>(c, alpha, in, y, out, HopPoly{sp32(v), sp32(v), sp32(v), (float)zr, 0.f, (float)zi});
+    cudaEvent_t e0 = nullptr;
+    prof_begin(c, &e0);
+    WD_TRY(hop_poly_links<3>(c, alpha, in, y, out, HopPoly{sp32(v), sp32(v), sp32(v), (float)zr, 0.f, (float)zi}));
+    // the hop's bytes and v
+    const double v_bytes = 96.0 * (double)c->g.Vh;
+    prof_end(c, e0, hop_bytes(WD_F32, WD_F32, true, c->recon == WD_RECON_12 ? 48 : 72, c->g.Vh) + v_bytes, WD_F32);
+    return WD_OK;
   }
   WsGuard w(c);
   Field k;
