@@ -275,27 +275,7 @@ int zero(wd_ctx* c, const Field& f) {
 }
 
 // ---------------------------------------------------------------------------
-// inner products
-template <class T, class A, class B>
-__global__ void __launch_bounds__(BL_THREADS) k_dot(long n, A a, B b, Reduce red) {
-  pdl_enter();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  double v[2] = {0.0, 0.0};
-  if (i < n) {
-    cpx<T> x[12], y[12];
-    a.template loadT<false>(i, x);
-    b.template loadT<false>(i, y);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) {
-      cpx<T> p = cmulc(x[j], y[j]);
-      v[0] += (double)p.r;
-      v[1] += (double)p.i;
-    }
-  }
-  double tot[2];
-  grid_sum<2>(red, v, tot);
-}
-// FP64 fields, word by word: <a, b>, and |a|^2
+// inner products of FP64 fields, word by word: <a, b>, and |a|^2
 __global__ void __launch_bounds__(BL_THREADS) k_dot64(long n, const double2* a, const double2* b, Reduce red) {
   pdl_enter();
   double v[2] = {0.0, 0.0};
@@ -327,22 +307,11 @@ static int check_sum(wd_ctx* c) {
 }
 
 int dot(wd_ctx* c, const Field& a, const Field& b, double* re, double* im) {
-  const long n = c->g.Vh;
+  if (a.fmt != WD_F64 || b.fmt != WD_F64) return fail(WD_ERR_ARG, "dot: FP64 fields");
   WD_TRY(check_sum(c));
-  if (a.fmt == WD_F64 && b.fmt == WD_F64) {
-    pdl_launch(c, k_dot64, sum_blocks(12 * n), BL_THREADS, 0, 12 * n, (const double2*)a.data, (const double2*)b.data,
-               reducer_host(c));
-    WD_CHECK_LAUNCH();
-  } else {
-    WD_TRY(with_fmt(a, [&](auto A) {
-      return with_fmt(b, [&](auto B) {
-        using T = typename Pick<decltype(A), decltype(B)>::T;
-        pdl_launch(c, k_dot<T, decltype(A), decltype(B)>, nblocks(n, BL_THREADS), BL_THREADS, 0, n, A, B, reducer_host(c));
-        WD_CHECK_LAUNCH();
-        return (int)WD_OK;
-      });
-    }));
-  }
+  const long n = 12 * c->g.Vh;
+  pdl_launch(c, k_dot64, sum_blocks(n), BL_THREADS, 0, n, (const double2*)a.data, (const double2*)b.data, reducer_host(c));
+  WD_CHECK_LAUNCH();
   double v[2];
   WD_TRY(fetch_host(c, 2, v));
   if (re) *re = v[0];
@@ -396,7 +365,7 @@ int norm2_any(wd_ctx* c, const Field& b, const Field& x, double* bb, bool* nonze
 }
 
 int norm2(wd_ctx* c, const Field& a, double* out) {
-  if (a.fmt != WD_F64) return dot(c, a, a, out, nullptr);
+  if (a.fmt != WD_F64) return fail(WD_ERR_ARG, "norm2: FP64 fields");
   WD_TRY(check_sum(c));
   const long n = 12 * c->g.Vh;
   pdl_launch(c, k_norm64, sum_blocks(n), BL_THREADS, 0, n, (const double2*)a.data, reducer_host(c));
