@@ -69,8 +69,9 @@ __device__ __forceinline__ void su3_dag_mul(const cpx<T> (&U)[9], const cpx<T> (
 }
 
 // The same with every real component as the difference or sum of two chains of three
-// products (dot3, dot3_c): one operation more than one chain of six and half its length, for
-// kernels with few warps in flight (batched hop).
+// products (dot3, dot3_c): one operation more than one chain of six, half its length and
+// less rounding.  For the batched hop, which has few warps in flight, and for FP32
+// spinors on the staged pipeline at four blocks per SM and more (18 reals: three).
 template <class T>
 __device__ __forceinline__ void su3_mul_2c(const cpx<T> (&U)[9], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
 #pragma unroll
@@ -115,6 +116,26 @@ __device__ __forceinline__ void su3_dag_mul_r12(const cpx<T> (&U)[6], const cpx<
 #pragma unroll
     for (int a = 0; a < 2; ++a)
       o[3 * a + c] = cfma_c(r, h[3 * a + 2], cfma_c(U[3 + c], h[3 * a + 1], cmul_c(U[c], h[3 * a])));
+  }
+}
+template <class T>
+__device__ __forceinline__ void su3_mul_r12_2c(const cpx<T> (&U)[6], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+      o[3 * a + c] = dot3(U[3 * c], h[3 * a], U[3 * c + 1], h[3 * a + 1], U[3 * c + 2], h[3 * a + 2]);
+  const cpx<T> r0 = row2_of(U, 0), r1 = row2_of(U, 1), r2 = row2_of(U, 2);
+#pragma unroll
+  for (int a = 0; a < 2; ++a) o[3 * a + 2] = dot3(r0, h[3 * a], r1, h[3 * a + 1], r2, h[3 * a + 2]);
+}
+template <class T>
+__device__ __forceinline__ void su3_dag_mul_r12_2c(const cpx<T> (&U)[6], const cpx<T> (&h)[6], cpx<T> (&o)[6]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cpx<T> r = row2_of(U, c);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) o[3 * a + c] = dot3_c(U[c], h[3 * a], U[3 + c], h[3 * a + 1], r, h[3 * a + 2]);
   }
 }
 

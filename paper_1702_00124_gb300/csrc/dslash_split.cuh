@@ -3,9 +3,7 @@
 //
 // A block works on 32 sites: warp w forms u = U h (or U^dag h) of direction w for
 // all of them, the eight u's meet in shared memory, and the block's warps share
-// the 12 components of the sum, the epilogue and the store.  The sum runs
-// over the directions in the order of the one-thread-per-site kernels, so the results
-// are bit for bit theirs.
+// the 12 components of the sum, the epilogue and the store.
 //
 // FP64, up to SPLIT_MAX_VH_F64 sites per parity: GB300 has half an FP64 lane per
 // scheduler and clock, so a warp instruction holds its scheduler's pipe for 33 ns
@@ -69,15 +67,16 @@ __device__ __forceinline__ cpx<T> split_term(const cpx<T>* u) {
     return ipow<q>(u[(D * 6 + k) * SPL_SITES]);
   }
 }
+// a direction's two neighbours first: partial sums of two, four, six and eight terms round
+// less than those of two to eight (K_hat FP32 against FP64 at 8^3 x 16: 5.59e-8 -> 5.41e-8)
+template <int J, int MU, bool DAG, class T> __device__ __forceinline__ cpx<T> split_pair(const cpx<T>* u) {
+  return split_term<J, 2 * MU, DAG>(u) + split_term<J, 2 * MU + 1, DAG>(u);
+}
 template <int J, bool DAG, class T> __device__ __forceinline__ cpx<T> split_sum(const cpx<T>* u) {
-  cpx<T> v = split_term<J, 0, DAG>(u);
-  v = v + split_term<J, 1, DAG>(u);
-  v = v + split_term<J, 2, DAG>(u);
-  v = v + split_term<J, 3, DAG>(u);
-  v = v + split_term<J, 4, DAG>(u);
-  v = v + split_term<J, 5, DAG>(u);
-  v = v + split_term<J, 6, DAG>(u);
-  return v + split_term<J, 7, DAG>(u);
+  cpx<T> v = split_pair<J, 0, DAG>(u);
+  v = v + split_pair<J, 1, DAG>(u);
+  v = v + split_pair<J, 2, DAG>(u);
+  return v + split_pair<J, 3, DAG>(u);
 }
 // the same with J known at run time (uniform in a warp)
 template <bool DAG, class T> __device__ __forceinline__ cpx<T> split_sum_at(int j, const cpx<T>* u) {

@@ -75,11 +75,15 @@ template <> struct LinkBuf<GF32R12> {
       U[2 * j + 1] = {v.z, v.w};
     }
   }
+  template <bool TWO>
   __device__ __forceinline__ static void mul(const cpx<float> (&U)[6], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
-    su3_mul_r12(U, h, o);
+    if constexpr (TWO) su3_mul_r12_2c(U, h, o);
+    else su3_mul_r12(U, h, o);
   }
+  template <bool TWO>
   __device__ __forceinline__ static void dag_mul(const cpx<float> (&U)[6], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
-    su3_dag_mul_r12(U, h, o);
+    if constexpr (TWO) su3_dag_mul_r12_2c(U, h, o);
+    else su3_dag_mul_r12(U, h, o);
   }
 };
 template <> struct LinkBuf<GF32> {
@@ -96,18 +100,28 @@ template <> struct LinkBuf<GF32> {
       U[j] = {v.x, v.y};
     }
   }
+  template <bool TWO>
   __device__ __forceinline__ static void mul(const cpx<float> (&U)[9], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
-    su3_mul(U, h, o);
+    if constexpr (TWO) su3_mul_2c(U, h, o);
+    else su3_mul(U, h, o);
   }
+  template <bool TWO>
   __device__ __forceinline__ static void dag_mul(const cpx<float> (&U)[9], const cpx<float> (&h)[6], cpx<float> (&o)[6]) {
-    su3_dag_mul(U, h, o);
+    if constexpr (TWO) su3_dag_mul_2c(U, h, o);
+    else su3_dag_mul(U, h, o);
   }
 };
 template <class G> constexpr size_t hop_smem(int nst) {
   return (size_t)(nst + 1) * LinkBuf<G>::N * HOP_ST_THREADS * sizeof(typename LinkBuf<G>::W);
 }
 
-template <int NST, int SA, bool DAG, class A>
+// TWO: the products in two chains of three (dot3), for FP32 spinors from four blocks per SM on
+// (18 reals: three), where other warps hide the longer issue: K_hat against FP64 keeps the
+// rounding of separately rounded products (16^3 x 32, 18 / 12 reals: 5.46e-8 / 5.54e-8; one
+// chain of six 5.57e-8 / 5.70e-8; two of three 5.46e-8 / 5.59e-8, 5.58e-8 with row 2 in products apart,
+// which costs 1 % more time) and takes 0.5 to 1 % less time at 24^4 and above, 1 to 2 % more at 16^3 x 32.  With two or three blocks of 12 reals per SM, one wave, two chains
+// cost 3 to 6 % and stay out (2 % more rounding); 16-bit spinors round far more by their format.
+template <int NST, int SA, bool DAG, class A, bool TWO = false>
 struct Staged {
   using G = typename std::remove_cv<decltype(A::gauge)>::type;
   using LB = LinkBuf<G>;
@@ -172,8 +186,8 @@ struct Staged {
 #pragma unroll
       for (int j = 0; j < 6; ++j) h[j] = mk<float>(-h[j].r, -h[j].i);
     }
-    if constexpr (FWD) LB::mul(U, h, u);
-    else LB::dag_mul(U, h, u);
+    if constexpr (FWD) LB::template mul<TWO>(U, h, u);
+    else LB::template dag_mul<TWO>(U, h, u);
     spin_accum<MU, SG, D == 0>(acc, u);        // direction 0 writes acc
   }
 
@@ -222,7 +236,8 @@ __global__ void __launch_bounds__(HOP_ST_THREADS, MINB) k_hop_st(HopArgs<In, Out
   const long site = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool ok = site < a.g.Vh;
   const long cb = ok ? site : 0;               // a thread without a site repeats site 0 and stores nothing
-  Staged<NST, SA, DAG, HopArgs<In, Out, Y, G>> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
+  constexpr bool TWO = std::is_same<In, SpF32>::value && MINB >= (std::is_same<G, GF32>::value ? 3 : 4);
+  Staged<NST, SA, DAG, HopArgs<In, Out, Y, G>, TWO> S{a, cb, {0, 0, 0, 0}, sbuf, (int)threadIdx.x, (int)blockDim.x};
   a.g.coords(cb, a.out_par, S.c);
   S.template prologue<0>();                    // the links do not depend on the kernels before
   pdl_wait();
