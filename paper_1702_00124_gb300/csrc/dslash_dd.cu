@@ -18,8 +18,9 @@
 // stride and sign), the projection one per mu, so the kernel stays inside the
 // instruction cache; all eight directions unrolled in one thread did not (1.24 ms per hop at
 // 32^3 x 64), which had split the hop into two launches with a partial sum in
-// between.  Bound by FP32 issue: about 9,000 FP32 instructions a site, 230 us per hop at
-// 32^3 x 64; 1.6 GB would take 240 us.
+// between.  FP32 issue bounds it (72 % of the slots taken, 54 to 58 % of them by the FMA pipe) with
+// memory 44 % busy: about 9,000 FP32 instructions a site would take 230 us per hop at 32^3 x 64 and its
+// 1.6 GB 240 us, the hop takes about 430 us.
 // K_hat in a chain (conversions included), two launches -> this: 32^3 x 64 2349 -> 1992 us,
 // 24^4 501 -> 338, 16^3 x 32 201 -> 143, 8^3 x 16 113 -> 30, 4^4 115 -> 19; without the
 // links' way through shared memory 2126, 365, 157, 29, 27.  Error against FP64

@@ -16,7 +16,7 @@
 // How deep (hop_depth): a lattice of many waves of blocks is bound by HBM and wants
 // resident blocks; one that fits the SMs at once is bound by the chain of
 // eight neighbour reads, and registers that no second block would use hold more of them
-// in flight.  K_hat in a chain on 152 SMs, its conversion from FP64 included, us, by depth
+// in flight.  K_hat in a chain on 152 SMs, its conversion from FP64 included (products in one chain), us, by depth
 // (NST, SA, blocks per SM), FP32 spinors:
 //                       12 reals                           18 reals
 //                 blocks (2,1,5) (4,2,4) (6,3,3) (6,5,2)   (2,1,5) (4,2,4) (4,3,3) (5,5,2)

@@ -101,7 +101,8 @@ static int poly_force(wd_ctx* c, double kappa, const std::vector<double>& rr, co
   // three inside k_minus), for what the pool takes it keeps: as many roots share a launch as
   // the vectors that are free at the time hold (16 roots: 3, 1, 3, 1, 4, 4).  Whole force of
   // 16 roots at 16^3 x 32 (FP32): one launch for each checkpoint segment, with vectors
-  // of its own (15 more), 1.99 ms; 1, 2, 1, 2, 2, ... roots 2.18 ms; this 2.06 ms.
+  // of its own (15 more), 1.99 ms; 1, 2, 1, 2, 2, ... roots 2.18 ms; this 2.06 ms (2.02 ms with
+  // the outer products' matrix products in two chains).
   // `spare` holds the vectors not in use: cp, the R at the segments' ends; buf, ro, mr, mro,
   // the R of one segment with D_oe R, M_hat R and D^dag_oe M_hat R, formed while K_hat
   // is applied to them in the segment's rebuild; L, lo, ml, mlo, the same of a group of L.
